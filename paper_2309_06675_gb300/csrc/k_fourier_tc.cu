@@ -528,7 +528,9 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   return fn;
 }
 
-bool encode_2d(CUtensorMap* map, const void* gptr, uint64_t inner, uint64_t outer, uint32_t box_inner,
+}  // namespace
+
+bool tc_encode_bf16(CUtensorMap* map, const void* gptr, uint64_t inner, uint64_t outer, uint32_t box_inner,
                uint32_t box_outer) {
   auto enc = get_encode();
   if (!enc) return false;
@@ -541,6 +543,8 @@ bool encode_2d(CUtensorMap* map, const void* gptr, uint64_t inner, uint64_t oute
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
+
+namespace {
 
 int grid_for(int64_t total, int threads) {
   int64_t b = (total + threads - 1) / threads;
@@ -592,8 +596,8 @@ cudaError_t launch_fourier_tc(const void* A, const void* Bt, const int* col_exp,
     return cudaErrorInvalidValue;
   const int vel0 = vel_w > 0 ? vw2 : INT_MAX;
   CUtensorMap mA, mB;
-  if (!encode_2d(&mA, A, (uint64_t)Kp, (uint64_t)NSLICE * Mpad, BK, BM)) return cudaErrorInvalidValue;
-  if (!encode_2d(&mB, Bt, (uint64_t)Kp, (uint64_t)NSLICE * Npad, BK, BN)) return cudaErrorInvalidValue;
+  if (!tc_encode_bf16(&mA, A, (uint64_t)Kp, (uint64_t)NSLICE * Mpad, BK, BM)) return cudaErrorInvalidValue;
+  if (!tc_encode_bf16(&mB, Bt, (uint64_t)Kp, (uint64_t)NSLICE * Npad, BK, BN)) return cudaErrorInvalidValue;
   const size_t sm = fourier_tc_smem();
   const int nt = Npad / BN;
   // first column tile that lies entirely at or after red_n0

@@ -142,6 +142,9 @@ struct Plan {
   int escale = 0;                   // that power: the basis holds 2^escale H(R)
   int ql_cap = 0;                   // QL sweeps per eigenvalue (0 = the kernels' default)
   bool ql_fp64 = false;             // MIXED: FP64 QL and its eigenvalues (kubo_options.ql_fp64)
+  bool tc64 = false;                // FP64: step (1) as seven-slice products on the tensor cores
+  int fourier_n = 0;                // its k-points when the call has no batch buffers (kubo_bloch)
+  int f64_k = 0;                    // k-points per sub-batch of its coefficient slices
   int group_m = 8;                  // tensor-core Fourier sum: M tiles rasterised together
   int symv_parts = 4;               // Householder reduction: column partitions of its symv
   bool model = false;   // needs the prepared Fourier basis
@@ -203,6 +206,18 @@ int auto_chunk(int W, int n_eta, int64_t n_total, size_t extra_per_k = 0) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(c, n_total));
 }
 
+// Step (1) of the FP64 mode on the tensor cores (seven slices) instead of the FP64 pipe.  The
+// FMA kernel takes 6 N_R W^2 operations per k-point at 1.2 TFLOP/s; the tensor-core form adds
+// three launches and the slicing of the basis, and pads to 64 vectors and 32 columns.
+// The sliced basis (42 bytes per complex entry of H(R)) stays within 16 GiB.
+constexpr double kTc64MinFlops = 1e8;
+constexpr size_t kTc64MaxBasis = (size_t)16 << 30;
+constexpr size_t kTc64CoefBytes = (size_t)2 << 30;   // coefficient slices of a sub-batch
+bool use_tc64(int W, int N_R, int64_t n) {
+  const size_t basis = (size_t)2 * tc64_slices() * tc64_pad_n(W) * tc_pad_k(N_R);
+  return W >= 4 && N_R >= 16 && 6.0 * N_R * W * W * (double)n >= kTc64MinFlops && basis <= kTc64MaxBasis;
+}
+
 void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
   (void)n_list_outputs_unused;
   Bump b;
@@ -233,6 +248,17 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
       p.o_Hp = b.take(sizeof(double) * (size_t)p.chunk * WW);
       p.o_Xp = b.take(sizeof(double) * (size_t)p.chunk * WW);
       p.o_Yp = b.take(sizeof(double) * (size_t)p.chunk * WW);
+      const int nf = std::max(p.chunk, p.fourier_n);
+      p.tc64 = p.precision == KUBO_FP64 && !p.sep && use_tc64(p.W, p.N_R, nf);
+      if (p.tc64) {
+        p.Npad = tc64_pad_n(p.W);
+        p.Kp = tc_pad_k(p.N_R);
+        const size_t per_k = (size_t)2 * tc64_slices() * p.Kp;
+        p.f64_k = (int)std::max<size_t>(128, std::min<size_t>((size_t)nf, kTc64CoefBytes / per_k / 128 * 128));
+        p.o_Bt = b.take((size_t)2 * tc64_slices() * p.Npad * p.Kp);
+        p.o_cexp = b.take(sizeof(int) * (size_t)p.Npad);
+        p.o_A = b.take(per_k * (size_t)tc_pad_m(p.f64_k));
+      }
     }
   }
   if (p.eigh) {
@@ -504,6 +530,10 @@ kubo_status prepare_model(Call& c, const double* H_R, const RInfo& ri) {
     StageTimer tm(c, KUBO_STAGE_PREP, 1);
     KCHECK(launch_basis_split(c.at<double>(p.o_Bp), c.at<int>(p.o_Rh), p.N_h, p.W, p.Npad, p.Kp, c.at<int>(p.o_cexp), c.at<char>(p.o_Bt), c.s));
   }
+  if (p.tc64) {
+    StageTimer tm(c, KUBO_STAGE_PREP, 2);
+    KCHECK(launch_basis_split64(c.at<double>(p.o_Bp), c.at<int>(p.o_Rh), p.N_h, p.W, p.Npad, p.Kp, c.at<int>(p.o_cexp), c.at<char>(p.o_Bt), c.s));
+  }
   return read_status(c);
 }
 
@@ -534,6 +564,26 @@ EighBufs make_eigh_bufs(const Call& c) {
   if (c.p.ql_cap > 0) b.ql_cap = c.p.ql_cap;
   b.symv_parts = c.p.symv_parts;
   return b;
+}
+
+// Step (1) in FP64 for the k-points of kl: on the tensor cores (in sub-batches whose coefficient
+// slices fit their buffer) or on the FP64 pipe.
+cudaError_t fourier64(const Call& c, const Model& md, const KList& kl, double* Hp, double* Xp,
+                      double* Yp) {
+  const Plan& p = c.p;
+  if (!p.tc64) return launch_fourier_fp64(md, p.mesh, kl, Hp, Xp, Yp, c.s);
+  const size_t WW = (size_t)p.W * p.W;
+  for (int t0 = 0; t0 < kl.n; t0 += p.f64_k) {
+    const KList sub{kl.idx ? kl.idx + t0 : nullptr, kl.base + t0, std::min(p.f64_k, kl.n - t0)};
+    const int Mb = tc_pad_m(sub.n);
+    cudaError_t e = launch_coef_split64(md, p.mesh, sub, Mb, p.Kp, c.at<char>(p.o_A), c.s);
+    if (e == cudaSuccess)
+      e = launch_fourier_tc64(c.at<char>(p.o_A), c.at<char>(p.o_Bt), c.at<int>(p.o_cexp), Mb, p.Npad,
+                              p.Kp, sub.n, p.W, Hp + t0 * WW, Xp + t0 * WW, Yp + t0 * WW,
+                              c.at<DevStatus>(p.o_status), c.s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Eigenvalues (sorted) and eigenvectors U = Q D Z of n tridiagonalised matrices whose
@@ -672,8 +722,8 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
   DevStatus* st = c.at<DevStatus>(p.o_status);
   double2* U = c.at<double2>(p.o_U);
   if (!fourier_done) {
-    StageTimer tm(c, KUBO_STAGE_FOURIER, 1);
-    KCHECK(launch_fourier_fp64(md, p.mesh, kl, Hp, Xp, Yp, c.s));
+    StageTimer tm(c, KUBO_STAGE_FOURIER, p.tc64 ? 2 : 1);
+    KCHECK(fourier64(c, md, kl, Hp, Xp, Yp));
   }
   {
     StageTimer tm(c, KUBO_STAGE_TRIDIAG, 1);
@@ -933,8 +983,8 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
     KList kl{nullptr, base, (int)std::min<int64_t>(p.chunk, ke - base)};
     const int n = kl.n;
     {
-      StageTimer tm(c, KUBO_STAGE_FOURIER, 1);
-      KCHECK(launch_fourier_fp64(md, p.mesh, kl, Hp, Xp, Yp, c.s));
+      StageTimer tm(c, KUBO_STAGE_FOURIER, p.tc64 ? 2 : 1);
+      KCHECK(fourier64(c, md, kl, Hp, Xp, Yp));
     }
     {
       StageTimer tm(c, KUBO_STAGE_TRIDIAG, 1);
@@ -1109,6 +1159,8 @@ kubo_status run_job(Call& c, const Job& j, const kubo_problem& pr, const kubo_op
   KCHECK(launch_pack_basis((const double2*)pr.H_R, jt.pairs, j.ri.idx0, p.N_h, p.W, c.at<double>(p.o_Bp), c.s, p.escale));
   if (tc_fourier(p.precision))
     KCHECK(launch_basis_split(c.at<double>(p.o_Bp), jt.Rh, p.N_h, p.W, p.Npad, p.Kp, c.at<int>(p.o_cexp), c.at<char>(p.o_Bt), c.s));
+  if (p.tc64)
+    KCHECK(launch_basis_split64(c.at<double>(p.o_Bp), jt.Rh, p.N_h, p.W, p.Npad, p.Kp, c.at<int>(p.o_cexp), c.at<char>(p.o_Bt), c.s));
   const int n_out = p.n_eta * p.n_EF;
   KCHECK(cudaMemsetAsync(c.at<char>(p.o_acc), 0, sizeof(double2) * n_out, c.s));
   Model md = make_model(c);
@@ -1779,6 +1831,7 @@ kubo_status kubo_bloch(const double* H_R, const int32_t* R_vecs, int W, int N_R,
     p.precision = o.precision;
     p.mesh = Mesh{kmesh[0], kmesh[1], kmesh[2], (int64_t)kmesh[0] * kmesh[1] * kmesh[2]};
     p.chunk = tc_fourier(o.precision) ? (int)std::min<int64_t>(n_k, o.chunk_k > 0 ? o.chunk_k : 8192) : 0;
+    p.fourier_n = (int)std::min<int64_t>(n_k, 1 << 19);
     p.model = true;
     plan_layout(p, false, 0);
     c.s = (cudaStream_t)o.stream;
@@ -1808,7 +1861,7 @@ kubo_status kubo_bloch(const double* H_R, const int32_t* R_vecs, int W, int N_R,
       const int64_t step = 1 << 19;   // grid.y = step / 16 <= 65535
       for (int64_t t0 = 0; t0 < n_k && r == KUBO_OK && !tc_fourier(p.precision); t0 += step) {
         KList kl{kidx + t0, 0, (int)std::min<int64_t>(step, n_k - t0)};
-        if (launch_fourier_fp64(md, p.mesh, kl, Hk + t0 * WW, dHx + t0 * WW, dHy + t0 * WW, c.s) != cudaSuccess) {
+        if (fourier64(c, md, kl, Hk + t0 * WW, dHx + t0 * WW, dHy + t0 * WW) != cudaSuccess) {
           cudaGetLastError();
           r = KUBO_ERR_CUDA;
         }

@@ -293,6 +293,18 @@ cudaError_t launch_fourier_tc(const void* A, const void* Bt, const int* col_exp,
                               int Kp, int n_rows, double* out, int ldc, DevStatus* st,
                               cudaStream_t s, int red_n0,
                               int group_m = 8, int vel_w = 0);
+// FP64-grade tensor-core Fourier sum: seven slices per operand (k_fourier_tc64.cu).  Operand
+// bytes: Bt 2 slices Npad Kp, A 2 slices Mpad Kp (Mpad = tc_pad_m(k-points), Kp = tc_pad_k(N_R));
+// packed FP64 H, d_x H, d_y H out ([n_rows][W*W] each).
+int tc64_pad_n(int W);
+int tc64_slices();
+cudaError_t launch_basis_split64(const double* Bp, const int* Rh, int N_h, int W, int Npad, int Kp,
+                                 int* col_exp, void* Bt, cudaStream_t s);
+cudaError_t launch_coef_split64(const Model& md, const Mesh& mesh, const KList& kl, int Mpad,
+                                int Kp, void* A, cudaStream_t s);
+cudaError_t launch_fourier_tc64(const void* A, const void* Bt, const int* col_exp, int Mpad,
+                                int Npad, int Kp, int n_rows, int W, double* Hp, double* Xp,
+                                double* Yp, DevStatus* st, cudaStream_t s);
 // the tensor-core kernel's bounded mbarrier wait on a barrier that never completes
 cudaError_t launch_bounded_wait_check(uint32_t limit, DevStatus* st, cudaStream_t s);
 // rows [n][ld] (H | dxH | dyH packed) -> three packed arrays [n][W*W]

@@ -189,4 +189,8 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 }
 
 }  // namespace tc
+
+// tensor map of a row-major bf16 matrix [outer][inner], 128-byte swizzle (k_fourier_tc.cu)
+bool tc_encode_bf16(CUtensorMap* map, const void* gptr, uint64_t inner, uint64_t outer,
+                    uint32_t box_inner, uint32_t box_outer);
 }  // namespace kubo
