@@ -1,4 +1,5 @@
-// Steps (3)-(4) of List 1/2 ("convert" + "evaluate"), FP64, one CTA per k-point:
+// Steps (3)-(4) of List 1/2 ("convert" + "evaluate") for the FP32-rotation modes, W <= 64, one CTA
+// per k-point (the FP64 form: k_fixed.cu):
 //   v^a = U^dagger (d_a H) U            (a = x, y)
 //   Omega_n = -2 sum_{m != n} Im(v^x_nm conj(v^y_nm)) / ((E_n - E_m)^2 + eta^2)   (Eq. 3)
 // (v^y_mn = conj(v^y_nm) because v^y is Hermitian.)  Both rotations are register-tiled
@@ -20,70 +21,6 @@ constexpr int NT = 256;
 constexpr int MAXE = 8;
 // 16 x 16 threads, each a TM x TM tile of the W x W products: TM = 1, 2, 4 for W up to 16,
 // 32, 64 (the smallest tile that covers W, so no thread multiplies padding)
-
-// acc[i][j] = sum_q op(A)[r_i][q] * B[q][c_j],  r_i = ty + 16 i, c_j = tx + 16 j
-template <int TM, bool ADJ>
-__device__ __forceinline__ void cgemm_tile(const double2* __restrict__ A,
-                                           const double2* __restrict__ B, int W, int LD,
-                                           int ty, int tx, double2 (&acc)[TM][TM]) {
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TM; ++j) acc[i][j] = make_double2(0.0, 0.0);
-  for (int q = 0; q < W; ++q) {
-    double2 a[TM], bb[TM];
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-      int r = ty + 16 * i;
-      double2 v = make_double2(0.0, 0.0);
-      if (r < W) {
-        if (ADJ) { v = A[q * LD + r]; v.y = -v.y; }
-        else v = A[r * LD + q];
-      }
-      a[i] = v;
-    }
-#pragma unroll
-    for (int j = 0; j < TM; ++j) {
-      int c = tx + 16 * j;
-      bb[j] = c < W ? B[q * LD + c] : make_double2(0.0, 0.0);
-    }
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TM; ++j) {
-        acc[i][j].x = fma(a[i].x, bb[j].x, acc[i][j].x);
-        acc[i][j].x = fma(-a[i].y, bb[j].y, acc[i][j].x);
-        acc[i][j].y = fma(a[i].x, bb[j].y, acc[i][j].y);
-        acc[i][j].y = fma(a[i].y, bb[j].x, acc[i][j].y);
-      }
-  }
-}
-
-template <int TM>
-__device__ __forceinline__ void store_tile(double2* C, int W, int LD, int ty, int tx,
-                                           const double2 (&acc)[TM][TM]) {
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TM; ++j) {
-      int r = ty + 16 * i, c = tx + 16 * j;
-      if (r < W && c < W) C[r * LD + c] = acc[i][j];
-    }
-}
-
-template <typename TIn>
-__device__ __forceinline__ void unpack_hermitian(const TIn* __restrict__ P, double2* A, int W,
-                                                 int LD, int t) {
-  const FastDiv dW(W);
-  for (int idx = t; idx < W * W; idx += NT) {
-    const int i = (int)dW.div(idx), j = idx - i * W;
-    double2 a;
-    if (i < j) a = make_double2((double)P[i * W + j], (double)P[j * W + i]);
-    else if (i > j) a = make_double2((double)P[j * W + i], -(double)P[i * W + j]);
-    else a = make_double2((double)P[i * W + i], 0.0);
-    A[i * LD + j] = a;
-  }
-}
 
 // max_j |E_j| of a shared array, by warp 0 on the bit patterns (for non-negative doubles the
 // integer order is the numeric order; NaN patterns count as 0): no FP64 instruction, where a
@@ -252,61 +189,6 @@ __device__ __forceinline__ void curvature_epilogue(const V* sVx, const V (&vy)[T
     for (int q = 0; q < 16; ++q) { sr += p[q]; sc += p[16 + q]; }
     Om[e * eta_stride + k * W + n] = sr + sc;
   }
-}
-
-// X and Y: packed Hermitian rows of leading dimension ld (FP64 rows of the FP64 Fourier
-// kernel, or FP32 rows of the tensor-core one).
-template <typename TIn, int TM>
-__global__ void __launch_bounds__(NT) berry_fp64_kernel(const double* __restrict__ E,
-                                                        const double2* __restrict__ U,
-                                                        const TIn* __restrict__ Xp,
-                                                        const TIn* __restrict__ Yp, int64_t ld,
-                                                        int W,
-                                                        const double* __restrict__ etas,
-                                                        int n_eta, double* __restrict__ Om,
-                                                        int64_t eta_stride, int pad) {
-  extern __shared__ double2 sm[];
-  const int LD = W + pad;   // pad = 1: conflict-free column walks; 0: the padding ablation
-  double2* sU = sm;
-  double2* sA = sU + W * LD;
-  double2* sB = sA + W * LD;
-  double* red = (double*)sA;   // reused (sA and beyond) after the pair terms are formed
-  __shared__ double sE[64];
-  __shared__ double sEta[MAXE];
-  __shared__ double s_emax;
-
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int64_t k = blockIdx.x;
-  const size_t WW = (size_t)W * W;
-
-  const FastDiv dW(W);
-  for (int idx = t; idx < W * W; idx += NT) {
-    const int r = (int)dW.div(idx);
-    sU[r * LD + idx - r * W] = U[k * WW + idx];
-  }
-  unpack_hermitian(Xp + k * ld, sA, W, LD, t);
-  for (int j = t; j < W; j += NT) sE[j] = E[k * W + j];
-  if (t < n_eta) sEta[t] = etas[t];
-  __syncthreads();
-  emax_warp0(sE, W, t, &s_emax);
-
-  double2 acc[TM][TM];
-  cgemm_tile<TM, false>(sA, sU, W, LD, ty, tx, acc);        // T = X U
-  __syncthreads();
-  store_tile<TM>(sA, W, LD, ty, tx, acc);
-  __syncthreads();
-  cgemm_tile<TM, true>(sU, sA, W, LD, ty, tx, acc);         // v^x = U^H T
-  __syncthreads();
-  store_tile<TM>(sA, W, LD, ty, tx, acc);
-  unpack_hermitian(Yp + k * ld, sB, W, LD, t);
-  __syncthreads();
-  cgemm_tile<TM, false>(sB, sU, W, LD, ty, tx, acc);        // T = Y U
-  __syncthreads();
-  store_tile<TM>(sB, W, LD, ty, tx, acc);
-  __syncthreads();
-  cgemm_tile<TM, true>(sU, sB, W, LD, ty, tx, acc);         // v^y = U^H T
-  curvature_epilogue<TM, double2>(sA, acc, sE, sEta, n_eta, s_emax, W, LD, ty, tx, t, red, Om,
-                              eta_stride, k);
 }
 
 // ------------------------------------------------------------------ mixed precision
@@ -1394,44 +1276,6 @@ __global__ void __launch_bounds__(TF_NT, 2) berry_tf32_kernel(
 }
 
 }  // namespace
-
-size_t berry_fp64_smem(int W, int n_eta) {
-  size_t mat = (size_t)W * (W + 1) * sizeof(double2);
-  size_t red = (size_t)n_eta * W * 2 * 16 * sizeof(double);
-  return mat + (2 * mat > red ? 2 * mat : red);
-}
-
-template <typename TIn>
-cudaError_t launch_berry_fp64_t(const double* E, const double2* U, const TIn* Xp, const TIn* Yp,
-                                int64_t ld, int W, int n, const double* etas, int n_eta, double* Om,
-                                int64_t eta_stride, cudaStream_t s, int pad) {
-  if (n <= 0) return cudaSuccess;
-  size_t sm = berry_fp64_smem(W, n_eta);
-  auto go = [&](auto kern) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    kern<<<n, NT, sm, s>>>(E, U, Xp, Yp, ld, W, etas, n_eta, Om, eta_stride, pad ? 1 : 0);
-    return cudaGetLastError();
-  };
-  if (W <= 16) return go(berry_fp64_kernel<TIn, 1>);
-  if (W <= 32) return go(berry_fp64_kernel<TIn, 2>);
-  return go(berry_fp64_kernel<TIn, 4>);
-}
-
-cudaError_t launch_berry_fp64(const double* E, const double2* U, const double* Xp,
-                              const double* Yp, int W, int n, const double* etas, int n_eta,
-                              double* Om, int64_t eta_stride, cudaStream_t s, int pad) {
-  return launch_berry_fp64_t<double>(E, U, Xp, Yp, (int64_t)W * W, W, n, etas, n_eta, Om,
-                                     eta_stride, s, pad);
-}
-
-cudaError_t launch_berry_fp64_rows(const double* E, const double2* U, const double* C,
-                                   int64_t ld, int W, int n, const double* etas, int n_eta,
-                                   double* Om, int64_t eta_stride, cudaStream_t s, int pad) {
-  const int64_t WW = (int64_t)W * W;
-  return launch_berry_fp64_t<double>(E, U, C + WW, C + 2 * WW, ld, W, n, etas, n_eta, Om,
-                                     eta_stride, s, pad);
-}
 
 // bytes of the U assembly's staging area (reflectors, then the block factors G and T)
 static size_t asm_stage_bytes(int W) {

@@ -154,6 +154,8 @@ struct Plan {
   bool lbuf = false;    // W > SMALL_W_MAX: scratch of the multi-pass kernels
   bool grad = false;    // reverse-mode buffers (kubo_ahc_grad)
   bool iit = false;     // inverse-iteration scratch (separate eigenvector kernel)
+  bool lean = false;    // a caller's workspace too small for Z and the iteration scratch (W <= 64)
+  bool user_u = false;  // eigenvectors from the caller (kubo_berry_batched): column norms on the device
   int iit_slots = 0;
   // separable Fourier sum: bounding box, pairs per batch, planes of the range
   bool sep = false;
@@ -164,7 +166,7 @@ struct Plan {
          o_acc = 0, o_Hp = 0, o_Xp = 0, o_Yp = 0, o_E = 0, o_U = 0, o_Om = 0, o_d = 0, o_e = 0,
          o_ph = 0, o_refl = 0, o_tau = 0, o_lam = 0, o_part = 0,
          o_HR = 0, o_EF = 0, o_out = 0, o_Bt = 0, o_A = 0, o_C64 = 0, o_cexp = 0, o_L = 0,
-         o_iit = 0, o_box = 0, o_sepA = 0, o_sepB = 0, o_sepBy = 0;
+         o_iit = 0, o_Z = 0, o_ue = 0, o_box = 0, o_sepA = 0, o_sepB = 0, o_sepBy = 0;
   // reverse mode: six complex W x W work matrices per k, Ebar, packed [Hbar|dxHbar|dyHbar],
   // the Fourier coefficient rows of the batch and the accumulated G rows
   size_t o_gw = 0, o_Ebar = 0, o_Mbar = 0, o_Coef = 0, o_Gacc = 0;
@@ -288,7 +290,16 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
     p.o_fOm = b.take(sizeof(double) * (size_t)p.fix_cap * p.W * p.n_eta);
   }
   if (p.lbuf) p.o_L = b.take(large_region_bytes(p.W) * (size_t)std::max(1, p.chunk));
-  p.iit = p.eigh && (p.W > SMALL_W_MAX || f32_rotation(p.precision));
+  // eigenvectors Z of T, W <= 64 with FP64 eigenvectors U: in the buffer of H (not read after
+  // the reduction), or in one of their own where H is the caller's or part of the mixed rows
+  if (p.eigh && p.W <= SMALL_W_MAX) {
+    if (p.model && !tc_fourier(p.precision)) p.o_Z = p.o_Hp;
+    else if (!p.lean && (!p.model || p.fixup || !f32_rotation(p.precision)))
+      p.o_Z = b.take(sizeof(double) * WW * (size_t)std::max(1, p.chunk));
+  }
+  // column norms of the caller's U (up to 48 of them in the unused part of the broadenings' block)
+  if (p.user_u) p.o_ue = p.chunk <= 48 ? p.o_etas + sizeof(double) * MAX_ETA : b.take(sizeof(int) * (size_t)p.chunk);
+  p.iit = p.eigh && !p.lean;
   if (p.iit) {
     p.iit_slots = iit_slots_for(p.W, std::max(1, p.chunk));
     p.o_iit = b.take(sizeof(double) * iit_scratch_doubles(p.W, p.iit_slots));
@@ -315,6 +326,22 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
     p.o_out = b.take(sizeof(double) * (size_t)p.n_eta * p.n_EF);
   }
   p.total = b.off;
+}
+
+// Halves the batch until the layout fits a caller's workspace (entry points whose batches are
+// independent matrices).
+void fit_workspace(Plan& p, const kubo_options& o) {
+  const int chunk = p.chunk;
+  while (o.workspace && p.total > o.workspace_bytes && p.chunk > 1) {
+    p.chunk = (p.chunk + 1) / 2;
+    plan_layout(p, false, 0);
+  }
+  if (!o.workspace || p.total <= o.workspace_bytes || p.W > SMALL_W_MAX || p.lean) return;
+  // not even one matrix: the single-launch kernels, whose scratch is in shared memory
+  p.lean = true;
+  p.chunk = chunk;
+  plan_layout(p, false, 0);
+  fit_workspace(p, o);
 }
 
 // ------------------------------------------------------------------ device allocations
@@ -593,7 +620,12 @@ cudaError_t fourier64(const Call& c, const Model& md, const KList& kl, double* H
 cudaError_t eigh_vectors(const Call& c, int n, const EighBufs& eb, double* E, double2* U,
                          bool f32u = false, bool rq = false) {
   const Plan& p = c.p;
-  if (p.W <= SMALL_W_MAX) return launch_backtransform(p.W, n, eb, E, U, c.s, p.pad);
+  if (p.W <= SMALL_W_MAX) {
+    if (p.lean) return launch_backtransform(p.W, n, eb, E, U, c.s, p.pad);
+    double* Z = U ? c.at<double>(p.o_Z) : nullptr;
+    cudaError_t e = launch_iit(p.W, n, eb, E, Z, c.at<double>(p.o_iit), p.iit_slots, c.s);
+    return e != cudaSuccess || !U ? e : launch_reflect_fix(p.W, n, eb, Z, U, c.s, p.pad);
+  }
   double* Z = U ? c.at<double>(p.o_L) : nullptr;
   cudaError_t e = Z && df_eigh(p.precision)
                       ? launch_iit_df(p.W, n, eb, E, Z, c.at<double>(p.o_iit), p.iit_slots, c.s)
@@ -623,13 +655,19 @@ cudaError_t berry_any(const Call& c, const double* E, const double2* U, const do
     return launch_berry_large(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, f32, L, L + cap,
                               L + 2 * cap, c.s);
   }
+  if (!f32) {
+    int* ue = p.user_u ? c.at<int>(p.o_ue) : nullptr;
+    if (ue) {
+      cudaError_t e = launch_unorm(U, p.W, n, ue, c.s);
+      if (e != cudaSuccess) return e;
+    }
+    return launch_berry_fix(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, ue, c.s, p.pad);
+  }
   if (rows) {
     const double* C = X - (size_t)p.W * p.W;   // the row start (H | dxH | dyH)
-    return f32 ? launch_berry_mixed_rows(E, U, C, ld, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad)
-               : launch_berry_fp64_rows(E, U, C, ld, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad);
+    return launch_berry_mixed_rows(E, U, C, ld, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad);
   }
-  return f32 ? launch_berry_mixed_from_f64(E, U, X, Y, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad)
-             : launch_berry_fp64(E, U, X, Y, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad);
+  return launch_berry_mixed_from_f64(E, U, X, Y, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad);
 }
 
 // Steps (1)-(4) for one batch [t0, t0+n) of a k-list; E and U go to the chunk buffers, Omega
@@ -699,7 +737,7 @@ kubo_status run_batch_mixed(Call& c, const Model& md, const KList& kl, double* E
     return KUBO_OK;
   }
   {
-    StageTimer tm(c, KUBO_STAGE_BACKTRANSFORM, p.W > SMALL_W_MAX ? 2 : 1);
+    StageTimer tm(c, KUBO_STAGE_BACKTRANSFORM, 2);
     KCHECK(eigh_vectors(c, kl.n, eb, Eout, U, f32_rotation(p.precision),
                         rq_eigenvalues(p.precision, p.ql_fp64)));
   }
@@ -752,7 +790,7 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
     return KUBO_OK;
   }
   {
-    StageTimer tm(c, KUBO_STAGE_BACKTRANSFORM, p.W > SMALL_W_MAX ? 2 : 1);
+    StageTimer tm(c, KUBO_STAGE_BACKTRANSFORM, 2);
     KCHECK(eigh_vectors(c, kl.n, eb, Eout, U, f32_rotation(p.precision)));
   }
   {
@@ -810,7 +848,7 @@ kubo_status fixup_batch(Call& c, const Model& md, const KList& kl, const double*
   for (int c0 = 0; c0 < cnt; c0 += p.fix_cap) {
     const int nf = std::min(p.fix_cap, cnt - c0);
     KList fl{kid + c0, 0, nf};
-    StageTimer tm(c, KUBO_STAGE_FIXUP, p.W > SMALL_W_MAX ? 11 : 6);
+    StageTimer tm(c, KUBO_STAGE_FIXUP, p.W > SMALL_W_MAX ? 11 : 7);
     KCHECK(launch_fourier_fp64(md, p.mesh, fl, c.at<double>(p.o_fHp), c.at<double>(p.o_fXp), c.at<double>(p.o_fYp), c.s));
     KCHECK(launch_tridiag(c.at<double>(p.o_fHp), p.W, nf, eb, c.s));
     KCHECK(launch_ql(p.W, nf, eb, st, c.s));
@@ -995,7 +1033,7 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
       KCHECK(launch_ql(p.W, n, eb, st, c.s));
     }
     {
-      StageTimer tm(c, KUBO_STAGE_BACKTRANSFORM, p.W > SMALL_W_MAX ? 2 : 1);
+      StageTimer tm(c, KUBO_STAGE_BACKTRANSFORM, 2);
       KCHECK(eigh_vectors(c, n, eb, E, U));
     }
     if (out) {
@@ -1890,6 +1928,7 @@ kubo_status kubo_eigh_batched(const double* A, int W, int64_t n, double* E, doub
     p.eigh = true;
     p.lbuf = W > SMALL_W_MAX;
     plan_layout(p, false, 0);
+    fit_workspace(p, o);
     c.s = (cudaStream_t)o.stream;
     kubo_status r = c.acquire(o);
     if (r != KUBO_OK) return r;
@@ -1929,15 +1968,17 @@ kubo_status kubo_berry_batched(const double* E, const double* U, const double* d
     Call c;
     Plan& p = c.p;
     p.W = W; p.n_eta = o.n_eta > 0 ? o.n_eta : 1; p.n_EF = 1;
+    p.chunk = o.chunk_k > 0 ? o.chunk_k : auto_chunk(W, p.n_eta, n);
     p.lbuf = W > SMALL_W_MAX;   // the GEMM products of large orders go through the workspace
-    p.chunk = p.lbuf ? (o.chunk_k > 0 ? o.chunk_k : auto_chunk(W, p.n_eta, n)) : 0;
+    p.user_u = !p.lbuf;
     plan_layout(p, false, 0);
+    fit_workspace(p, o);
     c.s = (cudaStream_t)o.stream;
     kubo_status r = c.acquire(o);
     if (r != KUBO_OK) return r;
     r = upload_etas(c, o, eta);
     const size_t WW = (size_t)W * W;
-    const int64_t step = p.lbuf ? p.chunk : 1 << 30;
+    const int64_t step = p.chunk;
     for (int64_t t0 = 0; t0 < n && r == KUBO_OK; t0 += step) {
       int nn = (int)std::min<int64_t>(step, n - t0);
       if (berry_any(c, E + t0 * W, (const double2*)U + t0 * WW, dHx + t0 * WW, dHy + t0 * WW, (int64_t)WW,

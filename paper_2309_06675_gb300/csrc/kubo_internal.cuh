@@ -214,18 +214,11 @@ cudaError_t launch_iit_df(int W, int n, EighBufs b, double* E, double* Z, double
 cudaError_t launch_backtransform(int W, int n, EighBufs b, double* E, double2* U,
                                  cudaStream_t s, int pad = 1);
 
-cudaError_t launch_berry_fp64(const double* E, const double2* U, const double* Xp,
-                              const double* Yp, int W, int n, const double* etas, int n_eta,
-                              double* Om, int64_t eta_stride, cudaStream_t s, int pad = 1);
-
 // rotations from packed dH rows of leading dimension ld (d_x H at column offset W*W, d_y H at
-// 2*W*W, as written by the tensor-core Fourier kernel): in FP32 (mixed) or in FP64
+// 2*W*W, as written by the tensor-core Fourier kernel), in FP32
 cudaError_t launch_berry_mixed_rows(const double* E, const double2* U, const double* C,
                                     int64_t ld, int W, int n, const double* etas, int n_eta,
                                     double* Om, int64_t eta_stride, cudaStream_t s, int pad = 1);
-cudaError_t launch_berry_fp64_rows(const double* E, const double2* U, const double* C,
-                                   int64_t ld, int W, int n, const double* etas, int n_eta,
-                                   double* Om, int64_t eta_stride, cudaStream_t s, int pad = 1);
 
 // FP32 rotations with U = Q D Z assembled in FP32 inside the kernel from Z and the eigensolver
 // factors in eb (phase, refl, tau), W <= 64.  vel32 (these and the two tensor-core forms
@@ -332,6 +325,16 @@ cudaError_t launch_fixup_scatter(const int* pos, int cnt, int W, int n_eta, cons
                                  const double* Omfix, int64_t fix_eta_stride, double* E, double* Om,
                                  int64_t eta_stride, cudaStream_t s);
 
+// FP64-grade products on the integer pipe, W <= 64 (k_fixed.cu).  Rotations and curvature from
+// packed FP64 dH rows of leading dimension ld; ue: per-matrix exponent of U's column norms (from
+// launch_unorm), null for unit columns.  U = Q D Z from the eigenvectors Z of T.
+cudaError_t launch_unorm(const double2* U, int W, int n, int* ue, cudaStream_t s);
+cudaError_t launch_berry_fix(const double* E, const double2* U, const double* Xp, const double* Yp,
+                             int64_t ld, int W, int n, const double* etas, int n_eta, double* Om,
+                             int64_t eta_stride, const int* ue, cudaStream_t s, int pad = 1);
+cudaError_t launch_reflect_fix(int W, int n, EighBufs b, const double* Z, double2* U, cudaStream_t s,
+                               int pad = 1);
+
 // k_large.cu: sorted eigenvalues E and eigenvectors Z of T by inverse iteration ([n][W][W]
 // real, column m for sorted eigenvalue m; Z may be null: eigenvalues only), any W <= 128,
 // at most `slots` persistent CTAs (iit_max_slots(W) fill the GPU) with
@@ -399,6 +402,5 @@ size_t tridiag_smem(int W);
 size_t tridiag_df_smem(int W);
 size_t backtransform_smem(int W);
 size_t ql_smem(int W);
-size_t berry_fp64_smem(int W, int n_eta);
 
 }  // namespace kubo

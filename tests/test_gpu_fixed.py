@@ -1,0 +1,83 @@
+"""Integer-pipe products of FP64 grade (rotations, U = Q D Z) against extended precision.
+
+Orders around the tiles (2 x 2 below 13, 4 x 2 from there; 4 reflectors per block), magnitudes far from
+1, eigenvectors that are not normalised, non-finite operands.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(W, n, seed):
+    rng = np.random.default_rng(seed)
+    z = rng.standard_normal((3, n, W, W)) + 1j * rng.standard_normal((3, n, W, W))
+    A = z + z.conj().transpose(0, 1, 3, 2)
+    E, U = np.linalg.eigh(A[0])
+    return A, E, U
+
+
+def _velocities(U, X, Y):
+    L = np.clongdouble
+    Uh = U.conj().transpose(0, 2, 1).astype(L)
+    return Uh @ X.astype(L) @ U.astype(L), Uh @ Y.astype(L) @ U.astype(L)
+
+
+def _curvature(E, vx, vy, eta):
+    d2 = (E[:, :, None] - E[:, None, :]).astype(np.longdouble) ** 2 + np.longdouble(eta) ** 2
+    num = -2 * (vx * vy.conj()).imag
+    T = num / np.where(d2 == 0, 1, d2)
+    T[:, np.arange(E.shape[1]), np.arange(E.shape[1])] = 0
+    # size of the terms that enter Omega_n, for the error bound
+    size = (np.abs(vx).max((1, 2)) * np.abs(vy).max((1, 2)))[:, None, None] / d2
+    return T.sum(2), size
+
+
+@pytest.mark.parametrize("W", [1, 2, 3, 4, 5, 11, 12, 13, 16, 31, 33, 48, 63, 64])
+@pytest.mark.parametrize("sx,sy,su", [(1.0, 1.0, 1.0), (2.0 ** 130, 2.0 ** -90, 1.0), (1.0, 1.0, 3.0)])
+def test_curvature(W, sx, sy, su):
+    import torch
+    import paper_2309_06675_gb300 as kubo
+    n = 7 if W <= 64 else 2
+    A, E, U = _problem(W, n, W)
+    X, Y, U = A[1] * sx, A[2] * sy, U * su
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()   # noqa: E731
+    got = kubo.berry_batched(d(E), d(U), kubo.pack_hermitian(d(X)), kubo.pack_hermitian(d(Y)),
+                             etas=[1e-2, 0.5]).cpu().numpy()
+    vx, vy = _velocities(U, X, Y)
+    for e, eta in enumerate([1e-2, 0.5]):
+        ref, size = _curvature(E, vx, vy, eta)
+        # v to 2^-51 of the norm of the operands (at most W times the largest entry of v)
+        bound = (size * W * 2.0 ** -49).sum(2)
+        assert (np.abs(got[e] - ref) <= bound).all(), float((np.abs(got[e] - ref) / bound).max())
+
+
+def test_non_finite_operands():
+    import torch
+    import paper_2309_06675_gb300 as kubo
+    A, E, U = _problem(20, 4, 1)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()   # noqa: E731
+    X = kubo.pack_hermitian(d(A[1]))
+    Y = kubo.pack_hermitian(d(A[2]))
+    X[1, 7] = float("inf")
+    Ud = d(U)
+    Ud[2, 3, 4] = float("nan")
+    got = kubo.berry_batched(d(E), Ud, X, Y, eta=0.1).cpu().numpy()[0]
+    assert np.isfinite(got[0]).all() and np.isfinite(got[3]).all()
+    assert np.isnan(got[1]).all() and np.isnan(got[2]).all()
+
+
+@pytest.mark.parametrize("W", [1, 2, 3, 6, 7, 18, 32, 33, 47, 64])
+def test_eigenvectors(W):
+    import torch
+    import paper_2309_06675_gb300 as kubo
+    n = 9
+    A = _problem(W, n, 100 + W)[0][0]
+    E, U = kubo.eigh_batched(kubo.pack_hermitian(torch.from_numpy(A).cuda()), W)
+    E, U = E.cpu().numpy(), U.cpu().numpy()
+    L = np.clongdouble
+    norm = np.abs(E).max(1)[:, None, None]
+    res = np.abs(A.astype(L) @ U.astype(L) - U.astype(L) * E[:, None, :]) / norm
+    orth = np.abs(U.conj().transpose(0, 2, 1).astype(L) @ U.astype(L) - np.eye(W))
+    # a W-step reduction at 2^-52 of the norm per step and entry
+    assert res.max() <= 4 * W * 2.0 ** -52 and orth.max() <= 4 * W * 2.0 ** -52, (res.max(), orth.max())
