@@ -29,6 +29,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include "digits.cuh"
 #include "kubo_internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -37,11 +38,12 @@ namespace kubo {
 namespace {
 
 using namespace tc;
+using namespace dig;
 
 constexpr int BM = 128;          // k-points per tile (UMMA M)
 constexpr int BN = 32;           // output columns per tile: 7 levels x 32 columns x 2 sets of TMEM
 constexpr int BK = 64;           // K per block: one 128-byte swizzle row of bf16
-constexpr int NS = 7;            // slices per operand and levels kept: 28 digit products
+constexpr int NS = ND;           // seven slices per operand and levels kept: 28 digit products
 constexpr int NACC = 2;          // accumulator sets: one drained while the other is filled
 constexpr int SET_COLS = 256;    // TMEM columns of a set (7 x 32 used)
 constexpr int DRAIN = 2;         // K blocks per drain: 7 x 128 x 2^14 < 2^24
@@ -62,36 +64,6 @@ constexpr int EXP_NONFINITE = INT_MAX;     // column with an infinite or NaN bas
 __host__ __device__ constexpr uint32_t idesc_n(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
-
-// ------------------------------------------------------------------ digits
-// round(x 2^(55 - e)) for |x| <= 2^e, from the FP64 bit pattern (round half up of the
-// magnitude; no FP64 instruction): |q| <= 2^55
-__device__ __forceinline__ long long fixed55(double x, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  int ex = (int)((b >> 52) & 0x7FF);
-  unsigned long long m = b & ((1ull << 52) - 1);
-  if (ex == 0) ex = 1;
-  else m |= 1ull << 52;
-  const int sh = 1020 + e - ex;   // x 2^(55-e) = m 2^(ex - 1075 + 55 - e) = m 2^-sh, sh >= -3
-  const unsigned long long q = sh <= 0 ? m << -sh : (sh < 64 ? (m + (1ull << (sh - 1))) >> sh : 0ull);
-  return (b >> 63) ? -(long long)q : (long long)q;
-}
-// signed base-256 digits of q (|q| <= 2^55), most significant first, as FP32 integers: adding
-// 128 to the six low digits makes them plain bytes; a byte b becomes the float b - 128 by
-// placing it in the mantissa of 2^23 and subtracting 2^23 + 128 (exact).  The upper half of
-// such a float is the digit in BF16.
-__device__ __forceinline__ void digits7(long long q, uint32_t (&d)[NS]) {
-  const long long v = q + 0x0000808080808080ll;
-  const uint32_t lo = (uint32_t)v, hi = (uint32_t)((unsigned long long)v >> 32);
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {   // byte j of v -> digit 6 - j
-    const uint32_t f = __byte_perm(j < 4 ? lo : hi, 0x4B000000u, 0x7650u | (j & 3));
-    d[6 - j] = __float_as_uint(__uint_as_float(f) - 8388736.0f);
-  }
-  d[0] = __float_as_uint((float)(int)(v >> 48));
-}
-// two digits as a bf16 pair (a low)
-__device__ __forceinline__ uint32_t bf16_pair(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
 
 // ------------------------------------------------------------------ operand preparation
 // e[a W^2 + q] (a = H, d_x, d_y; padding columns 0): exponent with |basis| < 2^e over K, from the
@@ -234,15 +206,102 @@ __global__ void __launch_bounds__(256) coef_slice7_kernel(Model md, Mesh mesh, K
   }
 }
 
+// ------------------------------------------------------------------ transposed sum (gradient)
+// G_rows[1 + 2 N_h][3 W^2] += Coef^T . [Hbar | dxHbar | dyHbar]: the same GEMM with the k-points as its
+// inner index.  A[s][row][k]: rows 1, cos k.R_h, sin k.R_h (grad_finalize_kernel's order), zero for
+// k >= n.
+__global__ void __launch_bounds__(256) coef_t_slice7_kernel(Model md, Mesh mesh, KList kl, int Mpad,
+                                                            int Kp, __nv_bfloat16* __restrict__ A) {
+  const int npair = Kp / 2;
+  const size_t plane = (size_t)Mpad * Kp;
+  const FastDiv f1((uint32_t)mesh.N1), f2((uint32_t)mesh.N2), f3((uint32_t)mesh.N3);
+  const int64_t total = (int64_t)(md.N_h + 1) * npair;
+  for (int64_t idx = blockIdx.x * (int64_t)256 + threadIdx.x; idx < total; idx += (int64_t)gridDim.x * 256) {
+    const int h = (int)(idx / npair) - 1;
+    const int k2 = 2 * (int)(idx % npair);
+    uint32_t dc[2][NS], ds[2][NS];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+#pragma unroll
+      for (int i = 0; i < NS; ++i) dc[b][i] = ds[b][i] = 0u;
+      if (k2 + b >= kl.n) continue;
+      if (h < 0) {
+        dc[b][0] = __float_as_uint(128.0f);
+      } else {
+        int j1, j2, j3;
+        mesh_coords(mesh, klist_get(kl, k2 + b), j1, j2, j3);
+        const int* r = md.Rh + 3 * h;
+        const double2 p = cmul(md.tab[md.tab_off[0] + posmod((long long)j1 * r[0], f1)],
+                               md.tab[md.tab_off[1] + posmod((long long)j2 * r[1], f2)]);
+        const double2 c = cmul(p, md.tab[md.tab_off[2] + posmod((long long)j3 * r[2], f3)]);
+        digits7(fixed55(c.x, 0), dc[b]);
+        digits7(fixed55(c.y, 0), ds[b]);
+      }
+    }
+    __nv_bfloat16* rc = A + (size_t)(1 + h) * Kp + k2;
+    __nv_bfloat16* rs = A + (size_t)(1 + md.N_h + h) * Kp + k2;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      *reinterpret_cast<uint32_t*>(rc + i * plane) = bf16_pair(dc[0][i], dc[1][i]);
+      if (h >= 0) *reinterpret_cast<uint32_t*>(rs + i * plane) = bf16_pair(ds[0][i], ds[1][i]);
+    }
+  }
+}
+
+// e[c]: exponent above column c of M [n][N] (rows blockIdx.y * 256 ..; e starts far below zero)
+__global__ void __launch_bounds__(256) col_exp7_kernel(const double* __restrict__ M, int n, int N,
+                                                       int* __restrict__ e) {
+  __shared__ unsigned red[8][32];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int c = blockIdx.x * 32 + x;
+  unsigned m = 0u;
+  if (c < N)
+    for (int k = blockIdx.y * 256 + y; k < min(n, (int)blockIdx.y * 256 + 256); k += 8)
+      m = max(m, (unsigned)(mag_bits(M[(size_t)k * N + c]) >> 32));
+  red[y][x] = m;
+  __syncthreads();
+  if (y == 0 && c < N) {
+    for (int i = 1; i < 8; ++i) m = max(m, red[i][x]);
+    const int ex = (int)(m >> 20);
+    atomicMax(&e[c], ex == 0x7FF ? EXP_NONFINITE : ex - 1022);
+  }
+}
+
+// Bt[s][c][k] of M [n][N]: 32 columns x 64 k per block, transposed through shared memory
+__global__ void __launch_bounds__(256) col_slice7_kernel(const double* __restrict__ M, int n, int N,
+                                                         const int* __restrict__ e, int Npad, int Kp,
+                                                         __nv_bfloat16* __restrict__ Bt) {
+  __shared__ double sm[64][33];
+  const int c0 = blockIdx.x * 32, k0 = blockIdx.y * 64;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  for (int kk = y; kk < 64; kk += 8) {
+    const int k = k0 + kk, c = c0 + x;
+    sm[kk][x] = k < n && c < N ? M[(size_t)k * N + c] : 0.0;
+  }
+  __syncthreads();
+  const size_t plane = (size_t)Npad * Kp;
+  for (int cc = y; cc < 32; cc += 8) {
+    const int c = c0 + cc;
+    if (c >= N) break;
+    const int ec = e[c] == EXP_NONFINITE ? 1024 : e[c];
+    uint32_t d0[NS], d1[NS];
+    digits7(fixed55(sm[2 * x][cc], ec), d0);
+    digits7(fixed55(sm[2 * x + 1][cc], ec), d1);
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+      *reinterpret_cast<uint32_t*>(Bt + i * plane + (size_t)c * Kp + k0 + 2 * x) = bf16_pair(d0[i], d1[i]);
+  }
+}
+
 // ------------------------------------------------------------------ the tcgen05 GEMM
 // Persistent: CTA b walks tiles b, b + gridDim.x, ...; group_m M tiles per column tile in a row,
 // so a B tile serves several tiles and the group's A slices stay in L2.
 __global__ void __launch_bounds__(TC_THREADS, 1)
     fourier_tc64_kernel(const __grid_constant__ CUtensorMap mapA,
                         const __grid_constant__ CUtensorMap mapB, const int* __restrict__ col_exp,
-                        int Mpad, int Npad, int nkb, int n_rows, int WW, double* __restrict__ Hp,
-                        double* __restrict__ Xp, double* __restrict__ Yp, DevStatus* st,
-                        int group_m, bool vec) {
+                        int Mpad, int Npad, int nkb, int n_rows, int WW, double* Hp, double* Xp,
+                        double* Yp, int64_t ldo, bool accum, DevStatus* st, int group_m,
+                        bool vec) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t a_full[NA], a_empty[NA], b_full[NB], b_empty[NB];
@@ -417,7 +476,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         mbar_arrive(&acc_empty[a]);
       }
       if (!ok) break;
-      const int grow = m0 + row;
+      const int64_t grow = m0 + row;
       if (grow < n_rows) {
         // C = 2^e (hi 2^-30 + lo 2^-62): both parts are exact in FP64, the FMA rounds once
         const int n1 = n0 + c_lo;
@@ -435,10 +494,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (vec) {
           if (n1 < 3 * WW) {
             const int a = n1 / WW;
-            double* dst = (a == 0 ? Hp : a == 1 ? Xp : Yp) + (size_t)grow * WW + (n1 - a * WW);
+            double* dst = (a == 0 ? Hp : a == 1 ? Xp : Yp) + grow * ldo + (n1 - a * WW);
 #pragma unroll
-            for (int j = 0; j < EPI_COLS; j += 2)
-              *reinterpret_cast<double2*>(dst + j) = make_double2(v[j], v[j + 1]);
+            for (int j = 0; j < EPI_COLS; j += 2) {
+              double2 w = make_double2(v[j], v[j + 1]);
+              if (accum) {
+                const double2 o = *reinterpret_cast<const double2*>(dst + j);
+                w.x += o.x;
+                w.y += o.y;
+              }
+              *reinterpret_cast<double2*>(dst + j) = w;
+            }
           }
         } else {
 #pragma unroll
@@ -446,7 +512,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             const int n = n1 + j;
             if (n < 3 * WW) {
               const int a = n < WW ? 0 : n < 2 * WW ? 1 : 2;
-              (a == 0 ? Hp : a == 1 ? Xp : Yp)[(size_t)grow * WW + (n - a * WW)] = v[j];
+              double* dst = (a == 0 ? Hp : a == 1 ? Xp : Yp) + grow * ldo + (n - a * WW);
+              *dst = accum ? *dst + v[j] : v[j];
             }
           }
         }
@@ -497,9 +564,10 @@ cudaError_t launch_coef_split64(const Model& md, const Mesh& mesh, const KList& 
   return cudaGetLastError();
 }
 
-cudaError_t launch_fourier_tc64(const void* A, const void* Bt, const int* col_exp, int Mpad,
-                                int Npad, int Kp, int n_rows, int W, double* Hp, double* Xp,
-                                double* Yp, DevStatus* st, cudaStream_t s) {
+// out: three arrays [n_rows][W^2] of row stride ldo, overwritten or added to
+static cudaError_t launch_gemm7(const void* A, const void* Bt, const int* col_exp, int Mpad, int Npad,
+                                int Kp, int n_rows, int W, double* Hp, double* Xp, double* Yp,
+                                int64_t ldo, bool accum, DevStatus* st, cudaStream_t s) {
   if (n_rows <= 0) return cudaSuccess;
   if (Mpad % BM || Npad % BN || Kp % BK) return cudaErrorInvalidValue;
   CUtensorMap mA, mB;
@@ -515,11 +583,37 @@ cudaError_t launch_fourier_tc64(const void* A, const void* Bt, const int* col_ex
   // 48 MB of the L2, so that the basis is read from HBM once per group
   const int64_t per_m = (int64_t)BM * Kp * 2 * NS;
   const int group_m = (int)std::max<int64_t>(1, std::min<int64_t>(64, ((int64_t)48 << 20) / per_m));
-  const bool vec = W % 4 == 0 && (((uintptr_t)Hp | (uintptr_t)Xp | (uintptr_t)Yp) & 15) == 0;
+  const bool vec = W % 4 == 0 && ldo % 2 == 0 && (((uintptr_t)Hp | (uintptr_t)Xp | (uintptr_t)Yp) & 15) == 0;
   const int tiles = (Mpad / BM) * (Npad / BN);
   fourier_tc64_kernel<<<std::min(tiles, std::max(nsm, 1)), TC_THREADS, SMEM_BYTES, s>>>(
-      mA, mB, col_exp, Mpad, Npad, Kp / BK, n_rows, W * W, Hp, Xp, Yp, st, group_m, vec);
+      mA, mB, col_exp, Mpad, Npad, Kp / BK, n_rows, W * W, Hp, Xp, Yp, ldo, accum, st, group_m, vec);
   return cudaGetLastError();
+}
+
+cudaError_t launch_fourier_tc64(const void* A, const void* Bt, const int* col_exp, int Mpad,
+                                int Npad, int Kp, int n_rows, int W, double* Hp, double* Xp,
+                                double* Yp, DevStatus* st, cudaStream_t s) {
+  return launch_gemm7(A, Bt, col_exp, Mpad, Npad, Kp, n_rows, W, Hp, Xp, Yp, (int64_t)W * W, false, st, s);
+}
+
+cudaError_t launch_grad_fourier_t(const Model& md, const Mesh& mesh, const KList& kl, const double* Mbar,
+                                  void* A, void* Bt, int* col_exp, double* Gacc, DevStatus* st,
+                                  cudaStream_t s) {
+  if (kl.n <= 0) return cudaSuccess;
+  const int WW = md.W * md.W, N = 3 * WW, rows = 1 + 2 * md.N_h;
+  const int Npad = tc64_pad_n(md.W), Mpad = tc_pad_m(rows), Kp = tc_pad_k(kl.n);
+  const int64_t total = (int64_t)(md.N_h + 1) * (Kp / 2);
+  coef_t_slice7_kernel<<<(int)std::min<int64_t>((total + 255) / 256, 152 * 32), 256, 0, s>>>(
+      md, mesh, kl, Mpad, Kp, (__nv_bfloat16*)A);
+  cudaError_t e = cudaMemsetAsync(col_exp, 0xC0, sizeof(int) * (size_t)Npad, s);
+  if (e != cudaSuccess) return e;
+  col_exp7_kernel<<<dim3((N + 31) / 32, (kl.n + 255) / 256), 256, 0, s>>>(Mbar, kl.n, N, col_exp);
+  col_slice7_kernel<<<dim3((N + 31) / 32, Kp / 64), 256, 0, s>>>(Mbar, kl.n, N, col_exp, Npad, Kp,
+                                                                  (__nv_bfloat16*)Bt);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_gemm7(A, Bt, col_exp, Mpad, Npad, Kp, rows, md.W, Gacc, Gacc + WW, Gacc + 2 * WW, N, true,
+                      st, s);
 }
 
 }  // namespace kubo

@@ -1,5 +1,5 @@
 // Reverse mode of steps (1)-(4) (Eq. 2-3): the gradient of L = sum_{e,j} g[e][j] S_e(E_F_j)
-// with respect to every entry of H(R), FP64 throughout.
+// with respect to every entry of H(R), in FP64 grade.
 //
 // Per k-point, from the forward quantities E, U, v^x = U^dagger dxH U, v^y = U^dagger dyH U:
 //   a[e][n]  = sum_j g[e][j] occ_j(E_n) / N_k,   a'[e][n] = sum_j g[e][j] occ_j'(E_n) / N_k
@@ -16,6 +16,8 @@
 // evaluated as one real GEMM over the canonical half set of R: rows (1, cos k.R_h, sin k.R_h)
 // against the packed Hermitian columns [Hbar | dxHbar | dyHbar], accumulated over batches in
 // a fixed order (deterministic), and unfolded into G(R_h), G(-R_h) = G(R_h)^dagger, G(0).
+// This file: the elementwise kernels between the matrix products, which run on the tensor cores in
+// FP64 grade (k_zgemm_tc64.cu, k_fourier_tc64.cu).
 #include <algorithm>
 
 #include "kubo_internal.cuh"
@@ -24,87 +26,8 @@ namespace kubo {
 
 namespace {
 
-constexpr int GT = 64, GK = 16;   // GEMM tiles: up to 64 x 64 outputs, K steps of 16
 constexpr int MAXE = 8;
 constexpr int PW = 128;            // threads of the per-k kernels (W <= 128)
-
-// ------------------------------------------------------------------ batched complex GEMM
-// C[k] = op(A[k]) op(B[k]) (+ C[k]), W x W complex FP64, op = identity or conjugate transpose.
-// Output tile T = 16 TM (TM x TM per thread); TM = 2 for W <= 32 so no thread multiplies padding.
-template <bool HA, bool HB, bool ACC, int TM>
-__global__ void __launch_bounds__(256) zgemm_kernel(const double2* __restrict__ A,
-                                                    const double2* __restrict__ B,
-                                                    double2* __restrict__ C, int W) {
-  constexpr int T = 16 * TM;
-  __shared__ double2 As[T][GK + 1];
-  __shared__ double2 Bs[GK][T + 1];
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int nt = (W + T - 1) / T;
-  const int r0 = (blockIdx.y / nt) * T, c0 = (blockIdx.y % nt) * T;
-  const size_t base = (size_t)blockIdx.x * W * W;
-  const double2* Ak = A + base;
-  const double2* Bk = B + base;
-  double ax[TM][TM], ay[TM][TM];
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TM; ++j) { ax[i][j] = 0.0; ay[i][j] = 0.0; }
-  for (int q0 = 0; q0 < W; q0 += GK) {
-    for (int idx = t; idx < T * GK; idx += 256) {
-      int r, q;
-      if (HA) { q = idx / T; r = idx % T; } else { r = idx / GK; q = idx % GK; }
-      const int gr = r0 + r, gq = q0 + q;
-      double2 a = make_double2(0.0, 0.0);
-      if (gr < W && gq < W) {
-        if (HA) { a = Ak[(size_t)gq * W + gr]; a.y = -a.y; }
-        else a = Ak[(size_t)gr * W + gq];
-      }
-      As[r][q] = a;
-    }
-    for (int idx = t; idx < GK * T; idx += 256) {
-      int q, c;
-      if (HB) { c = idx / GK; q = idx % GK; } else { q = idx / T; c = idx % T; }
-      const int gq = q0 + q, gc = c0 + c;
-      double2 b = make_double2(0.0, 0.0);
-      if (gq < W && gc < W) {
-        if (HB) { b = Bk[(size_t)gc * W + gq]; b.y = -b.y; }
-        else b = Bk[(size_t)gq * W + gc];
-      }
-      Bs[q][c] = b;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < GK; ++q) {
-      double2 a[TM], b[TM];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[ty + 16 * i][q];
-#pragma unroll
-      for (int j = 0; j < TM; ++j) b[j] = Bs[q][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-          ax[i][j] = fma(a[i].x, b[j].x, ax[i][j]);
-          ax[i][j] = fma(-a[i].y, b[j].y, ax[i][j]);
-          ay[i][j] = fma(a[i].x, b[j].y, ay[i][j]);
-          ay[i][j] = fma(a[i].y, b[j].x, ay[i][j]);
-        }
-    }
-    __syncthreads();
-  }
-  double2* Ck = C + base;
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TM; ++j) {
-      const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * j;
-      if (r < W && c < W) {
-        double2 v = make_double2(ax[i][j], ay[i][j]);
-        if (ACC) { const double2 o = Ck[(size_t)r * W + c]; v.x += o.x; v.y += o.y; }
-        Ck[(size_t)r * W + c] = v;
-      }
-    }
-}
 
 // ------------------------------------------------------------------ occupations
 __device__ __forceinline__ void occ_and_derivative(double E, double EF, double kT, double& f,
@@ -261,75 +184,6 @@ __global__ void pack3_kernel(const double2* __restrict__ A0, const double2* __re
   }
 }
 
-// Coef[row][kk] for row 0 (R = 0: 1), 1 + h (cos k.R_h), 1 + N_h + h (sin k.R_h)
-__global__ void grad_coef_kernel(Model md, Mesh mesh, KList kl, int ldc, double* __restrict__ Coef) {
-  const int64_t total = (int64_t)(md.N_h + 1) * kl.n;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int h = (int)(t / kl.n) - 1;
-    const int kk = (int)(t % kl.n);
-    if (h < 0) {
-      Coef[kk] = 1.0;
-      continue;
-    }
-    int j1, j2, j3;
-    mesh_coords(mesh, klist_get(kl, kk), j1, j2, j3);
-    const int* r = md.Rh + 3 * h;
-    const double2 e = mesh_phase(md.tab, md.tab_off, mesh, j1, j2, j3, r[0], r[1], r[2]);
-    Coef[(size_t)(1 + h) * ldc + kk] = e.x;
-    Coef[(size_t)(1 + md.N_h + h) * ldc + kk] = e.y;
-  }
-}
-
-// Gacc[M][N] += Coef[M][K] Mbar[K][N], real FP64, 64 x 64 tiles; K in order (deterministic)
-__global__ void __launch_bounds__(256) grad_fourier_t_kernel(const double* __restrict__ Coef,
-                                                             int ldc, const double* __restrict__ Mb,
-                                                             int M, int N, int K,
-                                                             double* __restrict__ Gacc) {
-  __shared__ double As[GT][GK + 1];
-  __shared__ double Bs[GK][GT + 1];
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int r0 = blockIdx.y * GT, c0 = blockIdx.x * GT;
-  double acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  for (int q0 = 0; q0 < K; q0 += GK) {
-    for (int idx = t; idx < GT * GK; idx += 256) {
-      const int r = idx / GK, q = idx % GK;
-      const int gr = r0 + r, gq = q0 + q;
-      As[r][q] = (gr < M && gq < K) ? Coef[(size_t)gr * ldc + gq] : 0.0;
-    }
-    for (int idx = t; idx < GK * GT; idx += 256) {
-      const int q = idx / GT, c = idx % GT;
-      const int gq = q0 + q, gc = c0 + c;
-      Bs[q][c] = (gq < K && gc < N) ? Mb[(size_t)gq * N + gc] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < GK; ++q) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[ty + 16 * i][q];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[q][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * j;
-      if (r < M && c < N) Gacc[(size_t)r * N + c] += acc[i][j];
-    }
-}
-
 // unpack element (i, j) of the Hermitian matrix whose packed form is P (W x W reals)
 __device__ __forceinline__ double2 herm_at(const double* P, int W, int i, int j) {
   if (i < j) return make_double2(P[i * W + j], P[j * W + i]);
@@ -368,26 +222,6 @@ __global__ void grad_finalize_kernel(const double* __restrict__ Gacc, const int*
 
 }  // namespace
 
-cudaError_t launch_zgemm_batched(bool hA, bool hB, bool acc, const double2* A, const double2* B,
-                                 double2* C, int W, int n, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const int T = W <= 32 ? 32 : GT;
-  const int tiles = (W + T - 1) / T;
-  dim3 grid(n, tiles * tiles);
-#define ZG(a, b, c)                                                          \
-  do {                                                                       \
-    if (T == 32) zgemm_kernel<a, b, c, 2><<<grid, 256, 0, s>>>(A, B, C, W);  \
-    else zgemm_kernel<a, b, c, 4><<<grid, 256, 0, s>>>(A, B, C, W);          \
-  } while (0)
-  if (!hA && !hB && !acc) ZG(false, false, false);
-  else if (!hA && !hB && acc) ZG(false, false, true);
-  else if (hA && !hB && !acc) ZG(true, false, false);
-  else if (!hA && hB && !acc) ZG(false, true, false);
-  else return cudaErrorInvalidValue;
-#undef ZG
-  return cudaGetLastError();
-}
-
 cudaError_t launch_grad_pairs(const double* E, const double2* vx, const double2* vy, int W, int n,
                               const double* g, const double* E_F, int n_EF, const double* etas,
                               int n_eta, double kT, double inv_Nk, double2* vbx, double2* vby,
@@ -413,23 +247,6 @@ cudaError_t launch_pack3(const double2* A0, const double2* A1, const double2* A2
   const int64_t total = (int64_t)n * W * W;
   const int b = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
   pack3_kernel<<<b, 256, 0, s>>>(A0, A1, A2, W, n, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_grad_coef(const Model& md, const Mesh& mesh, const KList& kl, int ldc,
-                             double* Coef, cudaStream_t s) {
-  if (kl.n <= 0) return cudaSuccess;
-  const int64_t total = (int64_t)(md.N_h + 1) * kl.n;
-  const int b = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
-  grad_coef_kernel<<<b, 256, 0, s>>>(md, mesh, kl, ldc, Coef);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_grad_fourier_t(const double* Coef, int ldc, const double* Mbar, int M, int N,
-                                  int K, double* Gacc, cudaStream_t s) {
-  if (K <= 0) return cudaSuccess;
-  dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT);
-  grad_fourier_t_kernel<<<grid, 256, 0, s>>>(Coef, ldc, Mbar, M, N, K, Gacc);
   return cudaGetLastError();
 }
 

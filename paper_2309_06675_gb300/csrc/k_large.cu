@@ -710,32 +710,6 @@ __global__ void __launch_bounds__(LW_MAX) curvature_large_kernel(const double* _
       if (e >= n_eta) break;
       Om[e * eta_stride + k * W + n] = ((double)hi[e] + (double)lo[e]) + fb[e];
     }
-  } else {
-    double rp[MAXE];
-#pragma unroll
-    for (int e = 0; e < MAXE; ++e) rp[e] = 0.0;
-    for (int m = 0; m < W; ++m) {
-      if (m == n) continue;
-      const int p = n < m ? n : m, q = n < m ? m : n;
-      const typename cx<T>::type vx = Vx[base + (size_t)p * W + q];
-      const typename cx<T>::type vy = Vy[base + (size_t)p * W + q];
-      const double num = -2.0 * ((double)vx.y * (double)vy.x - (double)vx.x * (double)vy.y);
-      const double dE = sE[p] - sE[q];
-      const double d2 = dE * dE;
-      const double sgn = n < m ? 1.0 : -1.0;   // T_nm = -T_mn: evaluated from the (p < q) entry
-#pragma unroll
-      for (int e = 0; e < MAXE; ++e) {
-        if (e >= n_eta) break;
-        const double eta = etas[e];
-        if (eta == 0.0 && d2 <= thr2) continue;
-        rp[e] += sgn * (num / fma(eta, eta, d2));
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < MAXE; ++e) {
-      if (e >= n_eta) break;
-      Om[e * eta_stride + k * W + n] = rp[e];
-    }
   }
 }
 
@@ -793,46 +767,22 @@ cudaError_t launch_reflect_wy(int W, int n, EighBufs b, const double* Z, float2*
   return cudaGetLastError();
 }
 
-// T[k] = X[k] U[k], X packed Hermitian rows of leading dimension ld, FP64 (any W <= 128)
-cudaError_t launch_herm_u(const double* X, int64_t ld, const double2* U, double2* T, int W, int n,
-                          cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  if (W > LW_MAX) return cudaErrorInvalidValue;
-  const int tiles = (W + GT - 1) / GT;
-  dim3 grid(n, tiles * tiles);
-  cgemm_herm_u_kernel<double><<<grid, 256, 0, s>>>(X, ld, U, W, T);
-  return cudaGetLastError();
-}
-
-// steps (3)-(4) for large W: X, Y packed Hermitian rows (leading dimension ld); U is float2
-// when f32 (formed in FP32 by launch_reflect_large), double2 otherwise.
-// f32 selects FP32 arithmetic for the products (mixed precision).  Tbuf, Vx, Vy: scratch of
-// n * W * W complex elements of the arithmetic type each.
+// steps (3)-(4) of the FP32-rotation modes for large W: X, Y packed Hermitian rows (leading
+// dimension ld), U float2.  Tbuf, Vx, Vy: scratch of n * W * W float2 each.
 cudaError_t launch_berry_large(const double* E, const void* Uv, const double* X, const double* Y,
                                int64_t ld, int W, int n, const double* etas, int n_eta, double* Om,
-                               int64_t eta_stride, bool f32, void* Tbuf, void* Vx, void* Vy,
-                               cudaStream_t s) {
+                               int64_t eta_stride, void* Tbuf, void* Vx, void* Vy, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (W > LW_MAX || n_eta > MAXE) return cudaErrorInvalidValue;
   const int tiles = (W + GT - 1) / GT;
   dim3 grid(n, tiles * tiles);
-  if (f32) {
-    const float2* U = (const float2*)Uv;
-    cgemm_herm_u_kernel<float><<<grid, 256, 0, s>>>(X, ld, U, W, (float2*)Tbuf);
-    cgemm_uh_t_kernel<float><<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vx);
-    cgemm_herm_u_kernel<float><<<grid, 256, 0, s>>>(Y, ld, U, W, (float2*)Tbuf);
-    cgemm_uh_t_kernel<float><<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vy);
-    curvature_large_kernel<float><<<n, LW_MAX, 0, s>>>(E, (const float2*)Vx, (const float2*)Vy, W,
-                                                        etas, n_eta, Om, eta_stride);
-  } else {
-    const double2* U = (const double2*)Uv;
-    cgemm_herm_u_kernel<double><<<grid, 256, 0, s>>>(X, ld, U, W, (double2*)Tbuf);
-    cgemm_uh_t_kernel<double><<<grid, 256, 0, s>>>(U, (const double2*)Tbuf, W, (double2*)Vx);
-    cgemm_herm_u_kernel<double><<<grid, 256, 0, s>>>(Y, ld, U, W, (double2*)Tbuf);
-    cgemm_uh_t_kernel<double><<<grid, 256, 0, s>>>(U, (const double2*)Tbuf, W, (double2*)Vy);
-    curvature_large_kernel<double><<<n, LW_MAX, 0, s>>>(E, (const double2*)Vx, (const double2*)Vy,
-                                                         W, etas, n_eta, Om, eta_stride);
-  }
+  const float2* U = (const float2*)Uv;
+  cgemm_herm_u_kernel<float><<<grid, 256, 0, s>>>(X, ld, U, W, (float2*)Tbuf);
+  cgemm_uh_t_kernel<float><<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vx);
+  cgemm_herm_u_kernel<float><<<grid, 256, 0, s>>>(Y, ld, U, W, (float2*)Tbuf);
+  cgemm_uh_t_kernel<float><<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vy);
+  curvature_large_kernel<float><<<n, LW_MAX, 0, s>>>(E, (const float2*)Vx, (const float2*)Vy, W,
+                                                      etas, n_eta, Om, eta_stride);
   return cudaGetLastError();
 }
 

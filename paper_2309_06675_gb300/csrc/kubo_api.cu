@@ -19,6 +19,12 @@ namespace {
 constexpr int MAX_W = LARGE_W_MAX;
 constexpr int SMALL_W_MAX = 64;      // beyond: the multi-pass eigenvector / rotation kernels
 constexpr int MAX_ETA = 8;
+// FP64 rotations: integer-pipe kernel (one launch, k-points packed in a CTA) up to this order, tensor-
+// core products above
+constexpr int FIX_W_MAX = 32;
+// k-points per sub-batch of the latter: T, v^x and v^y of a sub-batch (192 KB each at W = 64) are
+// written and read while they are in L2
+constexpr int ZG_BATCH = 152 * 8;
 constexpr int KSUM_KPB = 32;         // k-points per deterministic k-sum block (at least)
 constexpr size_t KSUM_PART_BYTES = (size_t)256 << 20;   // cap on the per-block partials
 // mixed precision: share of each batch (largest ||Omega(k)||_inf) redone in FP64
@@ -154,7 +160,8 @@ struct Plan {
   bool lbuf = false;    // W > SMALL_W_MAX: scratch of the multi-pass kernels
   bool grad = false;    // reverse-mode buffers (kubo_ahc_grad)
   bool iit = false;     // inverse-iteration scratch (separate eigenvector kernel)
-  bool lean = false;    // a caller's workspace too small for Z and the iteration scratch (W <= 64)
+  int zk = 0;           // k-points per sub-batch of the tensor-core rotations (FP64, W > FIX_W_MAX)
+  bool lean = false;    // a caller's workspace too small for Z, the iteration scratch and zg (W <= 64)
   bool user_u = false;  // eigenvectors from the caller (kubo_berry_batched): column norms on the device
   int iit_slots = 0;
   // separable Fourier sum: bounding box, pairs per batch, planes of the range
@@ -166,10 +173,11 @@ struct Plan {
          o_acc = 0, o_Hp = 0, o_Xp = 0, o_Yp = 0, o_E = 0, o_U = 0, o_Om = 0, o_d = 0, o_e = 0,
          o_ph = 0, o_refl = 0, o_tau = 0, o_lam = 0, o_part = 0,
          o_HR = 0, o_EF = 0, o_out = 0, o_Bt = 0, o_A = 0, o_C64 = 0, o_cexp = 0, o_L = 0,
-         o_iit = 0, o_Z = 0, o_ue = 0, o_box = 0, o_sepA = 0, o_sepB = 0, o_sepBy = 0;
+         o_iit = 0, o_Z = 0, o_ue = 0, o_zg = 0, o_ze = 0, o_box = 0, o_sepA = 0, o_sepB = 0, o_sepBy = 0;
   // reverse mode: six complex W x W work matrices per k, Ebar, packed [Hbar|dxHbar|dyHbar],
   // the Fourier coefficient rows of the batch and the accumulated G rows
-  size_t o_gw = 0, o_Ebar = 0, o_Mbar = 0, o_Coef = 0, o_Gacc = 0;
+  size_t o_gw = 0, o_ge = 0, o_Ebar = 0, o_Mbar = 0, o_tA = 0, o_tB = 0, o_texp = 0, o_Gacc = 0;
+  int t_k = 0;          // k-points per sub-batch of the transposed Fourier sum
   // mixed-precision fix-up buffers
   bool fixup = false;
   int fix_cap = 0;
@@ -297,6 +305,12 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
     else if (!p.lean && (!p.model || p.fixup || !f32_rotation(p.precision)))
       p.o_Z = b.take(sizeof(double) * WW * (size_t)std::max(1, p.chunk));
   }
+  p.zk = 0;
+  if ((p.berry || p.user_u) && !f32_rotation(p.precision) && p.W > FIX_W_MAX && !p.lean) {
+    p.zk = std::min(std::max(1, p.chunk), ZG_BATCH);
+    p.o_zg = b.take(3 * sizeof(double2) * WW * (size_t)p.zk);
+    p.o_ze = b.take(3 * sizeof(int) * (size_t)p.zk);
+  }
   // column norms of the caller's U (up to 48 of them in the unused part of the broadenings' block)
   if (p.user_u) p.o_ue = p.chunk <= 48 ? p.o_etas + sizeof(double) * MAX_ETA : b.take(sizeof(int) * (size_t)p.chunk);
   p.iit = p.eigh && !p.lean;
@@ -309,7 +323,14 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
     p.o_gw = b.take(6 * sizeof(double2) * ch * WW);
     p.o_Ebar = b.take(sizeof(double) * ch * p.W);
     p.o_Mbar = b.take(3 * sizeof(double) * ch * WW);
-    p.o_Coef = b.take(sizeof(double) * (size_t)(2 * p.N_h + 1) * ch);
+    p.o_ge = b.take(8 * sizeof(int) * ch);
+    // digit slices of the transposed sum's operands, k-points as its inner index: within 2 GiB
+    const size_t t_row = (size_t)2 * tc64_slices() * (tc64_pad_n(p.W) + tc_pad_m(2 * p.N_h + 1));
+    p.t_k = (int)std::max<size_t>(64, std::min<size_t>(std::min<size_t>(ch, 8192), kTc64CoefBytes / t_row / 64 * 64));
+    const size_t t_cols = (size_t)tc_pad_k(p.t_k);
+    p.o_tA = b.take((size_t)2 * tc64_slices() * tc_pad_m(2 * p.N_h + 1) * t_cols);
+    p.o_tB = b.take((size_t)2 * tc64_slices() * tc64_pad_n(p.W) * t_cols);
+    p.o_texp = b.take(sizeof(int) * (size_t)tc64_pad_n(p.W));
     p.o_Gacc = b.take(3 * sizeof(double) * (size_t)(2 * p.N_h + 1) * WW);
   }
   if (p.ksum) {
@@ -640,6 +661,35 @@ cudaError_t eigh_vectors(const Call& c, int n, const EighBufs& eb, double* E, do
   return launch_reflect_large(p.W, n, eb, Z, U, f32u, c.s);
 }
 
+// FP64 rotations by tensor-core products: T = dH U, v = U^H T (upper tiles), then the curvature.
+cudaError_t berry_tc64(const Call& c, const double* E, const double2* U, const int* ue, const double* X,
+                       const double* Y, int64_t ld, int n, double* Om, int64_t om_stride) {
+  const Plan& p = c.p;
+  const int64_t WW = (int64_t)p.W * p.W;
+  double2* T = c.at<double2>(p.o_zg);
+  double2* V[2] = {T + WW * p.zk, T + 2 * WW * p.zk};
+  int* eX = c.at<int>(p.o_ze);
+  int* eT = eX + p.zk;
+  DevStatus* st = c.at<DevStatus>(p.o_status);
+  for (int t0 = 0; t0 < n; t0 += p.zk) {
+    const int m = std::min(p.zk, n - t0);
+    const int* eU = ue ? ue + t0 : nullptr;
+    for (int a = 0; a < 2; ++a) {
+      const double* D = (a ? Y : X) + (int64_t)t0 * ld;
+      cudaError_t e = launch_maxexp(D, ld, (int)WW, m, eX, c.s);
+      if (e == cudaSuccess)
+        e = launch_zgemm_tc64(ZOp{D, ld, 2, eX}, ZOp{U + t0 * WW, 0, 0, eU}, T, eT, p.W, m, false, false, st, c.s);
+      if (e == cudaSuccess)
+        e = launch_zgemm_tc64(ZOp{U + t0 * WW, 0, 1, eU}, ZOp{T, 0, 0, eT}, V[a], nullptr, p.W, m, true, false, st, c.s);
+      if (e != cudaSuccess) return e;
+    }
+    cudaError_t e = launch_curvature64(E + (int64_t)t0 * p.W, V[0], V[1], p.W, m, c.at<double>(p.o_etas),
+                                       p.n_eta, Om + (int64_t)t0 * p.W, om_stride, c.s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // Steps (3)-(4) from packed Hermitian dH rows X, Y of leading dimension ld; f32 = FP32
 // products.  rows = X and Y are the W*W and 2*W*W column offsets of tensor-core output rows.
 cudaError_t berry_any(const Call& c, const double* E, const double2* U, const double* X,
@@ -647,21 +697,21 @@ cudaError_t berry_any(const Call& c, const double* E, const double2* U, const do
                       int64_t om_stride) {
   const Plan& p = c.p;
   const double* etas = c.at<double>(p.o_etas);
-  if (p.W > SMALL_W_MAX) {
-    const size_t WW = (size_t)p.W * p.W;
-    const size_t es = f32 ? sizeof(float2) : sizeof(double2);
-    char* L = c.at<char>(p.o_L);
-    const size_t cap = (size_t)std::max(1, p.chunk) * WW * es;
-    return launch_berry_large(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, f32, L, L + cap,
-                              L + 2 * cap, c.s);
-  }
   if (!f32) {
     int* ue = p.user_u ? c.at<int>(p.o_ue) : nullptr;
     if (ue) {
       cudaError_t e = launch_unorm(U, p.W, n, ue, c.s);
       if (e != cudaSuccess) return e;
     }
+    if (p.zk > 0) return berry_tc64(c, E, U, ue, X, Y, ld, n, Om, om_stride);
     return launch_berry_fix(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, ue, c.s, p.pad);
+  }
+  if (p.W > SMALL_W_MAX) {
+    const size_t WW = (size_t)p.W * p.W;
+    char* L = c.at<char>(p.o_L);
+    const size_t cap = (size_t)std::max(1, p.chunk) * WW * sizeof(float2);
+    return launch_berry_large(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, L, L + cap,
+                              L + 2 * cap, c.s);
   }
   if (rows) {
     const double* C = X - (size_t)p.W * p.W;   // the row start (H | dxH | dyH)
@@ -979,7 +1029,8 @@ kubo_status setup_ahc(Call& c, const kubo_options& o, const int32_t* R_vecs, int
 // per-k bytes of the reverse-mode buffers (for the automatic batch size)
 size_t grad_bytes_per_k(int W, int N_R) {
   const size_t WW = (size_t)W * W;
-  return 6 * 16 * WW + 8 * (size_t)W + 3 * 8 * WW + 8 * (size_t)N_R;
+  (void)N_R;
+  return 6 * 16 * WW + 8 * (size_t)W + 3 * 8 * WW + 32;
 }
 
 // Body of kubo_ahc_grad (device pointers): per batch the forward steps (1)-(3) in FP64, the
@@ -1013,7 +1064,9 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
   for (int q = 0; q < 6; ++q) bw[q] = c.at<double2>(p.o_gw) + q * cap;
   double* Ebar = c.at<double>(p.o_Ebar);
   double* Mbar = c.at<double>(p.o_Mbar);
-  double* Coef = c.at<double>(p.o_Coef);
+  int* eb_[6];
+  for (int q = 0; q < 6; ++q) eb_[q] = c.at<int>(p.o_ge) + (size_t)q * std::max(1, p.chunk);
+  int* eD = c.at<int>(p.o_ge) + (size_t)6 * std::max(1, p.chunk);
   double* Gacc = c.at<double>(p.o_Gacc);
   const double* etas = c.at<double>(p.o_etas);
   const double inv_Nk = 1.0 / (double)p.mesh.Nk;
@@ -1045,29 +1098,42 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
       KCHECK(launch_ksum_partial(E, Om, p.W, n, p.n_eta, (int64_t)n * p.W, E_F, p.n_EF, o.kT, part, p.kpb, c.s));
       KCHECK(launch_ksum_fold(part, (n + p.kpb - 1) / p.kpb, n_out, acc, c.s));
     }
-    StageTimer tm(c, KUBO_STAGE_ADJOINT, 17);
+    StageTimer tm(c, KUBO_STAGE_ADJOINT, 25);
+    const int W = p.W;
+    auto mm = [&](ZOp A, ZOp B, double2* C, int* ec, bool accum = false) {
+      return launch_zgemm_tc64(A, B, C, ec, W, n, false, accum, st, c.s);
+    };
+    const ZOp zU{U, 0, 0, nullptr}, zUh{U, 0, 1, nullptr};
+    auto op = [&](int q) { return ZOp{bw[q], 0, 0, eb_[q]}; };
+    auto exps = [&](int q) { return launch_maxexp(reinterpret_cast<const double*>(bw[q]), 2 * (int64_t)WW, (int)(2 * WW), n, eb_[q], c.s); };
     // v^x, v^y (full): b0 = U^H (X U), b1 = U^H (Y U)
-    KCHECK(launch_herm_u(Xp, (int64_t)WW, U, bw[5], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(true, false, false, U, bw[5], bw[0], p.W, n, c.s));
-    KCHECK(launch_herm_u(Yp, (int64_t)WW, U, bw[5], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(true, false, false, U, bw[5], bw[1], p.W, n, c.s));
+    for (int a = 0; a < 2; ++a) {
+      const double* D = a ? Yp : Xp;
+      KCHECK(launch_maxexp(D, (int64_t)WW, (int)WW, n, eD, c.s));
+      KCHECK(mm(ZOp{D, (int64_t)WW, 2, eD}, zU, bw[5], eb_[5]));
+      KCHECK(mm(zUh, op(5), bw[a], eb_[a]));
+    }
     // vbar^x -> b2, vbar^y -> b3, Ebar
-    KCHECK(launch_grad_pairs(E, bw[0], bw[1], p.W, n, g, E_F, p.n_EF, etas, p.n_eta, o.kT, inv_Nk, bw[2], bw[3], Ebar, c.s));
+    KCHECK(launch_grad_pairs(E, bw[0], bw[1], W, n, g, E_F, p.n_EF, etas, p.n_eta, o.kT, inv_Nk, bw[2], bw[3], Ebar, c.s));
+    KCHECK(exps(2));
+    KCHECK(exps(3));
     // N = vbar^x v^x + vbar^y v^y -> b4; Gp -> b0
-    KCHECK(launch_zgemm_batched(false, false, false, bw[2], bw[0], bw[4], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(false, false, true, bw[3], bw[1], bw[4], p.W, n, c.s));
-    KCHECK(launch_grad_gp(E, Ebar, bw[4], p.W, n, o.grad_eps, bw[0], c.s));
+    KCHECK(mm(op(2), op(0), bw[4], nullptr));
+    KCHECK(mm(op(3), op(1), bw[4], nullptr, true));
+    KCHECK(launch_grad_gp(E, Ebar, bw[4], W, n, o.grad_eps, bw[0], c.s));
+    KCHECK(exps(0));
     // Hbar = U Gp U^H -> b1, dxHbar = U vbar^x U^H -> b0, dyHbar = U vbar^y U^H -> b4
-    KCHECK(launch_zgemm_batched(false, false, false, U, bw[0], bw[5], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(false, true, false, bw[5], U, bw[1], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(false, false, false, U, bw[2], bw[5], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(false, true, false, bw[5], U, bw[0], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(false, false, false, U, bw[3], bw[5], p.W, n, c.s));
-    KCHECK(launch_zgemm_batched(false, true, false, bw[5], U, bw[4], p.W, n, c.s));
-    KCHECK(launch_pack3(bw[1], bw[0], bw[4], p.W, n, Mbar, c.s));
+    const int src[3] = {0, 2, 3}, dst[3] = {1, 0, 4};
+    for (int a = 0; a < 3; ++a) {
+      KCHECK(mm(zU, op(src[a]), bw[5], eb_[5]));
+      KCHECK(mm(op(5), ZOp{U, 0, 1, nullptr}, bw[dst[a]], nullptr));
+    }
+    KCHECK(launch_pack3(bw[1], bw[0], bw[4], W, n, Mbar, c.s));
     // transposed Fourier sum of the batch into the G rows
-    KCHECK(launch_grad_coef(md, p.mesh, kl, n, Coef, c.s));
-    KCHECK(launch_grad_fourier_t(Coef, n, Mbar, M, (int)(3 * WW), n, Gacc, c.s));
+    for (int t0 = 0; t0 < n; t0 += p.t_k) {
+      const KList sub{kl.idx ? kl.idx + t0 : nullptr, kl.base + t0, std::min(p.t_k, n - t0)};
+      KCHECK(launch_grad_fourier_t(md, p.mesh, sub, Mbar + (size_t)t0 * 3 * WW, c.at<char>(p.o_tA), c.at<char>(p.o_tB), c.at<int>(p.o_texp), Gacc, st, c.s));
+    }
   }
   r = read_status(c);
   if (r != KUBO_OK) return r;
@@ -1969,14 +2035,14 @@ kubo_status kubo_berry_batched(const double* E, const double* U, const double* d
     Plan& p = c.p;
     p.W = W; p.n_eta = o.n_eta > 0 ? o.n_eta : 1; p.n_EF = 1;
     p.chunk = o.chunk_k > 0 ? o.chunk_k : auto_chunk(W, p.n_eta, n);
-    p.lbuf = W > SMALL_W_MAX;   // the GEMM products of large orders go through the workspace
-    p.user_u = !p.lbuf;
+    p.user_u = true;
     plan_layout(p, false, 0);
     fit_workspace(p, o);
     c.s = (cudaStream_t)o.stream;
     kubo_status r = c.acquire(o);
     if (r != KUBO_OK) return r;
-    r = upload_etas(c, o, eta);
+    if (cudaMemsetAsync(c.at<char>(p.o_status), 0, sizeof(DevStatus), c.s) != cudaSuccess) r = KUBO_ERR_CUDA;
+    if (r == KUBO_OK) r = upload_etas(c, o, eta);
     const size_t WW = (size_t)W * W;
     const int64_t step = p.chunk;
     for (int64_t t0 = 0; t0 < n && r == KUBO_OK; t0 += step) {
@@ -1987,6 +2053,7 @@ kubo_status kubo_berry_batched(const double* E, const double* U, const double* d
         r = KUBO_ERR_CUDA;
       }
     }
+    if (r == KUBO_OK) r = read_status(c);
     c.release();
     if (cudaStreamSynchronize(c.s) != cudaSuccess && r == KUBO_OK) r = KUBO_ERR_CUDA;
     return r;

@@ -298,6 +298,12 @@ cudaError_t launch_coef_split64(const Model& md, const Mesh& mesh, const KList& 
 cudaError_t launch_fourier_tc64(const void* A, const void* Bt, const int* col_exp, int Mpad,
                                 int Npad, int Kp, int n_rows, int W, double* Hp, double* Xp,
                                 double* Yp, DevStatus* st, cudaStream_t s);
+// transposed sum of the gradient: Gacc [1 + 2 N_h][3 W^2] += Coef^T Mbar over the k-points of kl, Mbar
+// [n][3 W^2].  Operands A 2 slices tc_pad_m(1 + 2 N_h) tc_pad_k(n) bytes, Bt 2 slices tc64_pad_n(W)
+// tc_pad_k(n), col_exp tc64_pad_n(W) ints.
+cudaError_t launch_grad_fourier_t(const Model& md, const Mesh& mesh, const KList& kl, const double* Mbar,
+                                  void* A, void* Bt, int* col_exp, double* Gacc, DevStatus* st,
+                                  cudaStream_t s);
 // the tensor-core kernel's bounded mbarrier wait on a barrier that never completes
 cudaError_t launch_bounded_wait_check(uint32_t limit, DevStatus* st, cudaStream_t s);
 // rows [n][ld] (H | dxH | dyH packed) -> three packed arrays [n][W*W]
@@ -335,6 +341,27 @@ cudaError_t launch_berry_fix(const double* E, const double2* U, const double* Xp
 cudaError_t launch_reflect_fix(int W, int n, EighBufs b, const double* Z, double2* U, cudaStream_t s,
                                int pad = 1);
 
+// FP64-grade batched complex products on the tensor cores, W <= 128 (k_zgemm_tc64.cu):
+// C[k] = op(A[k]) op(B[k]) (+ C[k]).  kind 0: complex [n][W][W]; 1: its conjugate transpose; 2 (A
+// only): Hermitian, packed real rows of leading dimension ld.  e[k]: every part of matrix k is below
+// 2^e[k] in magnitude (ZEXP_BAD: infinite or NaN entries, the product is NaN); null: 0.
+// ec (may be null): the same for C.  upper: tiles strictly below the diagonal are not written.
+constexpr int ZEXP_BAD = 1 << 20;
+struct ZOp {
+  const void* p;
+  int64_t ld;
+  int kind;
+  const int* e;
+};
+cudaError_t launch_zgemm_tc64(const ZOp& A, const ZOp& B, double2* C, int* ec, int W, int n, bool upper,
+                              bool accum, DevStatus* st, cudaStream_t s);
+// e[k] of the len doubles at x + k ld
+cudaError_t launch_maxexp(const double* x, int64_t ld, int len, int n, int* e, cudaStream_t s);
+// Omega from the upper triangles of v^x and v^y ([n][W][W])
+cudaError_t launch_curvature64(const double* E, const double2* Vx, const double2* Vy, int W, int n,
+                               const double* etas, int n_eta, double* Om, int64_t eta_stride,
+                               cudaStream_t s);
+
 // k_large.cu: sorted eigenvalues E and eigenvectors Z of T by inverse iteration ([n][W][W]
 // real, column m for sorted eigenvalue m; Z may be null: eigenvalues only), any W <= 128,
 // at most `slots` persistent CTAs (iit_max_slots(W) fill the GPU) with
@@ -354,12 +381,11 @@ cudaError_t launch_reflect_large(int W, int n, EighBufs b, const double* Z, void
 size_t reflect_wy_scratch_bytes(int W);
 cudaError_t launch_reflect_wy(int W, int n, EighBufs b, const double* Z, float2* U, float2* wy,
                               cudaStream_t s);
-// steps (3)-(4) as batched complex GEMMs: X, Y packed Hermitian rows of leading dimension ld;
-// f32 = FP32 products.  Tbuf, Vx, Vy: n * W * W complex elements (of the product type) each.
+// steps (3)-(4) of the FP32-rotation modes as batched complex GEMMs: X, Y packed Hermitian rows of
+// leading dimension ld, U float2.  Tbuf, Vx, Vy: n * W * W float2 each.
 cudaError_t launch_berry_large(const double* E, const void* U, const double* X, const double* Y,
                                int64_t ld, int W, int n, const double* etas, int n_eta, double* Om,
-                               int64_t eta_stride, bool f32, void* Tbuf, void* Vx, void* Vy,
-                               cudaStream_t s);
+                               int64_t eta_stride, void* Tbuf, void* Vx, void* Vy, cudaStream_t s);
 
 // separable Fourier sum (k_fourier_sep.cu).  box: [2h1+1][2h2+1][2h3+1] index of (R1, R2, R3)
 // in the R list or -1.  Stage A once per call into A (sep_a_elems complex); per batch the
@@ -376,13 +402,7 @@ cudaError_t launch_sep_batch(const double2* A, const SepBox& sb, int W, const Me
                              int j1a, int np1, double2* B, double2* By, double* Hp, double* Xp,
                              double* Yp, cudaStream_t s);
 
-// T = X U with X packed Hermitian rows (leading dimension ld), FP64
-cudaError_t launch_herm_u(const double* X, int64_t ld, const double2* U, double2* T, int W, int n,
-                          cudaStream_t s);
-
 // reverse mode (k_grad.cu)
-cudaError_t launch_zgemm_batched(bool hA, bool hB, bool acc, const double2* A, const double2* B,
-                                 double2* C, int W, int n, cudaStream_t s);
 cudaError_t launch_grad_pairs(const double* E, const double2* vx, const double2* vy, int W, int n,
                               const double* g, const double* E_F, int n_EF, const double* etas,
                               int n_eta, double kT, double inv_Nk, double2* vbx, double2* vby,
@@ -391,10 +411,6 @@ cudaError_t launch_grad_gp(const double* E, const double* Ebar, const double2* N
                            double grad_eps, double2* Gp, cudaStream_t s);
 cudaError_t launch_pack3(const double2* A0, const double2* A1, const double2* A2, int W, int n,
                          double* out, cudaStream_t s);
-cudaError_t launch_grad_coef(const Model& md, const Mesh& mesh, const KList& kl, int ldc,
-                             double* Coef, cudaStream_t s);
-cudaError_t launch_grad_fourier_t(const double* Coef, int ldc, const double* Mbar, int M, int N,
-                                  int K, double* Gacc, cudaStream_t s);
 cudaError_t launch_grad_finalize(const double* Gacc, const int* pairs, const int* Rh, int idx0,
                                  int N_h, int W, double2* G, cudaStream_t s);
 

@@ -1,6 +1,7 @@
 """Integer-pipe products of FP64 grade (rotations, U = Q D Z) against extended precision.
 
-Orders around the tiles (2 x 2 below 13, 4 x 2 from there; 4 reflectors per block), magnitudes far from
+Orders around the tiles (2 x 2 below 13, 4 x 2 to 32, tensor-core tiles of up to 64 above; 4 reflectors
+per block), magnitudes far from
 1, eigenvectors that are not normalised, non-finite operands.
 """
 import numpy as np
@@ -33,7 +34,7 @@ def _curvature(E, vx, vy, eta):
     return T.sum(2), size
 
 
-@pytest.mark.parametrize("W", [1, 2, 3, 4, 5, 11, 12, 13, 16, 31, 33, 48, 63, 64])
+@pytest.mark.parametrize("W", [1, 2, 3, 4, 5, 11, 12, 13, 16, 24, 25, 32, 33, 48, 63, 64, 65, 97, 128])
 @pytest.mark.parametrize("sx,sy,su", [(1.0, 1.0, 1.0), (2.0 ** 130, 2.0 ** -90, 1.0), (1.0, 1.0, 3.0)])
 def test_curvature(W, sx, sy, su):
     import torch
