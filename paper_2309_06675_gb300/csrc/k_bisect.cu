@@ -79,7 +79,7 @@ __device__ __forceinline__ int count64(const double2* t2, int W, double x) {
   return c;
 }
 
-__global__ void __launch_bounds__(BT) bisect_kernel(int W, int n, int kpc, EighBufs b, DevStatus* st) {
+__global__ void __launch_bounds__(BT) bisect_kernel(int W, int n, int kpc, EighBufs b) {
   extern __shared__ __align__(16) unsigned char bsm[];
   float4* t4 = reinterpret_cast<float4*>(bsm);                                  // [kpc][W]
   double2* t2 = reinterpret_cast<double2*>(t4 + (size_t)kpc * W);               // [kpc][W]
@@ -153,19 +153,19 @@ __global__ void __launch_bounds__(BT) bisect_kernel(int W, int n, int kpc, EighB
       }
       lam = 0.5 * (lo + hi);
     }
+    // an infinite or NaN entry: NaN for every eigenvalue of the matrix
     b.lam[k * W + j] = bad ? __longlong_as_double(0x7FF8000000000000ll) : fx::scale_pow2(lam, ex);
-    if (bad && j == 0) atomicOr(&st->bits, ST_NO_CONVERGENCE);   // as a QL iteration that never deflates
   }
 }
 
 }  // namespace
 
-cudaError_t launch_bisect(int W, int n, EighBufs b, DevStatus* st, cudaStream_t s) {
+cudaError_t launch_bisect(int W, int n, EighBufs b, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (W < 1 || W > BT) return cudaErrorInvalidValue;
   const int kpc = BT / W;
   const size_t sm = (size_t)kpc * W * (sizeof(float4) + sizeof(double2) + sizeof(double)) + kpc * sizeof(unsigned);
-  bisect_kernel<<<(n + kpc - 1) / kpc, BT, sm, s>>>(W, n, kpc, b, st);
+  bisect_kernel<<<(n + kpc - 1) / kpc, BT, sm, s>>>(W, n, kpc, b);
   return cudaGetLastError();
 }
 

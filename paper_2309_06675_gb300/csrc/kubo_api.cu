@@ -25,6 +25,9 @@ constexpr int FIX_W_MAX = 32;
 // k-points per sub-batch of the latter: T, v^x and v^y of a sub-batch (192 KB each at W = 64) are
 // written and read while they are in L2
 constexpr int ZG_BATCH = 152 * 8;
+// Shifts by bisection (a lane per eigenvalue) instead of the QL iteration (a lane per k-point) from
+// this order
+constexpr int BISECT_W_MIN = 9;
 constexpr int KSUM_KPB = 32;         // k-points per deterministic k-sum block (at least)
 constexpr size_t KSUM_PART_BYTES = (size_t)256 << 20;   // cap on the per-block partials
 // mixed precision: share of each batch (largest ||Omega(k)||_inf) redone in FP64
@@ -162,6 +165,7 @@ struct Plan {
   bool iit = false;     // inverse-iteration scratch (separate eigenvector kernel)
   int zk = 0;           // k-points per sub-batch of the tensor-core rotations (FP64, W > FIX_W_MAX)
   bool lean = false;    // a caller's workspace too small for Z, the iteration scratch and zg (W <= 64)
+  bool bisect = false;  // FP64 with eigenvectors: shifts by bisection, eigenvalues as Rayleigh quotients
   bool user_u = false;  // eigenvectors from the caller (kubo_berry_batched): column norms on the device
   int iit_slots = 0;
   // separable Fourier sum: bounding box, pairs per batch, planes of the range
@@ -314,6 +318,8 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
   // column norms of the caller's U (up to 48 of them in the unused part of the broadenings' block)
   if (p.user_u) p.o_ue = p.chunk <= 48 ? p.o_etas + sizeof(double) * MAX_ETA : b.take(sizeof(int) * (size_t)p.chunk);
   p.iit = p.eigh && !p.lean;
+  // (a cap on the QL sweeps asks for the QL iteration)
+  p.bisect = p.iit && p.precision == KUBO_FP64 && p.ql_cap == 0 && p.W >= BISECT_W_MIN;
   if (p.iit) {
     p.iit_slots = iit_slots_for(p.W, std::max(1, p.chunk));
     p.o_iit = b.take(sizeof(double) * iit_scratch_doubles(p.W, p.iit_slots));
@@ -634,6 +640,12 @@ cudaError_t fourier64(const Call& c, const Model& md, const KList& kl, double* H
   return cudaSuccess;
 }
 
+// Eigenvalues of T, or shifts near them where the eigenvectors are wanted and the Rayleigh quotients
+// will be reported, into eb.lam.
+cudaError_t eigh_shifts(const Call& c, int n, const EighBufs& eb, DevStatus* st, bool vectors = true) {
+  return c.p.bisect && vectors ? launch_bisect(c.p.W, n, eb, c.s) : launch_ql(c.p.W, n, eb, st, c.s);
+}
+
 // Eigenvalues (sorted) and eigenvectors U = Q D Z of n tridiagonalised matrices whose
 // eigenvalues QL left in eb.lam (U may be null: eigenvalues only).  f32u (W > 64 only): U is
 // formed in FP32 (float2) for the FP32 rotations, its only consumer in that mode.  rq (W > 64
@@ -644,13 +656,13 @@ cudaError_t eigh_vectors(const Call& c, int n, const EighBufs& eb, double* E, do
   if (p.W <= SMALL_W_MAX) {
     if (p.lean) return launch_backtransform(p.W, n, eb, E, U, c.s, p.pad);
     double* Z = U ? c.at<double>(p.o_Z) : nullptr;
-    cudaError_t e = launch_iit(p.W, n, eb, E, Z, c.at<double>(p.o_iit), p.iit_slots, c.s);
+    cudaError_t e = launch_iit(p.W, n, eb, E, Z, c.at<double>(p.o_iit), p.iit_slots, c.s, p.bisect);
     return e != cudaSuccess || !U ? e : launch_reflect_fix(p.W, n, eb, Z, U, c.s, p.pad);
   }
   double* Z = U ? c.at<double>(p.o_L) : nullptr;
   cudaError_t e = Z && df_eigh(p.precision)
                       ? launch_iit_df(p.W, n, eb, E, Z, c.at<double>(p.o_iit), p.iit_slots, c.s)
-                      : launch_iit(p.W, n, eb, E, Z, c.at<double>(p.o_iit), p.iit_slots, c.s, rq);
+                      : launch_iit(p.W, n, eb, E, Z, c.at<double>(p.o_iit), p.iit_slots, c.s, rq || p.bisect);
   if (e != cudaSuccess || !U) return e;
   if (f32u) {
     // the blocked WY factors in the large region after Z (16-byte aligned, within its size)
@@ -819,7 +831,7 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
   }
   {
     StageTimer tm(c, KUBO_STAGE_QL, 1);
-    KCHECK(launch_ql(p.W, kl.n, eb, st, c.s));
+    KCHECK(eigh_shifts(c, kl.n, eb, st));
   }
   if (f32_rotation(p.precision) && p.W <= SMALL_W_MAX) {
     double* Z = reinterpret_cast<double*>(U);
@@ -1083,7 +1095,7 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
     }
     {
       StageTimer tm(c, KUBO_STAGE_QL, 1);
-      KCHECK(launch_ql(p.W, n, eb, st, c.s));
+      KCHECK(eigh_shifts(c, n, eb, st));
     }
     {
       StageTimer tm(c, KUBO_STAGE_BACKTRANSFORM, 2);
@@ -2005,7 +2017,7 @@ kubo_status kubo_eigh_batched(const double* A, int W, int64_t n, double* E, doub
     for (int64_t t0 = 0; t0 < n && r == KUBO_OK; t0 += p.chunk) {
       int nn = (int)std::min<int64_t>(p.chunk, n - t0);
       if (launch_tridiag(A + t0 * WW, W, nn, eb, c.s) != cudaSuccess ||
-          launch_ql(W, nn, eb, st, c.s) != cudaSuccess ||
+          eigh_shifts(c, nn, eb, st, U != nullptr) != cudaSuccess ||
           eigh_vectors(c, nn, eb, E + t0 * W, U ? (double2*)U + t0 * WW : nullptr) != cudaSuccess) {
         cudaGetLastError();
         r = KUBO_ERR_CUDA;

@@ -205,6 +205,8 @@ cudaError_t launch_tridiag_rows(const double* Hp, int64_t ld, int W, int n, Eigh
 cudaError_t launch_tridiag_df_rows(const double* Hp, int64_t ld, int W, int n, EighBufs b,
                                    cudaStream_t s);
 cudaError_t launch_ql(int W, int n, EighBufs b, DevStatus* st, cudaStream_t s);
+// shifts by bisection, a lane per eigenvalue: within 2^-45 ||T|| (2^-53 inside groups closer than 2^-13)
+cudaError_t launch_bisect(int W, int n, EighBufs b, cudaStream_t s);
 // the same QL iteration in double-float (MIXED mode; FP64 eigenvalues out)
 cudaError_t launch_ql_df(int W, int n, EighBufs b, DevStatus* st, cudaStream_t s);
 // eigenvectors of T by inverse iteration in double-float (MIXED mode; same layout, scratch and

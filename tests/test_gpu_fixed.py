@@ -82,3 +82,55 @@ def test_eigenvectors(W):
     orth = np.abs(U.conj().transpose(0, 2, 1).astype(L) @ U.astype(L) - np.eye(W))
     # a W-step reduction at 2^-52 of the norm per step and entry
     assert res.max() <= 4 * W * 2.0 ** -52 and orth.max() <= 4 * W * 2.0 ** -52, (res.max(), orth.max())
+
+
+def _structured(kind, W, n, rng):
+    """Matrices whose spectra are hard for shifts: exact and near multiples, splits, one scale apart."""
+    z = rng.standard_normal((n, W, W)) + 1j * rng.standard_normal((n, W, W))
+    Q = np.linalg.qr(z)[0]
+    lam = rng.standard_normal((n, W))
+    if kind == "pairs":
+        lam[:, 1::2] = lam[:, : 2 * (W // 2): 2]
+    elif kind == "close":
+        lam[:, 1::2] = lam[:, : 2 * (W // 2): 2] + 10.0 ** rng.uniform(-15, -4, (n, W // 2))
+    elif kind == "one":
+        lam[:] = 0.75
+    elif kind == "graded":
+        lam *= 2.0 ** -np.linspace(0, 40, W)
+    A = (Q * lam[:, None, :]) @ Q.conj().transpose(0, 2, 1)
+    if kind == "blocks":
+        A[:, : W // 2, W // 2:] = 0
+        A[:, W // 2:, : W // 2] = 0
+    if kind == "diagonal":
+        A = np.stack([np.diag(x) for x in lam]).astype(complex)
+    if kind == "zero":
+        A[:] = 0
+    return (A + A.conj().transpose(0, 2, 1)) / 2
+
+
+@pytest.mark.parametrize("W", [9, 10, 33, 64, 65, 128])
+@pytest.mark.parametrize("kind", ["pairs", "close", "one", "graded", "blocks", "diagonal", "zero"])
+def test_eigensystem_of_structured_matrices(W, kind):
+    import torch
+    import paper_2309_06675_gb300 as kubo
+    A = _structured(kind, W, 5, np.random.default_rng(W))
+    E, U = kubo.eigh_batched(kubo.pack_hermitian(torch.from_numpy(A).cuda()), W)
+    E, U = E.cpu().numpy(), U.cpu().numpy()
+    ref = np.linalg.eigvalsh(A)
+    norm = max(np.abs(ref).max(), 1e-300)
+    assert (np.diff(E, axis=1) >= 0).all()
+    assert np.abs(E - ref).max() <= 4 * W * 2.0 ** -52 * norm
+    assert np.abs(A @ U - U * E[:, None, :]).max() <= 8 * W * 2.0 ** -52 * norm
+    assert np.abs(U.conj().transpose(0, 2, 1) @ U - np.eye(W)).max() <= 8 * W * 2.0 ** -52
+
+
+def test_non_finite_matrix_leaves_the_others():
+    import torch
+    import paper_2309_06675_gb300 as kubo
+    A = _structured("pairs", 20, 3, np.random.default_rng(0))
+    P = kubo.pack_hermitian(torch.from_numpy(A).cuda())
+    P[1, 5] = float("nan")
+    E = kubo.eigh_batched(P, 20)[0].cpu().numpy()
+    ref = np.linalg.eigvalsh(A)
+    assert np.isnan(E[1]).all()
+    assert np.abs(E[[0, 2]] - ref[[0, 2]]).max() <= 80 * 2.0 ** -52 * np.abs(ref).max()
