@@ -1,0 +1,358 @@
+// Householder reduction H = Q D T D^dagger Q^dagger in FP64 grade on the integer pipe (fixed.cuh), for
+// the FP64 mode (the mixed modes' reduction stays the FP64 one of k_eigh.cu).
+//
+// The FP64 reduction runs at 92 % of the FP64 pipe (8 multiply-adds of 16 clocks per warp
+// for each trailing element and column).  Here the trailing matrix is held as 59-bit fixed-point
+// numbers relative to a power of two above its Frobenius norm, which the reduction's unitary
+// similarities never exceed; its symmetric product and its rank-2 update are sums of fixed-point
+// products.  A rounding is 2^-60 of that norm, at most 2^-57 of the spectral norm at W = 64, where an
+// FP64 update rounds every entry to 2^-54 of itself several times.  Only what one warp does per
+// column (the column's norm, the Householder vector's scale) is FP64.
+//
+// KP k-points per CTA, TPK threads each (2 x 128 at W <= 64, 4 x 64 at 32, 8 x 32 at 16, 16 x 16 at 8,
+// 1 x 512 above 64); warp 0 runs the scalar steps of all KP k-points at once, 32 / KP lanes each.
+// Per column i with reflector I - 2 w w^dagger (w a unit vector, kept in column i of A):
+//   1 (warp 0)  |x|, w = v / |v|, v = x + e^{i arg x_0} |x| e_0
+//   2 (all)     partial sums of p = A w
+//   3 (warp 0)  p, K = w^dagger p, h = p - K w
+//   4 (all)     A <- A - 2 (w h^dagger + h w^dagger), lower triangle
+// What bounds it: the integer multiply-adds (12 per complex product) and, for short columns, the
+// latency of steps 1 and 3, which the other CTAs of the SM fill.
+#include <algorithm>
+
+#include "fixed.cuh"
+#include "kubo_internal.cuh"
+
+namespace kubo {
+
+namespace {
+
+__device__ __forceinline__ int tri(int r, int c) { return (r * (r + 1) >> 1) + c; }
+
+__host__ __device__ constexpr int sp_len(int W, int TPK) { return TPK > 2 * W ? TPK : 2 * W; }
+__host__ __device__ constexpr size_t fix_bytes_per_k(int W, int TPK) {
+  return ((size_t)W * (W + 1) / 2 + sp_len(W, TPK) + W) * 16;
+}
+
+template <int KP, int TPK, int MINB>
+__global__ void __launch_bounds__(KP* TPK, MINB)
+    tridiag_fix_kernel(const double* __restrict__ Hp, int64_t ld, int W, int n, EighBufs b) {
+  constexpr int LPK = 32 / KP;   // warp 0's lanes per k-point; four rows each cover W
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int g = t / TPK, th = t - g * TPK;
+  const int NA = W * (W + 1) / 2, SP = sp_len(W, TPK);
+  const size_t per_k = (size_t)NA + SP + W;
+  int4* base = reinterpret_cast<int4*>(smraw);
+  int4* A = base + g * per_k;                                       // lower triangle, packed by rows
+  longlong2* sp = reinterpret_cast<longlong2*>(A + NA);             // partial sums; then h | w as limbs
+  unsigned char* rowtab = smraw + KP * per_k * 16;                  // row of a strictly lower element
+  __shared__ unsigned long long s_sq[KP];
+  __shared__ unsigned s_max[KP];
+  __shared__ int s_act[KP];
+  const int64_t k = (int64_t)blockIdx.x * KP + g;
+  const bool live = k < n;
+
+  if (t < KP) { s_sq[t] = 0ull; s_max[t] = 0u; }
+  for (int r = 1 + warp; r < W; r += KP * TPK / 32)
+    for (int c = lane; c < r; c += 32) rowtab[r * (r - 1) / 2 + c] = (unsigned char)r;
+  __syncthreads();
+  // ---- load, scale: 2^e above the Frobenius norm (|entry| < (m + 1) 2^(emax - 1037), m its 15 leading
+  // bits at the largest exponent)
+  {
+    double2* Ad = reinterpret_cast<double2*>(A);
+    const double* P = Hp + (live ? k : 0) * ld;
+    unsigned mx = 0u;
+    if (live)
+      for (int idx = th; idx < NA; idx += TPK) {
+        int r = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+        while (tri(r, 0) > idx) --r;
+        while (tri(r + 1, 0) <= idx) ++r;
+        const int c = idx - tri(r, 0);
+        const double2 a = r == c ? make_double2(P[r * W + r], 0.0) : make_double2(P[c * W + r], -P[r * W + c]);
+        Ad[idx] = a;
+        mx = max(mx, (unsigned)(max(mag_bits(a.x), mag_bits(a.y)) >> 32));
+      }
+    if (mx) atomicMax(&s_max[g], mx);
+    __syncthreads();
+    const int emax = (int)(s_max[g] >> 20);
+    unsigned long long s = 0ull;
+    if (live)
+      for (int idx = th; idx < NA; idx += TPK) {
+        const double2 a = Ad[idx];
+        const unsigned hx = (unsigned)(mag_bits(a.x) >> 32), hy = (unsigned)(mag_bits(a.y) >> 32);
+        const int sx = emax - (int)(hx >> 20), sy = emax - (int)(hy >> 20);
+        const unsigned m = (hx && sx < 15 ? (((hx & 0xFFFFFu) | 0x100000u) >> 6) >> sx : 0u) + 1u;
+        const unsigned l = (hy && sy < 15 ? (((hy & 0xFFFFFu) | 0x100000u) >> 6) >> sy : 0u) + 1u;
+        s += 2ull * ((hx ? m * m : 0u) + (unsigned long long)(hy ? l * l : 0u));   // (diagonal: twice its share)
+      }
+    if (s) atomicAdd(&s_sq[g], s);
+    __syncthreads();
+  }
+  const int emax = (int)(s_max[g] >> 20);
+  const bool bad = emax == 0x7FF;
+  const unsigned long long s2all = s_sq[g];
+  const int e = bad || s2all == 0ull ? 0 : emax - 1037 + ((64 - __clzll((long long)s2all) + 1) >> 1);
+  if (live) {
+    const double2* Ad = reinterpret_cast<const double2*>(A);
+    for (int idx = th; idx < NA; idx += TPK) {
+      const double2 a = Ad[idx];
+      A[idx] = bad ? make_int4(0, 0, 0, 0)
+                   : fx::climbs(fx::from_double(a.x, fx::BITS - e), fx::from_double(a.y, fx::BITS - e));
+    }
+  }
+  __syncthreads();
+
+  // warp 0's k-point
+  const int kk = lane / LPK, l = lane - kk * LPK;
+  int4* Ak = base + kk * per_k;
+  longlong2* spk = reinterpret_cast<longlong2*>(Ak + NA);
+  double2* betak = reinterpret_cast<double2*>(spk + SP);   // beta_i, in units of 2^(e - 59)
+  const int64_t kw = (int64_t)blockIdx.x * KP + kk;
+  const bool livek = kw < n;
+
+  for (int i = 0; i < W - 2; ++i) {
+    const int o = i + 1;       // first row of the trailing block
+    const int m = W - 1 - i;   // its size
+    if (warp == 0) {
+      double xr[4], xi[4];
+      double s2 = 0.0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = l + LPK * q;
+        xr[q] = xi[q] = 0.0;
+        if (r < m && livek) {
+          const int4 a = Ak[tri(o + r, i)];
+          xr[q] = (double)fx::value(a.x, a.y);
+          xi[q] = (double)fx::value(a.z, a.w);
+          if (r > 0) s2 = fma(xr[q], xr[q], fma(xi[q], xi[q], s2));
+        }
+      }
+#pragma unroll
+      for (int f = LPK / 2; f > 0; f >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, f);
+      const double ax = __shfl_sync(0xffffffffu, xr[0], kk * LPK), ay = __shfl_sync(0xffffffffu, xi[0], kk * LPK);
+      // |x| in the even lanes, |x_0| in the odd ones: one reciprocal square root
+      const double aa2 = fma(ax, ax, ay * ay);
+      const double arg = (l & 1) ? aa2 : aa2 + s2;
+      const double ri = mag_bits(arg) != 0ull ? rsqrt(arg) : 0.0;
+      const double root = arg * ri;
+      const double nrm = __shfl_sync(0xffffffffu, root, kk * LPK);
+      const double aa = __shfl_sync(0xffffffffu, root, kk * LPK + 1);
+      const double ra = __shfl_sync(0xffffffffu, ri, kk * LPK + 1);
+      const bool az = mag_bits(aa2) == 0ull;
+      const double px = az ? 1.0 : ax * ra, py = az ? 0.0 : ay * ra;   // the unit phase of x_0
+      const bool act = mag_bits(s2) != 0ull;
+      if (act) {
+        // v = (ph (|x| + |x_0|), x_1, ...), |v|^2 = 2 |x| (|x| + |x_0|)
+        const double tt = nrm + aa;
+        const double f = rsqrt(2.0 * nrm * tt);
+        if (l == 0) {
+          xr[0] = px * tt;
+          xi[0] = py * tt;
+          betak[i] = make_double2(-px * nrm, -py * nrm);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int r = l + LPK * q;
+          if (r < m)
+            Ak[tri(o + r, i)] = fx::climbs(fx::from_double(xr[q] * f, 58), fx::from_double(xi[q] * f, 58));
+        }
+      } else if (l == 0 && livek) {
+        betak[i] = make_double2(ax, ay);   // no reflection
+      }
+      if (l == 0) {
+        s_act[kk] = act ? 1 : 0;
+        if (livek) b.tau[kw * W + i] = act ? 2.0 : 0.0;
+      }
+    }
+    __syncthreads();
+    const bool act = s_act[g] != 0;
+    const int P = max(1, min(TPK / m, 8));   // column partitions of a row
+    if (act) {
+      const int part = th / m, r = th - part * m;
+      if (part < P) {
+        fx::Acc acc;
+        fx::zero(acc);
+        const int rowb = tri(o + r, o);
+        for (int c = part; c < m; c += P) {
+          const bool up = c > r;   // mirrored: the conjugate of (c, r)
+          const int4 a = A[up ? tri(o + c, o + r) : rowb + c];
+          const int4 w = A[tri(o + c, i)];
+          const int nz = -a.z, nw = -a.w;
+          const int4 as = make_int4(a.x, a.y, up ? nz : a.z, up ? nw : a.w);
+          fx::cmad(acc, as, up ? a.z : nz, up ? a.w : nw, w);
+        }
+        sp[part * m + r] = make_longlong2(fx::fold(acc.rh, acc.rm), fx::fold(acc.ih, acc.im));
+      }
+    }
+    __syncthreads();
+    if (warp == 0 && s_act[kk]) {
+      // (a k-point's lanes take this together; the shuffles stay inside its group)
+      const unsigned gm = (LPK == 32 ? 0xffffffffu : ((1u << (LPK & 31)) - 1u)) << (kk * LPK);
+      long long pr[4], pi[4];
+      int4 w[4];
+      long long ks = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = l + LPK * q;
+        pr[q] = pi[q] = 0;
+        w[q] = make_int4(0, 0, 0, 0);
+        if (r < m) {
+          long long sx = 0, sy = 0;
+          for (int p = 0; p < P; ++p) {
+            const longlong2 v = spk[p * m + r];
+            sx += v.x;
+            sy += v.y;
+          }
+          pr[q] = fx::rshift(sx, 2);
+          pi[q] = fx::rshift(sy, 2);
+          w[q] = Ak[tri(o + r, i)];
+          const int4 p4 = fx::climbs(pr[q], pi[q]);
+          long long h = 0, c = 0;   // Re(conj(w) p)
+          fx::mad(h, w[q].x, p4.x); fx::mad(c, w[q].x, p4.y); fx::mad(c, w[q].y, p4.x);
+          fx::mad(h, w[q].z, p4.z); fx::mad(c, w[q].z, p4.w); fx::mad(c, w[q].w, p4.z);
+          ks += fx::fold(h, c);
+        }
+      }
+#pragma unroll
+      for (int f = LPK / 2; f > 0; f >>= 1) ks += __shfl_xor_sync(gm, ks, f);
+      const int2 K = fx::limbs(fx::rshift(ks, 2));
+      __syncwarp(gm);   // every partial sum of the k-point has been read
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = l + LPK * q;
+        if (r < m) {
+          long long rh = 0, rm = 0, ih = 0, im = 0;
+          fx::mad(rh, K.x, w[q].x); fx::mad(rm, K.x, w[q].y); fx::mad(rm, K.y, w[q].x);
+          fx::mad(ih, K.x, w[q].z); fx::mad(im, K.x, w[q].w); fx::mad(im, K.y, w[q].z);
+          int4* s4 = reinterpret_cast<int4*>(spk);
+          s4[r] = fx::climbs(pr[q] - fx::rshift(fx::fold(rh, rm), 2), pi[q] - fx::rshift(fx::fold(ih, im), 2));
+          s4[W + r] = w[q];
+        }
+      }
+    }
+    __syncthreads();
+    if (act) {
+      const int4* hb = reinterpret_cast<const int4*>(sp);
+      const int4* wb = hb + W;
+      const int nlow = m * (m - 1) / 2;
+      for (int idx = th; idx < nlow; idx += TPK) {
+        const int r = rowtab[idx], c = idx - r * (r - 1) / 2;
+        const int4 hc = hb[c], wr = wb[r], wc = wb[c], hr = hb[r];
+        fx::Acc acc;
+        fx::zero(acc);
+        fx::cmadc(acc, hc, -hc.z, -hc.w, wr);   // w_r conj(h_c) + h_r conj(w_c), units 2^-61
+        fx::cmadc(acc, wc, -wc.z, -wc.w, hr);
+        int4* pa = &A[tri(o + r, o + c)];
+        const int4 a = *pa;
+        *pa = fx::climbs(fx::value(a.x, a.y) - fx::rshift(fx::fold(acc.rh, acc.rm), 1),
+                         fx::value(a.z, a.w) - fx::rshift(fx::fold(acc.ih, acc.im), 1));
+      }
+      for (int r = th; r < m; r += TPK) {
+        const int4 h = hb[r], w = wb[r];
+        long long hh = 0, c = 0;   // Re(w_r conj(h_r)), twice of it
+        fx::mad(hh, h.x, w.x); fx::mad(c, h.x, w.y); fx::mad(c, h.y, w.x);
+        fx::mad(hh, h.z, w.z); fx::mad(c, h.z, w.w); fx::mad(c, h.w, w.z);
+        int4* pa = &A[tri(o + r, o + r)];
+        const int2 x = fx::limbs(fx::value(pa->x, pa->y) - fx::fold(hh, c));
+        *pa = make_int4(x.x, x.y, 0, 0);
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---- outputs
+  const double nan = __longlong_as_double(0x7FF8000000000000ll);
+  if (live) {
+    double* dout = b.d + k * W;
+    for (int j = th; j < W; j += TPK) {
+      const int4 a = A[tri(j, j)];
+      dout[j] = bad ? nan : fx::scale_pow2((double)fx::value(a.x, a.y), e - fx::BITS);
+      if (j >= W - 2) b.tau[k * W + j] = 0.0;
+    }
+    double2* rout = b.refl + (size_t)k * W * W;
+    const FastDiv dW(W);
+    for (int idx = th; idx < W * W; idx += TPK) {
+      const int r = (int)dW.div(idx), c = idx - r * W;
+      double2 v = make_double2(0.0, 0.0);
+      if (r > c && c < W - 2) {
+        const int4 a = A[tri(r, c)];
+        v = make_double2(fx::to_double(fx::value(a.x, a.y), -58), fx::to_double(fx::value(a.z, a.w), -58));
+      }
+      rout[idx] = v;
+    }
+  }
+  if (warp == 0) {
+    // |beta_j|, and the phases D_0 = 1, D_{j+1} = D_j beta_j / |beta_j| as a scan over the k-point's lanes,
+    // lane l with j = 4 l .. 4 l + 3
+    const int emk = (int)(s_max[kk] >> 20);
+    const unsigned long long sqk = s_sq[kk];
+    const bool badk = emk == 0x7FF;
+    const int ek = badk || sqk == 0ull ? 0 : emk - 1037 + ((64 - __clzll((long long)sqk) + 1) >> 1);
+    double2 u[4], pr = make_double2(1.0, 0.0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = 4 * l + q;
+      u[q] = make_double2(1.0, 0.0);
+      if (j + 1 < W && livek) {
+        double2 bj;
+        if (j == W - 2) {
+          const int4 a = Ak[tri(W - 1, W - 2)];
+          bj = make_double2((double)fx::value(a.x, a.y), (double)fx::value(a.z, a.w));
+        } else {
+          bj = betak[j];
+        }
+        const double a2 = fma(bj.x, bj.x, bj.y * bj.y);
+        double a = 0.0;
+        if (mag_bits(a2) != 0ull) {
+          const double ra = rsqrt(a2);
+          a = a2 * ra;
+          u[q] = make_double2(bj.x * ra, bj.y * ra);
+        }
+        b.e[kw * W + j] = badk ? nan : fx::scale_pow2(a, ek - fx::BITS);
+      }
+      pr = cmul(pr, u[q]);
+    }
+    double2 sc = pr;
+#pragma unroll
+    for (int off = 1; off < LPK; off <<= 1) {
+      double2 o2;
+      o2.x = __shfl_up_sync(0xffffffffu, sc.x, off, LPK);
+      o2.y = __shfl_up_sync(0xffffffffu, sc.y, off, LPK);
+      if (l >= off) sc = cmul(o2, sc);
+    }
+    double2 D;
+    D.x = __shfl_up_sync(0xffffffffu, sc.x, 1, LPK);
+    D.y = __shfl_up_sync(0xffffffffu, sc.y, 1, LPK);
+    if (l == 0) D = make_double2(1.0, 0.0);
+    if (livek) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int j = 4 * l + q;
+        if (j < W) b.phase[kw * W + j] = D;
+        D = cmul(D, u[q]);
+      }
+      if (l == 0) b.e[kw * W + W - 1] = 0.0;
+    }
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_tridiag_fix(const double* Hp, int64_t ld, int W, int n, EighBufs b, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  auto go = [&](auto kern, int KP, int TPK) -> cudaError_t {
+    const size_t sm = KP * fix_bytes_per_k(W, TPK) + (size_t)W * (W - 1) / 2;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    kern<<<(n + KP - 1) / KP, KP * TPK, sm, s>>>(Hp, ld, W, n, b);
+    return cudaGetLastError();
+  };
+  if (W <= 8) return go(tridiag_fix_kernel<16, 16, 3>, 16, 16);
+  if (W <= 16) return go(tridiag_fix_kernel<8, 32, 3>, 8, 32);
+  if (W <= 32) return go(tridiag_fix_kernel<4, 64, 3>, 4, 64);
+  if (W <= 64) return go(tridiag_fix_kernel<2, 128, 3>, 2, 128);
+  return go(tridiag_fix_kernel<1, 512, 1>, 1, 512);
+}
+
+}  // namespace kubo

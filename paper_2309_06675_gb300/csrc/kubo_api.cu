@@ -827,7 +827,8 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
   }
   {
     StageTimer tm(c, KUBO_STAGE_TRIDIAG, 1);
-    KCHECK(launch_tridiag(Hp, p.W, kl.n, eb, c.s));
+    KCHECK(p.precision == KUBO_FP64 ? launch_tridiag_fix(Hp, (int64_t)p.W * p.W, p.W, kl.n, eb, c.s)
+                                    : launch_tridiag(Hp, p.W, kl.n, eb, c.s));
   }
   {
     StageTimer tm(c, KUBO_STAGE_QL, 1);
@@ -1091,7 +1092,7 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
     }
     {
       StageTimer tm(c, KUBO_STAGE_TRIDIAG, 1);
-      KCHECK(launch_tridiag(Hp, p.W, n, eb, c.s));
+      KCHECK(launch_tridiag_fix(Hp, (int64_t)WW, p.W, n, eb, c.s));
     }
     {
       StageTimer tm(c, KUBO_STAGE_QL, 1);
@@ -2016,7 +2017,7 @@ kubo_status kubo_eigh_batched(const double* A, int W, int64_t n, double* E, doub
     const size_t WW = (size_t)W * W;
     for (int64_t t0 = 0; t0 < n && r == KUBO_OK; t0 += p.chunk) {
       int nn = (int)std::min<int64_t>(p.chunk, n - t0);
-      if (launch_tridiag(A + t0 * WW, W, nn, eb, c.s) != cudaSuccess ||
+      if (launch_tridiag_fix(A + t0 * WW, (int64_t)WW, W, nn, eb, c.s) != cudaSuccess ||
           eigh_shifts(c, nn, eb, st, U != nullptr) != cudaSuccess ||
           eigh_vectors(c, nn, eb, E + t0 * W, U ? (double2*)U + t0 * WW : nullptr) != cudaSuccess) {
         cudaGetLastError();

@@ -197,6 +197,8 @@ cudaError_t launch_fourier_fp64(const Model& md, const Mesh& mesh, const KList& 
 // pad (fused back-transform and rotation kernels): leading dimension W + pad of the shared-
 // memory matrices; 1 (default) keeps column walks conflict-free, 0 is the padding ablation
 cudaError_t launch_tridiag(const double* Hp, int W, int n, EighBufs b, cudaStream_t s);
+// the FP64 mode's reduction, in FP64 grade on the integer pipe (unit reflectors, tau = 2 or 0)
+cudaError_t launch_tridiag_fix(const double* Hp, int64_t ld, int W, int n, EighBufs b, cudaStream_t s);
 // same reduction reading packed H from rows of leading dimension ld (tensor-core output)
 cudaError_t launch_tridiag_rows(const double* Hp, int64_t ld, int W, int n, EighBufs b,
                                 cudaStream_t s);

@@ -87,7 +87,7 @@ extern "C" kubo_status kubo_eigh_batched_noalloc(const double* A, int W, int64_t
     const size_t WW = (size_t)W * W;
     for (int64_t t0 = 0; t0 < n; t0 += B) {
       const int nn = (int)(n - t0 < B ? n - t0 : B);
-      if (launch_tridiag(A + t0 * WW, W, nn, b, s) != cudaSuccess ||
+      if (launch_tridiag_fix(A + t0 * WW, (int64_t)WW, W, nn, b, s) != cudaSuccess ||
           launch_ql(W, nn, b, st, s) != cudaSuccess ||
           launch_backtransform(W, nn, b, E + t0 * W, U ? (double2*)U + t0 * WW : nullptr, s) !=
               cudaSuccess) {
