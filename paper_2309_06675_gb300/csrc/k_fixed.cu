@@ -1,6 +1,6 @@
-// FP64-grade matrix work of steps (2)-(4) for W <= 64 on the integer pipe (fixed.cuh):
+// FP64-grade matrix work of steps (2)-(4) on the integer pipe (fixed.cuh):
 //
-//   berry_fix_kernel   v^a = U^dagger (d_a H) U for a = x, y and the curvature of Eq. 3
+//   berry_fix_kernel   v^a = U^dagger (d_a H) U for a = x, y and the curvature of Eq. 3 (W <= 64)
 //   reflect_fix_kernel U = Q D Z: the Householder reflectors applied to the eigenvectors of T
 //
 // Both were FP64 kernels at 85-96 % of the FP64 pipe; the products here are sums of 59-bit
@@ -302,7 +302,8 @@ __global__ void __launch_bounds__(256) unorm_kernel(const double2* __restrict__ 
 }
 
 // ------------------------------------------------------------------ U = Q D Z
-// One k-point per CTA: u (W x W limbs, 58 fractional bits) starts as D Z; the unit reflectors
+// One k-point (above W = 64: a third of its columns) per CTA: u (limbs, 58 fractional bits) starts as
+// its columns of D Z; the unit reflectors
 // w_j = v_j sqrt(tau_j / 2), H_j = I - 2 w_j w_j^dagger, are applied four at a time from the last:
 //   s_a = w_a^dagger u,   h_a = s_a - 2 sum_{b > a} (w_a^dagger w_b) h_b,   u -= 2 sum_a w_a h_a,
 // which is H_j0 H_j0+1 H_j0+2 H_j0+3 u with one pass for the four sums and one for the update (a
@@ -315,9 +316,9 @@ __host__ __device__ __forceinline__ int rf_blocks(int W) { return W > 2 ? (W - 2
 
 __global__ void __launch_bounds__(RF_NT, 2)
     reflect_fix_kernel(int W, EighBufs b, const double* __restrict__ Z, double2* __restrict__ Uout,
-                       int LD) {
+                       int CB, int LD) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  int4* su = reinterpret_cast<int4*>(smraw);              // [W][LD]
+  int4* su = reinterpret_cast<int4*>(smraw);              // [W][LD], CB columns
   int4* sw = su + (size_t)W * LD;                         // 2 x [W][RF_NB]: a block's reflectors by rows
   int4* sg = sw + (size_t)2 * W * RF_NB;                  // 2 x [6] w_a^dagger w_b
   int4* sp = sg + 12;                                     // [W] phases
@@ -326,16 +327,17 @@ __global__ void __launch_bounds__(RF_NT, 2)
   const int64_t k = blockIdx.x;
   const double* Zk = Z + (size_t)k * W * W;
   const double2* R = b.refl + (size_t)k * W * W;
-  const FastDiv dW(W);
+  const int cb0 = blockIdx.y * CB, ncol = min(CB, W - cb0);
+  const FastDiv dC(ncol);
   for (int j = t; j < W; j += nt) {
     const double2 p = b.phase[k * W + j];
     sp[j] = fx::climbs(fx::from_double(p.x, 58), fx::from_double(p.y, 58));
     sf[j] = sqrt(0.5 * b.tau[k * W + j]);
   }
   __syncthreads();
-  for (int idx = t; idx < W * W; idx += nt) {
-    const int r = (int)dW.div(idx), c = idx - r * W;
-    const int2 z = fx::limbs(fx::from_double(Zk[idx], 58));
+  for (int idx = t; idx < W * ncol; idx += nt) {
+    const int r = (int)dC.div(idx), c = idx - r * ncol;
+    const int2 z = fx::limbs(fx::from_double(Zk[(size_t)r * W + cb0 + c], 58));
     const int4 p = sp[r];
     long long rh = 0, rm = 0, ih = 0, im = 0;
     fx::mad(rh, p.x, z.x); fx::mad(rm, p.x, z.y); fx::mad(rm, p.y, z.x);
@@ -389,9 +391,9 @@ __global__ void __launch_bounds__(RF_NT, 2)
     const int buf = bk & 1, j0 = bk * RF_NB;
     if (bk > 0) stage(bk - 1, buf ^ 1);
     const int4* w = sw + (size_t)buf * W * RF_NB;
-    for (int c0 = 0; c0 < W; c0 += nt >> 2) {
-      const int c = min(c0 + (t >> 2), W - 1);
-      const bool act = c0 + (t >> 2) < W;
+    for (int c0 = 0; c0 < ncol; c0 += nt >> 2) {
+      const int c = min(c0 + (t >> 2), ncol - 1);
+      const bool act = c0 + (t >> 2) < ncol;
       fx::Acc s[RF_NB];
 #pragma unroll
       for (int a = 0; a < RF_NB; ++a) fx::zero(s[a]);
@@ -449,11 +451,80 @@ __global__ void __launch_bounds__(RF_NT, 2)
     __syncthreads();
   }
   double2* Uk = Uout + (size_t)k * W * W;
-  for (int idx = t; idx < W * W; idx += nt) {
-    const int r = (int)dW.div(idx), c = idx - r * W;
+  for (int idx = t; idx < W * ncol; idx += nt) {
+    const int r = (int)dC.div(idx), c = idx - r * ncol;
     const int4 u = su[r * LD + c];
-    Uk[idx] = make_double2(fx::to_double(fx::value(u.x, u.y), -58), fx::to_double(fx::value(u.z, u.w), -58));
+    Uk[(size_t)r * W + cb0 + c] = make_double2(fx::to_double(fx::value(u.x, u.y), -58), fx::to_double(fx::value(u.z, u.w), -58));
   }
+}
+
+// U = Q D Z for W <= 16: a thread per column of a k-point, its column in registers (limbs), 256 / W
+// k-points per CTA, the reflectors one at a time; no reductions across threads.  (A CTA per k-point
+// keeps 4 W lanes, one warp at W = 6, and pays its barriers for 4 reflectors.)
+template <int WM>
+__global__ void __launch_bounds__(256) reflect_small_kernel(int W, int n, int kpc, EighBufs b,
+                                                            const double* __restrict__ Z,
+                                                            double2* __restrict__ Uout) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  int4* swA = reinterpret_cast<int4*>(smraw);   // [kpc][W][W]: column j = unit reflector w_j
+  const int t = threadIdx.x;
+  const int lk = t / W, c = t - lk * W;
+  const int64_t k = (int64_t)blockIdx.x * kpc + lk;
+  const bool live = lk < kpc && k < n;
+  int4* sw = swA + (size_t)lk * W * W;
+  if (live) {   // thread c stages row c
+    const double2* R = b.refl + (size_t)k * W * W + (size_t)c * W;
+    for (int j = 0; j < W - 2; ++j) {
+      int4 w = make_int4(0, 0, 0, 0);
+      if (c > j) {
+        const double f = sqrt(0.5 * b.tau[k * W + j]);
+        const double2 v = R[j];
+        w = fx::climbs(fx::from_double(v.x * f, 58), fx::from_double(v.y * f, 58));
+      }
+      sw[c * W + j] = w;
+    }
+  }
+  __syncthreads();
+  if (!live) return;
+  int4 u[WM];
+#pragma unroll
+  for (int r = 0; r < WM; ++r) {
+    u[r] = make_int4(0, 0, 0, 0);
+    if (r < W) {
+      const double z = Z[(size_t)k * W * W + (size_t)r * W + c];
+      const double2 p = b.phase[k * W + r];
+      u[r] = fx::climbs(fx::from_double(p.x * z, 58), fx::from_double(p.y * z, 58));
+    }
+  }
+#pragma unroll 1
+  for (int j = W - 3; j >= 0; --j) {
+    fx::Acc s;
+    fx::zero(s);
+#pragma unroll
+    for (int r = 1; r < WM; ++r)
+      if (r < W && r > j) {
+        const int4 w = sw[r * W + j];
+        fx::cmadc(s, w, -w.z, -w.w, u[r]);
+      }
+    // h = w^dagger u (units 2^-60), u -= 2 w h
+    const int4 h = fx::climbs(fx::rshift(fx::fold(s.rh, s.rm), 2), fx::rshift(fx::fold(s.ih, s.im), 2));
+#pragma unroll
+    for (int r = 1; r < WM; ++r)
+      if (r < W && r > j) {
+        const int4 w = sw[r * W + j];
+        fx::Acc d;
+        fx::zero(d);
+        fx::cmad(d, h, -h.z, -h.w, w);
+        u[r] = fx::climbs(fx::value(u[r].x, u[r].y) - fx::rshift(fx::fold(d.rh, d.rm), 1),
+                          fx::value(u[r].z, u[r].w) - fx::rshift(fx::fold(d.ih, d.im), 1));
+      }
+  }
+  double2* Uk = Uout + (size_t)k * W * W;
+#pragma unroll
+  for (int r = 0; r < WM; ++r)
+    if (r < W)
+      Uk[r * W + c] = make_double2(fx::to_double(fx::value(u[r].x, u[r].y), -58),
+                                   fx::to_double(fx::value(u[r].z, u[r].w), -58));
 }
 
 }  // namespace
@@ -496,13 +567,27 @@ cudaError_t launch_berry_fix(const double* E, const double2* U, const double* Xp
 cudaError_t launch_reflect_fix(int W, int n, EighBufs b, const double* Z, double2* U, cudaStream_t s,
                                int pad) {
   if (n <= 0) return cudaSuccess;
-  if (W > 64) return cudaErrorInvalidValue;
-  const int LD = pad ? W | 1 : W;
+  if (W > LARGE_W_MAX) return cudaErrorInvalidValue;
+  if (W <= 16) {
+    const int kpc = 256 / W;
+    const size_t sm = (size_t)kpc * W * W * sizeof(int4);
+    auto go = [&](auto kern) -> cudaError_t {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e != cudaSuccess) return e;
+      kern<<<(n + kpc - 1) / kpc, 256, sm, s>>>(W, n, kpc, b, Z, U);
+      return cudaGetLastError();
+    };
+    return W <= 8 ? go(reflect_small_kernel<8>) : go(reflect_small_kernel<16>);
+  }
+  // all columns up to W = 64; above, an even third of them, so that two CTAs share an SM (90 KB at
+  // W = 128)
+  const int nb = W <= 64 ? 1 : 3, CB = (W + nb - 1) / nb;
+  const int LD = pad ? CB | 1 : CB;
   const size_t sm = ((size_t)W * LD + 2 * (size_t)W * RF_NB + 12 + W) * sizeof(int4) + (size_t)W * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(reflect_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  const int nt = std::min(RF_NT, (4 * W + 31) / 32 * 32);   // four lanes per column
-  reflect_fix_kernel<<<n, nt, sm, s>>>(W, b, Z, U, LD);
+  const int nt = std::min(RF_NT, (4 * CB + 31) / 32 * 32);   // four lanes per column
+  reflect_fix_kernel<<<dim3(n, (W + CB - 1) / CB), nt, sm, s>>>(W, b, Z, U, CB, LD);
   return cudaGetLastError();
 }
 

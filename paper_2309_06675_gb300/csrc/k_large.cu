@@ -4,9 +4,9 @@
 //                         iteration, one thread per cluster, persistent CTAs; LU factors in
 //                         per-CTA global scratch laid out [i][thread] (coalesced), iterates in
 //                         their column of Z (also used for W <= 64 when U is formed in FP32)
-//   reflect_large_kernel  U = Q D Z for one 32-column block of one k-point per CTA
-//   cgemm_herm_u_kernel   T = dH U   (dH from packed Hermitian rows)          } FP64 or FP32
-//   cgemm_uh_t_kernel     V = U^H T                                            } arithmetic
+//   reflect_wy_kernel     U = Q D Z in FP32 by blocked compact-WY products (FP64: k_fixed.cu)
+//   cgemm_herm_u_kernel   T = dH U   (dH from packed Hermitian rows)          } FP32 (FP64:
+//   cgemm_uh_t_kernel     V = U^H T                                            } k_zgemm_tc64.cu)
 //   curvature_large_kernel Omega_n = sum_{m != n} T_nm, every pair evaluated from the upper
 //                         triangle (exact antisymmetry), FP64 energy differences for every
 //                         eta (FP32 quotients for FP32 velocities)
@@ -33,8 +33,10 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
 }
 
 // ------------------------------------------------------------------ inverse iteration
-// Persistent: CTA b handles k = b, b + gridDim.x, ...; block = ldt = W rounded up to a warp;
-// thread j handles the cluster starting at sorted index j.  Z: [n][W][W] real, column m =
+// Persistent: CTA b handles the k-points kpc b .. kpc b + kpc - 1, then kpc gridDim.x further on;
+// kpc = blockDim / W k-points share the CTA (128 threads up to W = 64, W rounded up to a warp above:
+// at W = 6 a CTA of one k-point kept 6 of 32 lanes busy, 147,456 k-points 3.0 ms);
+// thread (k-point lk, j) handles the cluster starting at sorted index j.  Z: [n][W][W] real, column m =
 // eigenvector of sorted eigenvalue m.  scratch: per CTA [4][W][ldt] (reciprocal pivots, U1,
 // U2, multipliers), lane-interleaved so every access of a warp is one coalesced row segment.
 // rq: the eigenvalues written are the FP64 Rayleigh quotients z^T T z of the finished unit
@@ -47,10 +49,13 @@ __global__ void __launch_bounds__(LW_MAX, 8) iit_kernel(int W, int n, EighBufs b
                                                      double* __restrict__ Eout,
                                                      double* __restrict__ Z,
                                                      double* __restrict__ scratch, int rq) {
-  __shared__ double ws[LW_MAX], dd[LW_MAX], ee[LW_MAX];
-  __shared__ int newc[LW_MAX];
-  __shared__ double s_onenrm;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  __shared__ double wsA[LW_MAX], ddA[LW_MAX], eeA[LW_MAX];
+  __shared__ int newcA[LW_MAX];
+  __shared__ unsigned long long s_onenrm[LW_MAX];
+  const int t = threadIdx.x;
+  const int kpc = blockDim.x / W, lk = t / W, j = t - lk * W;
+  double *ws = wsA + lk * W, *dd = ddA + lk * W, *ee = eeA + lk * W;   // (lk < kpc: within LW_MAX)
+  int* newc = newcA + lk * W;
   const int ldt = blockDim.x;
   const size_t plane = (size_t)W * ldt;
   double* rU0 = scratch + (size_t)blockIdx.x * 4 * plane;
@@ -58,40 +63,40 @@ __global__ void __launch_bounds__(LW_MAX, 8) iit_kernel(int W, int n, EighBufs b
   double* U2 = U1 + plane;
   double* ML = U2 + plane;
   const double eps = 2.220446049250313e-16;
-  for (int64_t k = blockIdx.x; k < n; k += gridDim.x) {
-    __syncthreads();   // the previous k-point's shared arrays are no longer read
-    const double* lk = b.lam + k * W;
-    if (t < W) {
-      const double lj = lk[t];
+  for (int64_t kb = (int64_t)blockIdx.x * kpc; kb < n; kb += (int64_t)gridDim.x * kpc) {
+    const int64_t k = kb + lk;
+    const bool live = lk < kpc && k < n;
+    __syncthreads();   // the previous k-points' shared arrays are no longer read
+    if (live) {
+      const double* lam = b.lam + k * W;
+      const double lj = lam[j];
       const unsigned long long kj = order_key(lj);
       int rnk = 0;
       for (int i = 0; i < W; ++i) {
-        const unsigned long long ki = order_key(lk[i]);
-        rnk += (ki < kj) || (ki == kj && i < t);
+        const unsigned long long ki = order_key(lam[i]);
+        rnk += (ki < kj) || (ki == kj && i < j);
       }
       ws[rnk] = lj;
       Eout[k * W + rnk] = lj;
-      dd[t] = b.d[k * W + t];
-      ee[t] = b.e[k * W + t];
+      dd[j] = b.d[k * W + j];
+      ee[j] = b.e[k * W + j];
+      if (j == 0) s_onenrm[lk] = 0ull;
     }
     __syncthreads();
-    if (warp == 0) {
-      double mx = 0.0;
-      for (int i = lane; i < W; i += 32)
-        mx = fmax(mx, fabs(dd[i]) + (i > 0 ? ee[i - 1] : 0.0) + (i < W - 1 ? ee[i] : 0.0));
-      for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (lane == 0) s_onenrm = mx > 0.0 ? mx : 1.0;
+    if (live) {   // ||T||_1: a maximum of non-negative numbers, by their bits (NaN left out)
+      const double v = fmax(0.0, fabs(dd[j]) + (j > 0 ? ee[j - 1] : 0.0) + (j < W - 1 ? ee[j] : 0.0));
+      atomicMax(&s_onenrm[lk], (unsigned long long)__double_as_longlong(v));
     }
     __syncthreads();
-    const double onenrm = s_onenrm;
+    const double mx = live ? __longlong_as_double((long long)s_onenrm[lk]) : 1.0;
+    const double onenrm = mx > 0.0 ? mx : 1.0;
     const double ortol = 1e-3 * onenrm, pertol = 10.0 * eps * onenrm, tiny = eps * onenrm;
-    if (t < W) newc[t] = (t == 0) || (ws[t] - ws[t - 1] > ortol);
+    if (live) newc[j] = (j == 0) || (ws[j] - ws[j - 1] > ortol);
     __syncthreads();
     if (Z == nullptr) continue;
 
     double* Zk = Z + (size_t)k * W * W;
-    const int j = t;
-    if (j < W && newc[j]) {
+    if (live && newc[j]) {
       double lprev = 0.0, rprev = 0.0;
       for (int m = j; m < W && (m == j || !newc[m]); ++m) {
         double lam = ws[m];
@@ -180,99 +185,11 @@ __global__ void __launch_bounds__(LW_MAX, 8) iit_kernel(int W, int n, EighBufs b
   }
 }
 
-// ------------------------------------------------------------------ U = Q D Z, column blocks
-// One CTA per (32-column block, k-point): the block of D Z in shared memory, the reflectors
-// applied from the last to the first (U <- H_j U), eight reflectors at a time staged in shared
-// memory from coalesced row segments of the reflector matrix.
 template <typename T> struct cx;
-template <> struct cx<double> { typedef double2 type; __device__ static double2 make(double a, double b) { return make_double2(a, b); } };
 template <> struct cx<float> { typedef float2 type; __device__ static float2 make(double a, double b) { return make_float2((float)a, (float)b); } };
 
 constexpr int RB_COLS = 32;
 constexpr int RB_NT = 256;   // 8 threads per column
-constexpr int RB_J = 8;      // reflectors per staged block
-
-// T = float: U is formed in FP32 from the FP64 factors, for the FP32 rotations (its only
-// consumer in that mode); T = double: the FP64 eigenvectors.
-template <typename T>
-__global__ void __launch_bounds__(RB_NT) reflect_large_kernel(int W, EighBufs b,
-                                                              const double* __restrict__ Z,
-                                                              typename cx<T>::type* __restrict__ Uout) {
-  typedef typename cx<T>::type C2;
-  extern __shared__ __align__(16) unsigned char rb_smem[];
-  C2* ub = reinterpret_cast<C2*>(rb_smem);   // [W][RB_COLS + 1]
-  __shared__ C2 vs[RB_J][LW_MAX + 1];
-  const int LDB = RB_COLS + 1;
-  const int t = threadIdx.x;
-  const int c0 = blockIdx.y * RB_COLS;
-  const int64_t k = blockIdx.x;
-  const int ncol = min(RB_COLS, W - c0);
-  const double* Zk = Z + (size_t)k * W * W;
-  const double2* ph = b.phase + k * W;
-  for (int idx = t; idx < W * RB_COLS; idx += RB_NT) {
-    const int r = idx / RB_COLS, c = idx % RB_COLS;
-    C2 u = cx<T>::make(0.0, 0.0);
-    if (c < ncol) {
-      const double z = Zk[(size_t)r * W + c0 + c];
-      const double2 p = ph[r];
-      u = cx<T>::make(p.x * z, p.y * z);
-    }
-    ub[r * LDB + c] = u;
-  }
-  const double2* R = b.refl + (size_t)k * W * W;
-  const double* tau = b.tau + k * W;
-  const int c = t >> 3, q = t & 7;
-  const bool act = c < ncol;
-  for (int jhi = W - 3; jhi >= 0; jhi -= RB_J) {
-    const int jlo = max(0, jhi - RB_J + 1);
-    __syncthreads();   // the previous block of reflectors is no longer read
-    for (int idx = t; idx < W * RB_J; idx += RB_NT) {
-      const int r = idx / RB_J, jj = idx % RB_J, j = jlo + jj;
-      if (j <= jhi) {
-        const double2 v = r > j ? R[(size_t)r * W + j] : make_double2(0.0, 0.0);
-        vs[jj][r] = cx<T>::make(v.x, v.y);
-      }
-    }
-    __syncthreads();
-    for (int j = jhi; j >= jlo; --j) {
-      const T tj = (T)tau[j];
-      if (tj == (T)0) continue;
-      const int o = j + 1, m = W - 1 - j;
-      const C2* v = vs[j - jlo] + o;
-      T sx = 0, sy = 0;
-      if (act) {
-        for (int r = q; r < m; r += 8) {
-          const C2 vv = v[r];
-          const C2 u = ub[(o + r) * LDB + c];
-          sx = fma(vv.x, u.x, fma(vv.y, u.y, sx));   // conj(v) u
-          sy = fma(vv.x, u.y, fma(-vv.y, u.x, sy));
-        }
-      }
-#pragma unroll
-      for (int s = 1; s < 8; s <<= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, s);
-        sy += __shfl_xor_sync(0xffffffffu, sy, s);
-      }
-      sx *= tj; sy *= tj;
-      if (act) {
-        for (int r = q; r < m; r += 8) {
-          const C2 vv = v[r];
-          C2 u = ub[(o + r) * LDB + c];
-          u.x = fma(-sx, vv.x, fma(sy, vv.y, u.x));   // u -= s v
-          u.y = fma(-sx, vv.y, fma(-sy, vv.x, u.y));
-          ub[(o + r) * LDB + c] = u;
-        }
-      }
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  C2* Uk = Uout + (size_t)k * W * W;
-  for (int idx = t; idx < W * RB_COLS; idx += RB_NT) {
-    const int r = idx / RB_COLS, cc = idx % RB_COLS;
-    if (cc < ncol) Uk[(size_t)r * W + c0 + cc] = ub[r * LDB + cc];
-  }
-}
 
 // ------------------------------------------------------------------ U = Q D Z in FP32, blocked
 // For the FP32 rotations: Q = H_0 ... H_{W-3} applied in blocks of WY_NB = 8 reflectors in the
@@ -727,26 +644,13 @@ cudaError_t launch_iit(int W, int n, EighBufs b, double* E, double* Z, double* s
                        cudaStream_t s, bool rq) {
   if (n <= 0) return cudaSuccess;
   if (W > LW_MAX || slots < 1) return cudaErrorInvalidValue;
-  const int grid = std::min(n, slots);
-  iit_kernel<<<grid, iit_threads(W), 0, s>>>(W, n, b, E, Z, scratch, (rq && Z) ? 1 : 0);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reflect_large(int W, int n, EighBufs b, const double* Z, void* U, bool f32,
-                                 cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  dim3 grid(n, (W + RB_COLS - 1) / RB_COLS);
-  if (f32) {
-    const size_t sm = (size_t)W * (RB_COLS + 1) * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(reflect_large_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    reflect_large_kernel<float><<<grid, RB_NT, sm, s>>>(W, b, Z, (float2*)U);
-  } else {
-    const size_t sm = (size_t)W * (RB_COLS + 1) * sizeof(double2);
-    cudaError_t e = cudaFuncSetAttribute(reflect_large_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    reflect_large_kernel<double><<<grid, RB_NT, sm, s>>>(W, b, Z, (double2*)U);
-  }
+  // the scratch of `slots` CTAs of iit_threads(W), shared out to CTAs of up to 128 threads that hold
+  // 128 / W k-points each
+  const int total = slots * iit_threads(W);
+  const int bt = W > 64 ? iit_threads(W) : std::min(LW_MAX, total);
+  const int kpc = bt / W;
+  const int grid = std::max(1, std::min((n + kpc - 1) / kpc, total / bt));
+  iit_kernel<<<grid, bt, 0, s>>>(W, n, b, E, Z, scratch, (rq && Z) ? 1 : 0);
   return cudaGetLastError();
 }
 

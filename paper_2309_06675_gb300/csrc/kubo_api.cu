@@ -670,7 +670,7 @@ cudaError_t eigh_vectors(const Call& c, int n, const EighBufs& eb, double* E, do
     float2* wy = reinterpret_cast<float2*>((after_z + 255) & ~(uintptr_t)255);
     return launch_reflect_wy(p.W, n, eb, Z, reinterpret_cast<float2*>(U), wy, c.s);
   }
-  return launch_reflect_large(p.W, n, eb, Z, U, f32u, c.s);
+  return launch_reflect_fix(p.W, n, eb, Z, U, c.s, p.pad);
 }
 
 // FP64 rotations by tensor-core products: T = dH U, v = U^H T (upper tiles), then the curvature.

@@ -335,7 +335,7 @@ cudaError_t launch_fixup_scatter(const int* pos, int cnt, int W, int n_eta, cons
                                  const double* Omfix, int64_t fix_eta_stride, double* E, double* Om,
                                  int64_t eta_stride, cudaStream_t s);
 
-// FP64-grade products on the integer pipe, W <= 64 (k_fixed.cu).  Rotations and curvature from
+// FP64-grade products on the integer pipe (k_fixed.cu).  Rotations and curvature (W <= 64) from
 // packed FP64 dH rows of leading dimension ld; ue: per-matrix exponent of U's column norms (from
 // launch_unorm), null for unit columns.  U = Q D Z from the eigenvectors Z of T.
 cudaError_t launch_unorm(const double2* U, int W, int n, int* ue, cudaStream_t s);
@@ -377,9 +377,6 @@ size_t iit_scratch_doubles(int W, int slots);
 cudaError_t launch_iit(int W, int n, EighBufs b, double* E, double* Z, double* scratch, int slots,
                        cudaStream_t s,
                        bool rq = false);
-// U: float2 [n][W][W] when f32 (formed in FP32 for the FP32 rotations), else double2
-cudaError_t launch_reflect_large(int W, int n, EighBufs b, const double* Z, void* U, bool f32,
-                                 cudaStream_t s);
 // U = Q D Z in FP32 by blocked compact-WY products (W > 64, the FP32-rotation modes): per-k
 // FP32 factors in wy (reflect_wy_scratch_bytes(W) per k-point, 16-byte aligned)
 size_t reflect_wy_scratch_bytes(int W);
