@@ -22,33 +22,91 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
   s = t;
 }
 
-// occupation of a level at energy E for Fermi level EF: step (strict) or Fermi-Dirac
-__device__ __forceinline__ double occupation(double E, double EF, double kT) {
-  if (kT == 0.0) return E < EF ? 1.0 : 0.0;
-  double x = (E - EF) / kT;
-  double ex = exp(-fabs(x));
-  return x > 0.0 ? ex / (1.0 + ex) : 1.0 / (1.0 + ex);
+// exp(x / kT) as mantissa (0.7 .. 1.5) and power of two, |power| <= 2^26: Cody-Waite reduction by
+// ln 2 = LN2 + LN2L, with the division's remainder carried along, so that the error stays a few ulp
+// for any x / kT (products of two of these never lose what (E - E_F) / kT would keep)
+__device__ __forceinline__ double exp_parts(double x, double kT, int& p2) {
+  constexpr double LN2 = 0.69314718055994530942, LN2L = 2.3190468138462995584e-17;
+  const double q = x / kT;
+  const double lo = fma(-q, kT, x) / kT;
+  const double n = fmin(fmax(rint(q * 1.4426950408889634074), -6e7), 6e7);
+  p2 = (int)n;
+  if (fabs(q) > 4e7) return q == q ? 1.0 : q;   // (also where the remainder overflows)
+  return exp(fma(-n, LN2L, fma(-n, LN2, q)) + lo);
 }
 
-__global__ void ksum_partial_kernel(const double* __restrict__ E, const double* __restrict__ Om,
-                                    int W, int n, int n_eta, int64_t eta_stride,
-                                    const double* __restrict__ E_F, int n_EF, double kT,
-                                    double2* __restrict__ part, int kpb) {
-  const int b = blockIdx.x;
+// kT > 0.  f(E, E_F) = 1 / (1 + exp(E / kT) exp(-E_F / kT)): the exponentials are formed once per level
+// and once per Fermi level, and a (level, Fermi level) pair takes a product, a power of two from
+// integer instructions, a multiply-add and a reciprocal (7 FP64 instructions where an exp, a division by
+// kT and one by 1 + exp took about 45), shared by all broadenings.  A CTA's 256 threads are TJ Fermi levels
+// x KG groups of k-points (one Fermi level: 256 k-points at a time instead of one thread);
+// KT k-points' levels are staged in shared memory.  Sums in a fixed order (Neumaier).
+constexpr int FD_NT = 256;
+constexpr int FD_LEVELS = 3072;   // levels staged at a time
+constexpr int FD_MAXE = 8;
+__global__ void __launch_bounds__(FD_NT) ksum_fd_kernel(const double* __restrict__ E,
+                                                        const double* __restrict__ Om, int W, int n,
+                                                        int n_eta, int64_t eta_stride,
+                                                        const double* __restrict__ E_F, int n_EF,
+                                                        double kT, double2* __restrict__ part, int kpb,
+                                                        int TJ, int KT) {
+  extern __shared__ double fsm[];
+  double* sa = fsm;                                       // [KT][W] mantissas
+  int* se = reinterpret_cast<int*>(sa + (size_t)KT * W);  // [KT][W] powers of two
+  __shared__ double2 red[FD_NT];
+  const int b = blockIdx.x, t = threadIdx.x;
   const int kb = b * kpb, ke = min(n, kb + kpb);
+  const int KG = min(FD_NT / TJ, KT);
+  const int tj = t % TJ, kg = t / TJ;
   const int n_out = n_eta * n_EF;
-  for (int o = threadIdx.x; o < n_out; o += blockDim.x) {
-    const int e = o / n_EF, j = o % n_EF;
-    const double ef = E_F[j];
-    double s = 0.0, c = 0.0;
-    for (int k = kb; k < ke; ++k) {
-      const double* Ek = E + (size_t)k * W;
-      const double* Ok = Om + e * eta_stride + (size_t)k * W;
-      double v = 0.0;
-      for (int q = 0; q < W; ++q) v = fma(occupation(Ek[q], ef, kT), Ok[q], v);
-      neumaier_add(s, c, v);
+  for (int j0 = 0; j0 < n_EF; j0 += TJ) {
+    const int j = j0 + tj;
+    const bool on = j < n_EF && kg < KG;
+    int pb = 0;
+    const double mb = on ? exp_parts(-E_F[j], kT, pb) : 1.0;
+    double s[FD_MAXE], c[FD_MAXE];
+#pragma unroll
+    for (int e = 0; e < FD_MAXE; ++e) { s[e] = 0.0; c[e] = 0.0; }
+    for (int k0 = kb; k0 < ke; k0 += KT) {
+      const int nk = min(KT, ke - k0);
+      __syncthreads();
+      for (int i = t; i < nk * W; i += FD_NT) sa[i] = exp_parts(E[(size_t)k0 * W + i], kT, se[i]);
+      __syncthreads();
+      if (on)
+        for (int kk = kg; kk < nk; kk += KG) {
+          const double* O = Om + (size_t)(k0 + kk) * W;
+          double v[FD_MAXE];
+#pragma unroll
+          for (int e = 0; e < FD_MAXE; ++e) v[e] = 0.0;
+          for (int q = 0; q < W; ++q) {
+            const int p2 = max(-1022, min(1000, se[kk * W + q] + pb));
+            const double y = fma(sa[kk * W + q] * mb, __longlong_as_double((long long)(1023 + p2) << 52), 1.0);
+            const double f = recip_nr(y);
+#pragma unroll
+            for (int e = 0; e < FD_MAXE; ++e)
+              if (e < n_eta) v[e] = fma(f, O[e * eta_stride + q], v[e]);
+          }
+#pragma unroll
+          for (int e = 0; e < FD_MAXE; ++e)
+            if (e < n_eta) neumaier_add(s[e], c[e], v[e]);
+        }
     }
-    part[(size_t)b * n_out + o] = make_double2(s, c);
+#pragma unroll
+    for (int e = 0; e < FD_MAXE; ++e) {
+      if (e >= n_eta) break;
+      __syncthreads();
+      red[t] = make_double2(s[e], c[e]);
+      __syncthreads();
+      if (on && kg == 0) {
+        double s2 = 0.0, c2 = 0.0;
+        for (int g = 0; g < KG; ++g) {
+          const double2 r = red[g * TJ + tj];
+          neumaier_add(s2, c2, r.x);
+          c2 += r.y;
+        }
+        part[(size_t)b * n_out + e * n_EF + j] = make_double2(s2, c2);
+      }
+    }
   }
 }
 
@@ -260,14 +318,17 @@ cudaError_t launch_ksum_partial(const double* E, double* Om, int W, int n, int n
                                 double2* part, int kpb, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int nb = (n + kpb - 1) / kpb;
-  if (kT == 0.0 && n_eta <= KS_MAXE) {
+  if (n_eta > KS_MAXE) return cudaErrorInvalidValue;
+  if (kT == 0.0) {
     const int64_t rows = (int64_t)n_eta * n;
     const int pb = (int)std::min<int64_t>((rows + 127) / 128, 152 * 16);
     band_prefix_kernel<<<pb, 128, 0, s>>>(Om, W, n, n_eta, eta_stride);
     const int nt = std::min(256, (n_EF + 31) / 32 * 32);
     ksum_step_kernel<<<nb, nt, 0, s>>>(E, Om, W, n, n_eta, eta_stride, E_F, n_EF, part, kpb);
   } else {
-    ksum_partial_kernel<<<nb, 128, 0, s>>>(E, Om, W, n, n_eta, eta_stride, E_F, n_EF, kT, part, kpb);
+    const int TJ = std::min(n_EF, FD_NT), KT = std::min(kpb, std::max(1, FD_LEVELS / W));
+    const size_t sm = (size_t)KT * W * (sizeof(double) + sizeof(int));
+    ksum_fd_kernel<<<nb, FD_NT, sm, s>>>(E, Om, W, n, n_eta, eta_stride, E_F, n_EF, kT, part, kpb, TJ, KT);
   }
   return cudaGetLastError();
 }
