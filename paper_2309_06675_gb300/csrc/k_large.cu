@@ -185,8 +185,6 @@ __global__ void __launch_bounds__(LW_MAX, 8) iit_kernel(int W, int n, EighBufs b
   }
 }
 
-template <typename T> struct cx;
-template <> struct cx<float> { typedef float2 type; __device__ static float2 make(double a, double b) { return make_float2((float)a, (float)b); } };
 
 constexpr int RB_COLS = 32;
 constexpr int RB_NT = 256;   // 8 threads per column
@@ -402,62 +400,64 @@ __global__ void __launch_bounds__(RB_NT) reflect_wy_kernel(int W, EighBufs b,
 }
 
 // ------------------------------------------------------------------ batched complex GEMMs
-// 64 x 64 output tile per CTA, 16 x 16 threads with 4 x 4 strided micro-tiles, K tiles of 16.
+// 16 TM x 16 TM output tile per CTA, 16 x 16 threads with TM x TM strided micro-tiles, K tiles of 16:
+// TM = 3 for 64 < W <= 96 (two tiles of 48 per dimension, where two of 64 spend (128 / W)^2 of the
+// products on padding: W = 81, 10,648 k-points: rotation stage 13.4 -> 8.9 ms), 4 above.
 
-constexpr int GT = 64, GK = 16;
+constexpr int GK = 16;
 
 // C[k] = H[k] U[k]; H from packed Hermitian rows P (leading dimension ldp), U complex in the
 // compute type.
-template <typename T>
+template <int TM>
 __global__ void __launch_bounds__(256) cgemm_herm_u_kernel(const double* __restrict__ P, int64_t ldp,
-                                                           const typename cx<T>::type* __restrict__ U,
+                                                           const float2* __restrict__ U,
                                                            int W,
-                                                           typename cx<T>::type* __restrict__ C) {
-  typedef typename cx<T>::type C2;
-  __shared__ C2 As[GT][GK + 1];
-  __shared__ C2 Bs[GK][GT + 1];
+                                                           float2* __restrict__ C) {
+  constexpr int GT = 16 * TM;
+  __shared__ float2 As[GT][GK + 1];
+  __shared__ float2 Bs[GK][GT + 1];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
   const int nt = (W + GT - 1) / GT;
   const int r0 = (blockIdx.y / nt) * GT, c0 = (blockIdx.y % nt) * GT;
   const int64_t k = blockIdx.x;
   const double* Pk = P + k * ldp;
-  const C2* Uk = U + (size_t)k * W * W;
-  T ax[4][4], ay[4][4];
+  const float2* Uk = U + (size_t)k * W * W;
+  float ax[TM][TM], ay[TM][TM];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { ax[i][j] = 0; ay[i][j] = 0; }
+    for (int j = 0; j < TM; ++j) { ax[i][j] = 0; ay[i][j] = 0; }
   for (int q0 = 0; q0 < W; q0 += GK) {
     for (int idx = t; idx < GT * GK; idx += 256) {
       const int r = idx / GK, q = idx % GK;
       const int gr = r0 + r, gq = q0 + q;
-      C2 a = cx<T>::make(0.0, 0.0);
+      float2 a = make_float2(0.f, 0.f);
       if (gr < W && gq < W) {
-        if (gr < gq) a = cx<T>::make(Pk[gr * W + gq], Pk[gq * W + gr]);
-        else if (gr > gq) a = cx<T>::make(Pk[gq * W + gr], -Pk[gr * W + gq]);
-        else a = cx<T>::make(Pk[gr * W + gr], 0.0);
+        if (gr < gq) a = make_float2((float)Pk[gr * W + gq], (float)Pk[gq * W + gr]);
+        else if (gr > gq) a = make_float2((float)Pk[gq * W + gr], -(float)Pk[gr * W + gq]);
+        else a = make_float2((float)Pk[gr * W + gr], 0.f);
       }
       As[r][q] = a;
     }
     for (int idx = t; idx < GK * GT; idx += 256) {
       const int q = idx / GT, c = idx % GT;
       const int gq = q0 + q, gc = c0 + c;
-      C2 v = cx<T>::make(0.0, 0.0);
+      float2 v = make_float2(0.f, 0.f);
       if (gq < W && gc < W) v = Uk[(size_t)gq * W + gc];
       Bs[q][c] = v;
     }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < GK; ++q) {
-      C2 a[4], bb[4];
+      float2 a[TM], bb[TM];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[ty + 16 * i][q];
+      for (int i = 0; i < TM; ++i) a[i] = As[ty + 16 * i][q];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[q][tx + 16 * j];
+      for (int j = 0; j < TM; ++j) bb[j] = Bs[q][tx + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TM; ++j) {
           ax[i][j] = fma(a[i].x, bb[j].x, ax[i][j]);
           ax[i][j] = fma(-a[i].y, bb[j].y, ax[i][j]);
           ay[i][j] = fma(a[i].x, bb[j].y, ay[i][j]);
@@ -466,61 +466,61 @@ __global__ void __launch_bounds__(256) cgemm_herm_u_kernel(const double* __restr
     }
     __syncthreads();
   }
-  typename cx<T>::type* Ck = C + (size_t)k * W * W;
+  float2* Ck = C + (size_t)k * W * W;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < TM; ++j) {
       const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * j;
-      if (r < W && c < W) { C2 v; v.x = ax[i][j]; v.y = ay[i][j]; Ck[(size_t)r * W + c] = v; }
+      if (r < W && c < W) { float2 v; v.x = ax[i][j]; v.y = ay[i][j]; Ck[(size_t)r * W + c] = v; }
     }
 }
 
 // V[k] = U[k]^H Tm[k]
-template <typename T>
-__global__ void __launch_bounds__(256) cgemm_uh_t_kernel(const typename cx<T>::type* __restrict__ U,
-                                                         const typename cx<T>::type* __restrict__ Tm,
-                                                         int W, typename cx<T>::type* __restrict__ V) {
-  typedef typename cx<T>::type C2;
-  __shared__ C2 As[GT][GK + 1];
-  __shared__ C2 Bs[GK][GT + 1];
+template <int TM>
+__global__ void __launch_bounds__(256) cgemm_uh_t_kernel(const float2* __restrict__ U,
+                                                         const float2* __restrict__ Tm,
+                                                         int W, float2* __restrict__ V) {
+  constexpr int GT = 16 * TM;
+  __shared__ float2 As[GT][GK + 1];
+  __shared__ float2 Bs[GK][GT + 1];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
   const int nt = (W + GT - 1) / GT;
   const int r0 = (blockIdx.y / nt) * GT, c0 = (blockIdx.y % nt) * GT;
   const int64_t k = blockIdx.x;
-  const C2* Uk = U + (size_t)k * W * W;
-  const C2* Tk = Tm + (size_t)k * W * W;
+  const float2* Uk = U + (size_t)k * W * W;
+  const float2* Tk = Tm + (size_t)k * W * W;
   if (r0 >= c0 + GT) return;   // strictly below the diagonal: V is Hermitian, never read
-  T ax[4][4], ay[4][4];
+  float ax[TM][TM], ay[TM][TM];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { ax[i][j] = 0; ay[i][j] = 0; }
+    for (int j = 0; j < TM; ++j) { ax[i][j] = 0; ay[i][j] = 0; }
   for (int q0 = 0; q0 < W; q0 += GK) {
     for (int idx = t; idx < GT * GK; idx += 256) {
       const int q = idx / GT, r = idx % GT;   // coalesced along r (a row of U)
       const int gr = r0 + r, gq = q0 + q;
-      C2 a = cx<T>::make(0.0, 0.0);
+      float2 a = make_float2(0.f, 0.f);
       if (gr < W && gq < W) { a = Uk[(size_t)gq * W + gr]; a.y = -a.y; }
       As[r][q] = a;
     }
     for (int idx = t; idx < GK * GT; idx += 256) {
       const int q = idx / GT, c = idx % GT;
       const int gq = q0 + q, gc = c0 + c;
-      Bs[q][c] = (gq < W && gc < W) ? Tk[(size_t)gq * W + gc] : cx<T>::make(0.0, 0.0);
+      Bs[q][c] = (gq < W && gc < W) ? Tk[(size_t)gq * W + gc] : make_float2(0.f, 0.f);
     }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < GK; ++q) {
-      C2 a[4], bb[4];
+      float2 a[TM], bb[TM];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[ty + 16 * i][q];
+      for (int i = 0; i < TM; ++i) a[i] = As[ty + 16 * i][q];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[q][tx + 16 * j];
+      for (int j = 0; j < TM; ++j) bb[j] = Bs[q][tx + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TM; ++j) {
           ax[i][j] = fma(a[i].x, bb[j].x, ax[i][j]);
           ax[i][j] = fma(-a[i].y, bb[j].y, ax[i][j]);
           ay[i][j] = fma(a[i].x, bb[j].y, ay[i][j]);
@@ -529,13 +529,13 @@ __global__ void __launch_bounds__(256) cgemm_uh_t_kernel(const typename cx<T>::t
     }
     __syncthreads();
   }
-  C2* Vk = V + (size_t)k * W * W;
+  float2* Vk = V + (size_t)k * W * W;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < TM; ++j) {
       const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * j;
-      if (r < W && c < W) { C2 v; v.x = ax[i][j]; v.y = ay[i][j]; Vk[(size_t)r * W + c] = v; }
+      if (r < W && c < W) { float2 v; v.x = ax[i][j]; v.y = ay[i][j]; Vk[(size_t)r * W + c] = v; }
     }
 }
 
@@ -557,10 +557,9 @@ __device__ __forceinline__ void large_two_sum_acc(float& hi, float& lo, float x)
 }
 
 // ------------------------------------------------------------------ curvature, thread per band
-template <typename T>
 __global__ void __launch_bounds__(LW_MAX) curvature_large_kernel(const double* __restrict__ E,
-                                                                 const typename cx<T>::type* __restrict__ Vx,
-                                                                 const typename cx<T>::type* __restrict__ Vy,
+                                                                 const float2* __restrict__ Vx,
+                                                                 const float2* __restrict__ Vy,
                                                                  int W, const double* __restrict__ etas,
                                                                  int n_eta, double* __restrict__ Om,
                                                                  int64_t eta_stride) {
@@ -581,52 +580,50 @@ __global__ void __launch_bounds__(LW_MAX) curvature_large_kernel(const double* _
   if (n >= W) return;
   const double thr2 = (1e-12 * s_emax) * (1e-12 * s_emax);
   const size_t base = (size_t)k * W * W;
-  if constexpr (std::is_same<T, float>::value) {
-    // FP32 velocities: the numerator is FP32-grade already, so the quotient is formed in FP32
-    // as in the W <= 64 kernels -- dE = E_p - E_q, its square and the eta = 0 cut-off in FP64,
-    // Kahan's difference of products for Im(v^x v^y), the sums as exact FP32 pairs (Knuth's
-    // TwoSum), and the FP64 quotient for a denominator below 2^-86 (eta and a gap below
-    // ~1e-13).  Both orders of a pair read the same (p < q) entry with the same arithmetic, so
-    // T_mn = -T_nm holds exactly.
-    float hi[MAXE], lo[MAXE];
-    float eta2[MAXE];
+  // FP32 velocities: the numerator is FP32-grade already, so the quotient is formed in FP32
+  // as in the W <= 64 kernels -- dE = E_p - E_q, its square and the eta = 0 cut-off in FP64,
+  // Kahan's difference of products for Im(v^x v^y), the sums as exact FP32 pairs (Knuth's
+  // TwoSum), and the FP64 quotient for a denominator below 2^-86 (eta and a gap below
+  // ~1e-13).  Both orders of a pair read the same (p < q) entry with the same arithmetic, so
+  // T_mn = -T_nm holds exactly.
+  float hi[MAXE], lo[MAXE];
+  float eta2[MAXE];
 #pragma unroll
-    for (int e = 0; e < MAXE; ++e) {
-      hi[e] = 0.f;
-      lo[e] = 0.f;
-      eta2[e] = e < n_eta ? (float)(etas[e] * etas[e]) : 0.f;
-    }
-    double fb[MAXE];   // FP64 fallback terms
+  for (int e = 0; e < MAXE; ++e) {
+    hi[e] = 0.f;
+    lo[e] = 0.f;
+    eta2[e] = e < n_eta ? (float)(etas[e] * etas[e]) : 0.f;
+  }
+  double fb[MAXE];   // FP64 fallback terms
 #pragma unroll
-    for (int e = 0; e < MAXE; ++e) fb[e] = 0.0;
-    for (int m = 0; m < W; ++m) {
-      if (m == n) continue;
-      const int p = n < m ? n : m, q = n < m ? m : n;
-      const float2 vx = Vx[base + (size_t)p * W + q];
-      const float2 vy = Vy[base + (size_t)p * W + q];
-      const float num = -2.0f * large_diff_of_products(vx.y, vy.x, vx.x, vy.y);
-      const double dE = sE[p] - sE[q];
-      const double d2 = dE * dE;
-      const float d2f = (float)d2;
-      const bool small0 = d2 <= thr2;
-      const float sgn = n < m ? 1.f : -1.f;
-#pragma unroll
-      for (int e = 0; e < MAXE; ++e) {
-        if (e >= n_eta) break;
-        if (eta2[e] == 0.f && small0) continue;
-        const float den = d2f + eta2[e];
-        if (den < 0x1p-86f) {
-          fb[e] += (double)sgn * ((double)num / fma(etas[e], etas[e], d2));
-        } else {
-          large_two_sum_acc(hi[e], lo[e], sgn * (num / den));
-        }
-      }
-    }
+  for (int e = 0; e < MAXE; ++e) fb[e] = 0.0;
+  for (int m = 0; m < W; ++m) {
+    if (m == n) continue;
+    const int p = n < m ? n : m, q = n < m ? m : n;
+    const float2 vx = Vx[base + (size_t)p * W + q];
+    const float2 vy = Vy[base + (size_t)p * W + q];
+    const float num = -2.0f * large_diff_of_products(vx.y, vy.x, vx.x, vy.y);
+    const double dE = sE[p] - sE[q];
+    const double d2 = dE * dE;
+    const float d2f = (float)d2;
+    const bool small0 = d2 <= thr2;
+    const float sgn = n < m ? 1.f : -1.f;
 #pragma unroll
     for (int e = 0; e < MAXE; ++e) {
       if (e >= n_eta) break;
-      Om[e * eta_stride + k * W + n] = ((double)hi[e] + (double)lo[e]) + fb[e];
+      if (eta2[e] == 0.f && small0) continue;
+      const float den = d2f + eta2[e];
+      if (den < 0x1p-86f) {
+        fb[e] += (double)sgn * ((double)num / fma(etas[e], etas[e], d2));
+      } else {
+        large_two_sum_acc(hi[e], lo[e], sgn * (num / den));
+      }
     }
+  }
+#pragma unroll
+  for (int e = 0; e < MAXE; ++e) {
+    if (e >= n_eta) break;
+    Om[e * eta_stride + k * W + n] = ((double)hi[e] + (double)lo[e]) + fb[e];
   }
 }
 
@@ -678,14 +675,18 @@ cudaError_t launch_berry_large(const double* E, const void* Uv, const double* X,
                                int64_t eta_stride, void* Tbuf, void* Vx, void* Vy, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (W > LW_MAX || n_eta > MAXE) return cudaErrorInvalidValue;
-  const int tiles = (W + GT - 1) / GT;
-  dim3 grid(n, tiles * tiles);
   const float2* U = (const float2*)Uv;
-  cgemm_herm_u_kernel<float><<<grid, 256, 0, s>>>(X, ld, U, W, (float2*)Tbuf);
-  cgemm_uh_t_kernel<float><<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vx);
-  cgemm_herm_u_kernel<float><<<grid, 256, 0, s>>>(Y, ld, U, W, (float2*)Tbuf);
-  cgemm_uh_t_kernel<float><<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vy);
-  curvature_large_kernel<float><<<n, LW_MAX, 0, s>>>(E, (const float2*)Vx, (const float2*)Vy, W,
+  auto gemms = [&](auto herm_u, auto uh_t, int gt) {
+    const int tiles = (W + gt - 1) / gt;
+    const dim3 grid(n, tiles * tiles);
+    herm_u<<<grid, 256, 0, s>>>(X, ld, U, W, (float2*)Tbuf);
+    uh_t<<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vx);
+    herm_u<<<grid, 256, 0, s>>>(Y, ld, U, W, (float2*)Tbuf);
+    uh_t<<<grid, 256, 0, s>>>(U, (const float2*)Tbuf, W, (float2*)Vy);
+  };
+  if (W <= 96) gemms(cgemm_herm_u_kernel<3>, cgemm_uh_t_kernel<3>, 48);
+  else gemms(cgemm_herm_u_kernel<4>, cgemm_uh_t_kernel<4>, 64);
+  curvature_large_kernel<<<n, LW_MAX, 0, s>>>(E, (const float2*)Vx, (const float2*)Vy, W,
                                                       etas, n_eta, Om, eta_stride);
   return cudaGetLastError();
 }
