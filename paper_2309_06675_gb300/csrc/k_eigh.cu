@@ -68,8 +68,8 @@ __device__ __forceinline__ int symv_partitions(int m, int nt, int cap) {
 // NTT = 512 threads: one CTA (136 KB of shared memory at W = 128) holds an SM, and more warps
 // than 256 cover its barriers (W = 128: 235 -> 229 ms per 18,432 k-points; 1,024 threads
 // with twice the symv parts: 240 ms)
-template <typename T, int NTT>
-__global__ void __launch_bounds__(NTT, 1) tridiag_kernel(const T* __restrict__ Hp, int64_t ld, int W,
+template <typename T, int NTT, int MINB>
+__global__ void __launch_bounds__(NTT, MINB) tridiag_kernel(const T* __restrict__ Hp, int64_t ld, int W,
                                                      EighBufs b) {
   // the reflector is read from its column of A (not copied), the symv partials share their
   // array with p, and beta_i, tau_i go to the outputs as they are formed (beta_i into the phase
@@ -877,7 +877,10 @@ static cudaError_t launch_tridiag_ld(const double* Hp, int64_t ld, int W, int n,
     tridiag2_kernel<<<(n + 1) / 2, 512, sm2, s>>>(Hp, ld, W, n, b);
     return cudaGetLastError();
   }
-  return go(tridiag_kernel<double, TRI_NT>, TRI_NT);
+  // three CTAs per SM where their shared memory allows it (W <= 91: 75 KB), at 40 registers a thread; the
+  // 54 that one CTA takes allow two (W = 81, 10,648 k-points: 33.1 -> 30.5 ms)
+  if (3 * (sm + 1024 + 64) <= (size_t)228 * 1024) return go(tridiag_kernel<double, TRI_NT, 3>, TRI_NT);
+  return go(tridiag_kernel<double, TRI_NT, 1>, TRI_NT);
 }
 
 cudaError_t launch_tridiag(const double* Hp, int W, int n, EighBufs b, cudaStream_t s) {
