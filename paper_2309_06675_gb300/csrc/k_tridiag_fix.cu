@@ -10,14 +10,17 @@
 // column (the column's norm, the Householder vector's scale) is FP64.
 //
 // KP k-points per CTA, TPK threads each (2 x 128 at W <= 64, 4 x 64 at 32, 8 x 32 at 16, 16 x 16 at 8,
-// 1 x 512 above 64); warp 0 runs the scalar steps of all KP k-points at once, 32 / KP lanes each.
+// 1 x 256 or 384 above 64); warp 0 runs the scalar steps of all KP k-points at once, 32 / KP lanes each.
 // Per column i with reflector I - 2 w w^dagger (w a unit vector, kept in column i of A):
-//   1 (warp 0)  |x|, w = v / |v|, v = x + e^{i arg x_0} |x| e_0
-//   2 (all)     partial sums of p = A w
-//   3 (warp 0)  p, K = w^dagger p, h = p - K w
-//   4 (all)     A <- A - 2 (w h^dagger + h w^dagger), lower triangle
+//   1 (all)     partial sums of p = A w
+//   2 (warp 0)  p, K = w^dagger p, h = p - K w
+//   3 (warp 0)  column i + 1 of A <- A - 2 (w h^dagger + h w^dagger), its |x|, and the next
+//               w = v / |v|, v = x + e^{i arg x_0} |x| e_0
+//     (others)  the rest of the lower triangle of that update
+// The next column's reflector is a chain of some 2,000 clocks; beside the update it is hidden (on
+// its own between two barriers: W = 64, 4,096 k-points 2.87 ms, now 2.77; W = 97, 2,744: 11.4, now 11.0).
 // What bounds it: the integer multiply-adds (12 per complex product) and, for short columns, the
-// latency of steps 1 and 3, which the other CTAs of the SM fill.
+// latency of step 2, which the other CTAs of the SM fill.
 #include <algorithm>
 
 #include "fixed.cuh"
@@ -49,7 +52,7 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
   unsigned char* rowtab = smraw + KP * per_k * 16;                  // row of a strictly lower element
   __shared__ unsigned long long s_sq[KP];
   __shared__ unsigned s_max[KP];
-  __shared__ int s_act[KP];
+  __shared__ int s_act[2][KP];   // of the odd and of the even columns
   const int64_t k = (int64_t)blockIdx.x * KP + g;
   const bool live = k < n;
 
@@ -111,64 +114,91 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
   const int64_t kw = (int64_t)blockIdx.x * KP + kk;
   const bool livek = kw < n;
 
-  for (int i = 0; i < W - 2; ++i) {
-    const int o = i + 1;       // first row of the trailing block
-    const int m = W - 1 - i;   // its size
-    if (warp == 0) {
-      double xr[4], xi[4];
-      double s2 = 0.0;
+  // warp 0, for its k-point: the reflector of column i (rows i + 1 + r).  upd: the previous step's
+  // rank-2 update of that column (its trailing column 0) is still to be made, from h and w in spk.
+  auto reflector = [&](int i, bool upd) {
+    const int o = i + 1, m = W - 1 - i;
+    double xr[4], xi[4];
+    double s2 = 0.0;
+    const int4* h4 = reinterpret_cast<const int4*>(spk);
+    const int4 h0 = upd ? h4[0] : make_int4(0, 0, 0, 0), w0 = upd ? h4[W] : h0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = l + LPK * q;
+      xr[q] = xi[q] = 0.0;
+      if (r < m && livek) {
+        int4* pa = &Ak[tri(o + r, i)];
+        const int4 a = *pa;
+        long long vx = fx::value(a.x, a.y), vy = fx::value(a.z, a.w);
+        if (upd) {   // row r here is row r + 1 of the previous trailing block
+          const int4 hr = h4[r + 1], wr = h4[W + r + 1];
+          fx::Acc acc;
+          fx::zero(acc);
+          fx::cmadc(acc, h0, -h0.z, -h0.w, wr);   // w_r conj(h_0) + h_r conj(w_0), units 2^-61
+          fx::cmadc(acc, w0, -w0.z, -w0.w, hr);
+          vx -= fx::rshift(fx::fold(acc.rh, acc.rm), 1);
+          vy -= fx::rshift(fx::fold(acc.ih, acc.im), 1);
+          *pa = fx::climbs(vx, vy);
+        }
+        xr[q] = (double)vx;
+        xi[q] = (double)vy;
+        if (r > 0) s2 = fma(xr[q], xr[q], fma(xi[q], xi[q], s2));
+      }
+    }
+    if (upd && l == 0 && livek) {   // the diagonal entry above the column
+      int4* pa = &Ak[tri(i, i)];
+      long long hh = 0, c = 0;
+      fx::mad(hh, h0.x, w0.x); fx::mad(c, h0.x, w0.y); fx::mad(c, h0.y, w0.x);
+      fx::mad(hh, h0.z, w0.z); fx::mad(c, h0.z, w0.w); fx::mad(c, h0.w, w0.z);
+      const int2 x = fx::limbs(fx::value(pa->x, pa->y) - fx::fold(hh, c));
+      *pa = make_int4(x.x, x.y, 0, 0);
+    }
+    if (i >= W - 2) return;   // (the last column is only brought up to date)
+#pragma unroll
+    for (int f = LPK / 2; f > 0; f >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, f);
+    const double ax = __shfl_sync(0xffffffffu, xr[0], kk * LPK), ay = __shfl_sync(0xffffffffu, xi[0], kk * LPK);
+    // |x| in the even lanes, |x_0| in the odd ones: one reciprocal square root
+    const double aa2 = fma(ax, ax, ay * ay);
+    const double arg = (l & 1) ? aa2 : aa2 + s2;
+    const double ri = mag_bits(arg) != 0ull ? rsqrt(arg) : 0.0;
+    const double root = arg * ri;
+    const double nrm = __shfl_sync(0xffffffffu, root, kk * LPK);
+    const double aa = __shfl_sync(0xffffffffu, root, kk * LPK + 1);
+    const double ra = __shfl_sync(0xffffffffu, ri, kk * LPK + 1);
+    const bool az = mag_bits(aa2) == 0ull;
+    const double px = az ? 1.0 : ax * ra, py = az ? 0.0 : ay * ra;   // the unit phase of x_0
+    const bool act = mag_bits(s2) != 0ull;
+    if (act) {
+      // v = (ph (|x| + |x_0|), x_1, ...), |v|^2 = 2 |x| (|x| + |x_0|)
+      const double tt = nrm + aa;
+      const double f = rsqrt(2.0 * nrm * tt);
+      if (l == 0) {
+        xr[0] = px * tt;
+        xi[0] = py * tt;
+        betak[i] = make_double2(-px * nrm, -py * nrm);
+      }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int r = l + LPK * q;
-        xr[q] = xi[q] = 0.0;
-        if (r < m && livek) {
-          const int4 a = Ak[tri(o + r, i)];
-          xr[q] = (double)fx::value(a.x, a.y);
-          xi[q] = (double)fx::value(a.z, a.w);
-          if (r > 0) s2 = fma(xr[q], xr[q], fma(xi[q], xi[q], s2));
-        }
+        if (r < m)
+          Ak[tri(o + r, i)] = fx::climbs(fx::from_double(xr[q] * f, 58), fx::from_double(xi[q] * f, 58));
       }
-#pragma unroll
-      for (int f = LPK / 2; f > 0; f >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, f);
-      const double ax = __shfl_sync(0xffffffffu, xr[0], kk * LPK), ay = __shfl_sync(0xffffffffu, xi[0], kk * LPK);
-      // |x| in the even lanes, |x_0| in the odd ones: one reciprocal square root
-      const double aa2 = fma(ax, ax, ay * ay);
-      const double arg = (l & 1) ? aa2 : aa2 + s2;
-      const double ri = mag_bits(arg) != 0ull ? rsqrt(arg) : 0.0;
-      const double root = arg * ri;
-      const double nrm = __shfl_sync(0xffffffffu, root, kk * LPK);
-      const double aa = __shfl_sync(0xffffffffu, root, kk * LPK + 1);
-      const double ra = __shfl_sync(0xffffffffu, ri, kk * LPK + 1);
-      const bool az = mag_bits(aa2) == 0ull;
-      const double px = az ? 1.0 : ax * ra, py = az ? 0.0 : ay * ra;   // the unit phase of x_0
-      const bool act = mag_bits(s2) != 0ull;
-      if (act) {
-        // v = (ph (|x| + |x_0|), x_1, ...), |v|^2 = 2 |x| (|x| + |x_0|)
-        const double tt = nrm + aa;
-        const double f = rsqrt(2.0 * nrm * tt);
-        if (l == 0) {
-          xr[0] = px * tt;
-          xi[0] = py * tt;
-          betak[i] = make_double2(-px * nrm, -py * nrm);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int r = l + LPK * q;
-          if (r < m)
-            Ak[tri(o + r, i)] = fx::climbs(fx::from_double(xr[q] * f, 58), fx::from_double(xi[q] * f, 58));
-        }
-      } else if (l == 0 && livek) {
-        betak[i] = make_double2(ax, ay);   // no reflection
-      }
-      if (l == 0) {
-        s_act[kk] = act ? 1 : 0;
-        if (livek) b.tau[kw * W + i] = act ? 2.0 : 0.0;
-      }
+    } else if (l == 0 && livek) {
+      betak[i] = make_double2(ax, ay);   // no reflection
     }
-    __syncthreads();
-    const bool act = s_act[g] != 0;
+    if (l == 0) {
+      s_act[i & 1][kk] = act ? 1 : 0;
+      if (livek) b.tau[kw * W + i] = act ? 2.0 : 0.0;
+    }
+  };
+
+  if (warp == 0 && W > 2) reflector(0, false);
+  __syncthreads();
+  for (int i = 0; i < W - 2; ++i) {
+    const int o = i + 1;       // first row of the trailing block
+    const int m = W - 1 - i;   // its size
     const int P = max(1, min(TPK / m, 8));   // column partitions of a row
-    if (act) {
+    if (s_act[i & 1][g]) {
       const int part = th / m, r = th - part * m;
       if (part < P) {
         fx::Acc acc;
@@ -186,7 +216,7 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
       }
     }
     __syncthreads();
-    if (warp == 0 && s_act[kk]) {
+    if (warp == 0 && s_act[i & 1][kk]) {
       // (a k-point's lanes take this together; the shuffles stay inside its group)
       const unsigned gm = (LPK == 32 ? 0xffffffffu : ((1u << (LPK & 31)) - 1u)) << (kk * LPK);
       long long pr[4], pi[4];
@@ -232,30 +262,32 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
       }
     }
     __syncthreads();
-    if (act) {
-      const int4* hb = reinterpret_cast<const int4*>(sp);
-      const int4* wb = hb + W;
-      const int nlow = m * (m - 1) / 2;
-      for (int idx = th; idx < nlow; idx += TPK) {
-        const int r = rowtab[idx], c = idx - r * (r - 1) / 2;
+    // Warp 0 brings the next column up to date and forms its reflector (a chain of some 2,000 clocks)
+    // while the other warps update the rest of all KP trailing blocks.
+    if (warp == 0) {
+      reflector(i + 1, s_act[i & 1][kk] != 0);
+    } else {
+      const int m1 = m - 1;                  // trailing rows and columns 1 .. m - 1
+      const int nl = m1 * (m1 + 1) / 2;      // their lower triangle with the diagonal
+      const FastDiv dn((uint32_t)nl);
+      for (int it = t - 32; it < KP * nl; it += KP * TPK - 32) {
+        const int gg = KP == 1 ? 0 : (int)dn.div(it), idx = it - gg * nl;
+        if (!s_act[i & 1][gg]) continue;
+        // packed with its diagonal: row r' >= c', from the table of strictly lower elements of the block
+        // one larger (row r' + 1, column c')
+        const int r = rowtab[idx], c = idx - r * (r - 1) / 2 + 1;
+        int4* Ag = base + gg * per_k;
+        const int4* hb = Ag + NA;
+        const int4* wb = hb + W;
         const int4 hc = hb[c], wr = wb[r], wc = wb[c], hr = hb[r];
         fx::Acc acc;
         fx::zero(acc);
         fx::cmadc(acc, hc, -hc.z, -hc.w, wr);   // w_r conj(h_c) + h_r conj(w_c), units 2^-61
         fx::cmadc(acc, wc, -wc.z, -wc.w, hr);
-        int4* pa = &A[tri(o + r, o + c)];
+        int4* pa = &Ag[tri(o + r, o + c)];
         const int4 a = *pa;
         *pa = fx::climbs(fx::value(a.x, a.y) - fx::rshift(fx::fold(acc.rh, acc.rm), 1),
                          fx::value(a.z, a.w) - fx::rshift(fx::fold(acc.ih, acc.im), 1));
-      }
-      for (int r = th; r < m; r += TPK) {
-        const int4 h = hb[r], w = wb[r];
-        long long hh = 0, c = 0;   // Re(w_r conj(h_r)), twice of it
-        fx::mad(hh, h.x, w.x); fx::mad(c, h.x, w.y); fx::mad(c, h.y, w.x);
-        fx::mad(hh, h.z, w.z); fx::mad(c, h.z, w.w); fx::mad(c, h.w, w.z);
-        int4* pa = &A[tri(o + r, o + r)];
-        const int2 x = fx::limbs(fx::value(pa->x, pa->y) - fx::fold(hh, c));
-        *pa = make_int4(x.x, x.y, 0, 0);
       }
     }
     __syncthreads();
@@ -352,7 +384,13 @@ cudaError_t launch_tridiag_fix(const double* Hp, int64_t ld, int W, int n, EighB
   if (W <= 16) return go(tridiag_fix_kernel<8, 32, 3>, 8, 32);
   if (W <= 32) return go(tridiag_fix_kernel<4, 64, 3>, 4, 64);
   if (W <= 64) return go(tridiag_fix_kernel<2, 128, 3>, 2, 128);
-  return go(tridiag_fix_kernel<1, 512, 1>, 1, 512);
+  // above 64 one k-point per CTA, and more CTAs per SM before more threads: three of 256 threads where their
+  // shared memory fits (W <= 90), else 384 (two CTAs to W = 108).  4,096 k-points: W = 66 3.5 ms, W = 80 5.1
+  // (one CTA of 512: 8.6, 11.6; two of 512: 5.0, 6.9); 2,744: W = 97 6.5, W = 107 8.0, W = 128 17.5
+  // (256 threads: 6.7, 8.4, 19.2; one of 512: 11.0, 13.2, 18.2).
+  if (3 * (fix_bytes_per_k(W, 256) + (size_t)W * (W - 1) / 2 + 1024 + 64) <= (size_t)228 * 1024)
+    return go(tridiag_fix_kernel<1, 256, 3>, 1, 256);
+  return go(tridiag_fix_kernel<1, 384, 2>, 1, 384);
 }
 
 }  // namespace kubo
