@@ -302,13 +302,16 @@ __global__ void __launch_bounds__(256) unorm_kernel(const double2* __restrict__ 
 }
 
 // ------------------------------------------------------------------ U = Q D Z
-// One k-point (above W = 64: a third of its columns) per CTA: u (limbs, 58 fractional bits) starts as
+// One k-point (above W = 64: half of its columns) per CTA: u (limbs, 58 fractional bits) starts as
 // its columns of D Z; the unit reflectors
 // w_j = v_j sqrt(tau_j / 2), H_j = I - 2 w_j w_j^dagger, are applied four at a time from the last:
 //   s_a = w_a^dagger u,   h_a = s_a - 2 sum_{b > a} (w_a^dagger w_b) h_b,   u -= 2 sum_a w_a h_a,
 // which is H_j0 H_j0+1 H_j0+2 H_j0+3 u with one pass for the four sums and one for the update (a
 // triangular factor as in the compact WY form would need more range than the h_a, each at most
 // 1).  Four lanes share the rows of a column.
+// What bounds it: the 24 integer multiply-adds per element and reflector, each four cycles of a
+// sub-core's multiplier (80 % busy at W = 64): 4,096 k-points take 2.55 ms, with the update's operands pinned
+// (fixed.cuh); 3.4 before that.
 constexpr int RF_NT = 256;
 constexpr int RF_NB = 4;
 
@@ -412,10 +415,10 @@ __global__ void __launch_bounds__(RF_NT, 2)
           fx::mad(s[a].ih, x.z, u.x); fx::mad(s[a].im, x.z, u.y); fx::mad(s[a].im, x.w, u.x);
         }
       }
-      int4 h[RF_NB];
+      int4 h[RF_NB];   // -h_a
 #pragma unroll
       for (int a = RF_NB - 1; a >= 0; --a) {
-        long long re = fx::fold(s[a].rh, s[a].rm), im = -fx::fold(s[a].ih, s[a].im);   // units 2^-60
+        long long re = -fx::fold(s[a].rh, s[a].rm), im = fx::fold(s[a].ih, s[a].im);   // -s, units 2^-60
 #pragma unroll
         for (int o = 1; o < 4; o <<= 1) {
           re += __shfl_xor_sync(0xffffffffu, re, o);
@@ -434,16 +437,18 @@ __global__ void __launch_bounds__(RF_NT, 2)
       if (act)
 #pragma unroll 1
         for (int r = j0 + 1 + q; r < W; r += 4) {
+          // u + sum w (-h) / 2: the sums start at 2 u and the roundings' halves
+          const int4 u = su[r * LD + c];
           fx::Acc d;
-          fx::zero(d);
+          d.rh = (long long)u.x * (1 << (fx::LB + 1)) + (2 * u.y + 1);
+          d.ih = (long long)u.z * (1 << (fx::LB + 1)) + (2 * u.w + 1);
+          d.rm = d.im = 1 << (fx::LB - 1);
 #pragma unroll
           for (int a = 0; a < RF_NB; ++a) {
             const int4 x = w[r * RF_NB + a];
-            fx::cmad(d, h[a], -h[a].z, -h[a].w, x);
+            fx::cmad(d, x, -x.z, -x.w, fx::pin(h[a]));
           }
-          const int4 u = su[r * LD + c];
-          su[r * LD + c] = fx::climbs(fx::value(u.x, u.y) - fx::rshift(fx::fold(d.rh, d.rm), 1),
-                                      fx::value(u.z, u.w) - fx::rshift(fx::fold(d.ih, d.im), 1));
+          su[r * LD + c] = fx::climbs((d.rh + (d.rm >> fx::LB)) >> 1, (d.ih + (d.im >> fx::LB)) >> 1);
         }
     }
     __syncthreads();
@@ -514,7 +519,7 @@ __global__ void __launch_bounds__(256) reflect_small_kernel(int W, int n, int kp
         const int4 w = sw[r * W + j];
         fx::Acc d;
         fx::zero(d);
-        fx::cmad(d, h, -h.z, -h.w, w);
+        fx::cmad(d, w, -w.z, -w.w, fx::pin(h));
         u[r] = fx::climbs(fx::value(u[r].x, u[r].y) - fx::rshift(fx::fold(d.rh, d.rm), 1),
                           fx::value(u[r].z, u[r].w) - fx::rshift(fx::fold(d.ih, d.im), 1));
       }
@@ -579,9 +584,9 @@ cudaError_t launch_reflect_fix(int W, int n, EighBufs b, const double* Z, double
     };
     return W <= 8 ? go(reflect_small_kernel<8>) : go(reflect_small_kernel<16>);
   }
-  // all columns up to W = 64; above, an even third of them, so that two CTAs share an SM (90 KB at
-  // W = 128)
-  const int nb = W <= 64 ? 1 : 3, CB = (W + nb - 1) / nb;
+  // all columns up to W = 64, half of them above (W = 97, 2,736 k-points: halves 6.7 ms, thirds 7.3, quarters
+  // 6.9; W = 128: 14.5, 14.7, 15.8; W = 64, 4,096: all columns 2.55, halves 2.65; W = 32: 0.46, 0.50)
+  const int nb = W <= 64 ? 1 : 2, CB = (W + nb - 1) / nb;
   const int LD = pad ? CB | 1 : CB;
   const size_t sm = ((size_t)W * LD + 2 * (size_t)W * RF_NB + 12 + W) * sizeof(int4) + (size_t)W * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(reflect_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

@@ -134,8 +134,9 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
           const int4 hr = h4[r + 1], wr = h4[W + r + 1];
           fx::Acc acc;
           fx::zero(acc);
-          fx::cmadc(acc, h0, -h0.z, -h0.w, wr);   // w_r conj(h_0) + h_r conj(w_0), units 2^-61
-          fx::cmadc(acc, w0, -w0.z, -w0.w, hr);
+          const int4 hp = fx::pin(h0), wp = fx::pin(w0);
+          fx::cmadc(acc, hp, -hp.z, -hp.w, wr);   // w_r conj(h_0) + h_r conj(w_0), units 2^-61
+          fx::cmadc(acc, wp, -wp.z, -wp.w, hr);
           vx -= fx::rshift(fx::fold(acc.rh, acc.rm), 1);
           vy -= fx::rshift(fx::fold(acc.ih, acc.im), 1);
           *pa = fx::climbs(vx, vy);
@@ -253,8 +254,9 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
         const int r = l + LPK * q;
         if (r < m) {
           long long rh = 0, rm = 0, ih = 0, im = 0;
-          fx::mad(rh, K.x, w[q].x); fx::mad(rm, K.x, w[q].y); fx::mad(rm, K.y, w[q].x);
-          fx::mad(ih, K.x, w[q].z); fx::mad(im, K.x, w[q].w); fx::mad(im, K.y, w[q].z);
+          const int4 wq = fx::pin(w[q]), Kp = fx::pin(make_int4(K.x, K.y, 0, 0));
+          fx::mad(rh, Kp.x, wq.x); fx::mad(rm, Kp.x, wq.y); fx::mad(rm, Kp.y, wq.x);
+          fx::mad(ih, Kp.x, wq.z); fx::mad(im, Kp.x, wq.w); fx::mad(im, Kp.y, wq.z);
           int4* s4 = reinterpret_cast<int4*>(spk);
           s4[r] = fx::climbs(pr[q] - fx::rshift(fx::fold(rh, rm), 2), pi[q] - fx::rshift(fx::fold(ih, im), 2));
           s4[W + r] = w[q];
