@@ -11,15 +11,19 @@
 // K is an integer of at most 7 x 128 x 2^14 < 2^24, exact in the FP32 accumulator.
 //
 // One tile is 64 complex rows by up to 64 columns as a real product [re; im] (M = 128) with K = 2 W:
-// the rows [Ar | -Ai] and [Ai | Ar] against [Br; Bi].  A chunk is 16 of the inner index (32 of K); the
-// staging warps load it in FP64, cut it and write it to shared memory (128-byte swizzle, a row of 64
-// FP16 holding two chunks) while the MMAs of the other half run; the eight level sums of a
-// tile fill the 512 TMEM columns (N = 64); eight warps add them in one int64 (units
-// 2^-55 of the operand scales), convert, and write 16 columns at a time through shared memory.
+// the rows [Ar | -Ai] and [Ai | Ar] against [Br; Bi].  A chunk is 8 of the inner index (K = 16); two groups
+// of staging warps take the chunks in turn: load in FP64, cut, write to shared memory (128-byte swizzle, a
+// row of 64 FP16 holding four chunks) while the MMAs of the chunks before run.  The eight level
+// sums of a tile fill the 512 TMEM columns (N = 64); eight warps, each with both parts of 16
+// complex rows in its lanes, add them in one int64 (units 2^-55 of the operand scales), convert, and write 8
+// columns at a time through shared memory of their own.
 //
-// What bounds it: the MMAs (34 x 128 x N x 2 W / 4096 clocks per tile) and the staging of the next chunk
-// (about 500 instructions for each 8 complex entries) take about the same time.  FP64 FMA kernels
-// of the same products ran at 1.1 TFLOP/s; measured here: see the table beside the launcher.
+// What bounds it: a tile of W = 64 takes 16.8 us, where its MMAs (34 x 128 x N x 2 W / 4096 clocks) take 4.6,
+// the staging alone 12 (integer instructions at 44 % of their rate, the rest waits for loads and
+// between its steps) and the drain alone 9; the drain cannot overlap the MMAs, which need all of TMEM.
+// (One staging group with 16-index chunks and slabs shared by the eight drain warps: 20.8 us.)
+// W = 64, 4,096 k-points: the four products and the curvature take 2.2 ms (FP64 FMA kernels of the same
+// products ran at 1.1 TFLOP/s); W = 97, 2,744: 9.1 ms.
 //
 // Every mbarrier wait is bounded; a wait that gives up sets ST_TIMEOUT and the CTA returns.
 #include <algorithm>
@@ -37,16 +41,18 @@ using namespace tc;
 using namespace dig;
 
 constexpr int BM = 128;             // [re; im] of 64 complex rows
-constexpr int CH = 16;              // inner indices per chunk (K = 32)
-constexpr int GROUP = 4;            // chunks per drain (K = 128)
+constexpr int CH = 8;               // inner indices per chunk (K = 16)
+constexpr int NSLOT = 4;            // chunks in shared memory: 32 bytes each of a row
+constexpr int GROUP = 8;            // chunks per drain (K = 128)
 constexpr int NLEV = 8;
-constexpr int ROW_BYTES = 128;      // 64 BF16: two chunks
+constexpr int ROW_BYTES = 128;      // 64 FP16: four chunks
 constexpr int A_SLICE = BM * ROW_BYTES;          // 16 KB
-constexpr int STAGE_THREADS = 256;
+constexpr int STAGE_THREADS = 512;  // two groups of 256, alternate chunks
 constexpr int EPI_THREADS = 256;
-constexpr int THREADS = STAGE_THREADS + EPI_THREADS;   // 16 warps: 128 registers each
+constexpr int MMA_WARP = (STAGE_THREADS + EPI_THREADS) / 32;
+constexpr int THREADS = STAGE_THREADS + EPI_THREADS + 32;   // 25 warps: 80 registers each
 constexpr int TMEM_COLS = 512;
-constexpr int SLAB = 16;            // output columns written together
+constexpr int SLAB = 8;             // output columns written together
 constexpr int E_MIN = -1080;        // exponent of an all-zero operand
 
 __host__ __device__ __forceinline__ uint32_t idesc_n(int n) {
@@ -56,8 +62,8 @@ __host__ __device__ __forceinline__ uint32_t idesc_n(int n) {
 
 __device__ __forceinline__ int op_exp(const ZOp& o, int64_t k) { return o.e ? max(o.e[k], E_MIN) : 0; }
 
-// v 2^e in FP64: the conversion is one instruction of the (here idle) FP64 pipe, the power of two an
-// addition to the exponent field
+// v 2^e in FP64: the conversion runs on the (here idle) FP64 pipe, the power of two is an addition to the
+// exponent field (converting in integer instructions: 8 % more instructions, the same time)
 __device__ __forceinline__ double scaled_double(long long v, int e) {
   const double d = (double)v;
   if (e < -900 || e > 900) return fx::scale_pow2(d, e);
@@ -65,36 +71,36 @@ __device__ __forceinline__ double scaled_double(long long v, int e) {
 }
 
 // ------------------------------------------------------------------ operand fetch
-// A group of threads (128 for A, 2 ncp for B) brings one chunk of its operand, nrow rows (A) or columns
-// (B) from g0 on by 16 inner indices from q0 on, into shared memory: entry (r, q) to slot
-// raw[(q % 8) RAW_PITCH + r + nrow (q / 8)], where the thread that cuts row r's half chunk q / 8
-// reads its eight entries without bank conflicts.  Asynchronous copies (zeros outside the matrix), the
-// lanes along whichever index is contiguous in memory.
-constexpr int RAW_PITCH = STAGE_THREADS + 1;
+// Half a staging group (128 threads for A, 2 ncp for B) brings one chunk of its operand, nrow rows (A) or
+// columns (B) from g0 on by 8 inner indices, into shared memory: entry (r, q) to slot
+// raw[q RAW_PITCH + r], where the threads that cut row r read its eight entries without bank conflicts.
+// Asynchronous copies (zeros outside the matrix), the lanes along whichever index is contiguous in
+// memory.
+constexpr int RAW_PITCH = 129;   // 64 rows of A and up to 64 columns of B
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* dst, const void* src, bool on) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES),
                "r"(on ? BYTES : 0)
                : "memory");
 }
-// lanes along the inner index: rows (t / 16) + RS i, index t % 16; mask: rows inside the matrix
+// lanes along the inner index: rows (t / 8) + RS i, index t % 8; mask: rows inside the matrix
 template <int BYTES, int RS>
 __device__ __forceinline__ void fetch_rows(const char* src, int64_t step, const char* safe, double2* dst,
                                            unsigned mask, bool on) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < 4; ++i) {
     const bool g = on && ((mask >> i) & 1u);
     cp_async<BYTES>(dst + i * RS, g ? src : safe, g);
     src += step;
   }
 }
 // lanes along the rows: row t % nrow, inner indices (t / nrow) + 2 i, nq of them inside the matrix
-template <int BYTES, int NROW>
+template <int BYTES>
 __device__ __forceinline__ void fetch_cols(const char* src, int64_t step, const char* safe, char* dst, int nq) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < 4; ++i) {
     const bool g = 2 * i < nq;
-    cp_async<BYTES>(dst + (2 * (i & 3) * RAW_PITCH + NROW * (i >> 2)) * (int)sizeof(double2), g ? src : safe, g);
+    cp_async<BYTES>(dst + 2 * i * RAW_PITCH * (int)sizeof(double2), g ? src : safe, g);
     src += step;
   }
 }
@@ -102,13 +108,13 @@ __device__ __forceinline__ void fetch_cols(const char* src, int64_t step, const 
 template <int NROW>
 __device__ __forceinline__ void fetch_chunk(const ZOp& o, int64_t k, int W, bool is_b, int t, int g0, int glim,
                                             int c, double2* raw) {
-  constexpr int RS = NROW / 8;
-  const int rr = t >> 4, rq = t & 15;              // row-wise: first row, inner index
+  constexpr int RS = NROW / 4;
+  const int rr = t >> 3, rq = t & 7;               // row-wise: first row, inner index
   const int cr = t % NROW, cq = t / NROW;          // column-wise: row, first inner index
-  double2* rdst = raw + (rq & 7) * RAW_PITCH + rr + NROW * (rq >> 3);
+  double2* rdst = raw + rq * RAW_PITCH + rr;
   char* cdst = reinterpret_cast<char*>(raw + cq * RAW_PITCH + cr);
   const int left = glim - g0 - rr;                 // rows from rr on that exist
-  const unsigned mask = left <= 0 ? 0u : left > 7 * RS ? 0xFFu : (1u << ((left + RS - 1) / RS)) - 1u;
+  const unsigned mask = left <= 0 ? 0u : left > 3 * RS ? 0xFu : (1u << ((left + RS - 1) / RS)) - 1u;
   const bool ron = c * CH + rq < W;
   const int nq = g0 + cr < glim ? W - c * CH - cq : 0;
   if (o.kind == 2) {   // packed Hermitian rows: (P(r, q), P(q, r))
@@ -116,8 +122,8 @@ __device__ __forceinline__ void fetch_chunk(const ZOp& o, int64_t k, int W, bool
     const char* safe = reinterpret_cast<const char*>(P);
     fetch_rows<8, RS>(reinterpret_cast<const char*>(P + (int64_t)(g0 + rr) * W + c * CH + rq), (int64_t)RS * W * 8,
                       safe, rdst, mask, ron);
-    fetch_cols<8, NROW>(reinterpret_cast<const char*>(P + (int64_t)(c * CH + cq) * W + g0 + cr), (int64_t)2 * W * 8,
-                        safe, cdst + 8, nq);
+    fetch_cols<8>(reinterpret_cast<const char*>(P + (int64_t)(c * CH + cq) * W + g0 + cr), (int64_t)2 * W * 8,
+                  safe, cdst + 8, nq);
     return;
   }
   // A: (r, q) of the matrix or, conjugated, (q, r); B: (q, r) or, conjugated, (r, q)
@@ -127,7 +133,7 @@ __device__ __forceinline__ void fetch_chunk(const ZOp& o, int64_t k, int W, bool
     fetch_rows<16, RS>(reinterpret_cast<const char*>(P + (int64_t)(g0 + rr) * W + c * CH + rq),
                        (int64_t)RS * W * 16, safe, rdst, mask, ron);
   else
-    fetch_cols<16, NROW>(reinterpret_cast<const char*>(P + (int64_t)(c * CH + cq) * W + g0 + cr),
+    fetch_cols<16>(reinterpret_cast<const char*>(P + (int64_t)(c * CH + cq) * W + g0 + cr),
                          (int64_t)2 * W * 16, safe, cdst, nq);
 }
 // round(x 2^(55 - e)) for |x| <= 2^e with e2 = e + 1030 and e above -900 (zeros and subnormals are then
@@ -140,27 +146,40 @@ __device__ __forceinline__ long long fixed55_mid(double x, int e2) {
   const long long sg = (long long)((int)hi >> 31);
   return (q ^ sg) - sg;
 }
-// a thread's eight fetched entries (row gr, inner indices q0 ..) as fixed-point parts (55 fractional
-// bits below 2^e)
-__device__ __forceinline__ void take8(const double2* slot, int kind, int gr, int q0, int e,
-                                      long long (&re)[8], long long (&im)[8]) {
-  const bool mid = e > -900;   // (the same for all threads of an operand)
+// the real (part 0) or imaginary parts of eight fetched entries (row gr, inner indices q0 ..) in fixed point
+// (55 fractional bits below 2^e)
+__device__ __forceinline__ void take8(const double* slot, int kind, int part, int gr, int q0, int e,
+                                      long long (&v)[8]) {
+  double x[8];
+  if (kind == 2) {   // Hermitian, (a, b) = packed (r, q) and (q, r): Re is the one above the diagonal
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    double2 v = slot[i * RAW_PITCH];
-    // Hermitian: (a, b) = packed (r, q) and (q, r); Re is the one above the diagonal
-    if (kind == 2) v = gr < q0 + i ? v : gr > q0 + i ? make_double2(v.y, -v.x) : make_double2(v.x, 0.0);
-    if (kind == 1) v.y = __hiloint2double(__double2hiint(v.y) ^ (int)0x80000000, __double2loint(v.y));
-    re[i] = mid ? fixed55_mid(v.x, e + 1030) : fixed55(v.x, e);
-    im[i] = mid ? fixed55_mid(v.y, e + 1030) : fixed55(v.y, e);
+    for (int i = 0; i < 8; ++i) {
+      const int d = gr - q0 - i;
+      x[i] = slot[2 * i * RAW_PITCH + (d > 0 ? 1 - part : part)];
+      if (part) x[i] = d == 0 ? 0.0 : d > 0 ? -x[i] : x[i];
+    }
+  } else {
+    const int conj = kind == 1 && part ? (int)0x80000000 : 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      x[i] = slot[2 * i * RAW_PITCH + part];
+      x[i] = __hiloint2double(__double2hiint(x[i]) ^ conj, __double2loint(x[i]));
+    }
+  }
+  if (e > -900) {   // (the same for all threads of an operand)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = fixed55_mid(x[i], e + 1030);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = fixed55(x[i], e);
   }
 }
 
 // the seven digit slices of 8 values at 16-byte unit u of a row; TWO: also at unit u2 of a second row,
-// NEG with the opposite sign
-template <bool TWO, bool NEG>
+// with the sign bits flipped by neg
+template <bool TWO>
 __device__ __forceinline__ void put8(const long long (&q)[8], unsigned char* row, int u, unsigned char* row2,
-                                     int u2, int sw, int slice_bytes) {
+                                     int u2, uint32_t neg, int sw, int slice_bytes) {
   uint32_t d[4][ND];
 #pragma unroll
   for (int i = 0; i < 4; ++i) digits7_h2(q[2 * i], q[2 * i + 1], d[i]);
@@ -169,8 +188,7 @@ __device__ __forceinline__ void put8(const long long (&q)[8], unsigned char* row
     *reinterpret_cast<uint4*>(row + s * slice_bytes + ((u ^ sw) << 4)) = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
     if (TWO)
       *reinterpret_cast<uint4*>(row2 + s * slice_bytes + ((u2 ^ sw) << 4)) =
-          NEG ? make_uint4(h2_sub(0u, d[0][s]), h2_sub(0u, d[1][s]), h2_sub(0u, d[2][s]), h2_sub(0u, d[3][s]))
-              : make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
+          make_uint4(d[0][s] ^ neg, d[1][s] ^ neg, d[2][s] ^ neg, d[3][s] ^ neg);
   }
 }
 
@@ -215,30 +233,31 @@ __global__ void __launch_bounds__(THREADS, 1)
                       int nrt, int rr, int upper, int accum, DevStatus* st) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full[2], empty[2], acc_full, acc_empty, done_bar;
+  __shared__ __align__(8) uint64_t full[NSLOT], empty[NSLOT], acc_full, acc_empty, done_bar;
   __shared__ uint32_t tmem_base_sh;
-  __shared__ volatile int abort_sh, leave_sh, leave_epi_sh;
+  __shared__ volatile int abort_sh, leave_sh[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int B_SLICE = NCP * ROW_BYTES;
   unsigned char* sA = base;
   unsigned char* sB = sA + ND * A_SLICE;
   double2* raw0 = reinterpret_cast<double2*>(sB + ND * B_SLICE);
-  double2* slab = raw0 + 8 * RAW_PITCH;   // [64 rows][SLAB + 1]: a slab of output columns
+  double2* slab0 = raw0 + 2 * CH * RAW_PITCH;   // per epilogue warp [16 rows][SLAB + 1]: a slab of output columns
   const int nch = (W + CH - 1) / CH;
-  const int per_k = nrt * nrt;
-  const int64_t n_tiles = (int64_t)n * per_k;
+  // tile id: k-point, then row and column tile (nrt = 1 or 2 of them)
+  const int lg = nrt - 1, n_tiles = n << (2 * lg);
+  auto row_of = [&](int id) { return (id >> lg) & lg; };
+  auto col_of = [&](int id) { return id & lg; };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 2; ++s) { mbar_init(&full[s], STAGE_THREADS); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < NSLOT; ++s) { mbar_init(&full[s], STAGE_THREADS / 2); mbar_init(&empty[s], 1); }
     mbar_init(&acc_full, 1);
     mbar_init(&acc_empty, EPI_THREADS);
     mbar_init(&done_bar, 1);
     abort_sh = 0;
-    leave_sh = 0;
-    leave_epi_sh = 0;
+    leave_sh[0] = leave_sh[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 8) {
+  if (warp == MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_base_sh)),
                  "r"(TMEM_COLS)
@@ -249,31 +268,41 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
-  auto skip = [&](int in) { return upper && in / nrt > in % nrt; };
+  auto skip = [&](int id) { return upper && row_of(id) > col_of(id); };
 
-  if (warp < 8) {
-    // ---------------- staging: threads 0-127 a row of A and half a chunk, 128-255 a column of B
-    const bool is_b = threadIdx.x >= 128;
+  if (warp < STAGE_THREADS / 32) {
+    // ---------------- staging: two groups of 256 threads, chunks g = group, group + 2, ... of the CTA's
+    // sequence; in a group, threads 0-127 the real or imaginary parts of a row of A, 128-255 of a
+    // column of B
+    const int grp = threadIdx.x >> 8;
+    const bool is_b = (threadIdx.x & 128) != 0;
     const int t = threadIdx.x & 127;
-    const int nrow = is_b ? NCP : 64, nthr = is_b ? 2 * NCP : 128;
-    const int r = is_b ? t % NCP : t & 63, qg = is_b ? t / NCP : t >> 6;
-    const bool active = t < nthr;
+    const int nrow = is_b ? NCP : 64;
+    const int r = is_b ? t % NCP : t & 63, part = is_b ? t / NCP : t >> 6;
+    const bool active = t < 2 * nrow;
     const int sw = r & 7;
-    unsigned char* rowp = (is_b ? sB : sA) + r * ROW_BYTES;
-    double2* raw = raw0 + (is_b ? 128 : 0);
+    // row of A: [re; im] in blocks of 16 (an epilogue warp's 32 lanes hold both parts of 16 rows)
+    unsigned char* rowp = is_b ? sB + r * ROW_BYTES : sA + (32 * (r >> 4) + (r & 15)) * ROW_BYTES;
+    double2* raw = raw0 + grp * CH * RAW_PITCH + (is_b ? 64 : 0);
     const ZOp& O = is_b ? B : A;
-    int g = 0;
+    auto sync = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + grp) : "memory"); };
     bool ok = true;
     // the chunk being fetched: tile id, its matrix, the operand's first row there, exponent
-    int64_t id = blockIdx.x, k = 0;
+    int id = blockIdx.x, k = 0;
     int g0 = 0, e = 0, c = 0;
     auto enter = [&]() {   // the next tile to be worked on, from id on
-      while (id < n_tiles && skip((int)(id % per_k))) id += gridDim.x;
+      while (id < n_tiles && skip(id)) id += gridDim.x;
       if (id >= n_tiles) return;
-      k = id / per_k;
-      const int in = (int)(id - k * per_k);
-      g0 = (is_b ? in % nrt : in / nrt) * rr;
+      k = id >> (2 * lg);
+      g0 = (is_b ? col_of(id) : row_of(id)) * rr;
       e = op_exp(O, k);
+    };
+    auto advance = [&]() {
+      if (id < n_tiles && ++c == nch) {
+        c = 0;
+        id += gridDim.x;
+        enter();
+      }
     };
     auto fetch = [&]() {
       if (id < n_tiles && active) {
@@ -283,130 +312,131 @@ __global__ void __launch_bounds__(THREADS, 1)
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
     enter();
+    if (grp) advance();
     fetch();
-    while (id < n_tiles) {
-      const int h = g & 1;
-      long long re[8], im[8];
+    for (int g = grp; id < n_tiles; g += 2) {
+      const int h = g & (NSLOT - 1);
+      long long v[8];
       asm volatile("cp.async.wait_group 0;" ::: "memory");
-      asm volatile("bar.sync 1, 256;" ::: "memory");   // the chunk is complete
+      sync();   // the chunk is complete
       const bool stop = abort_sh != 0;
-      if (active) take8(raw + r + nrow * qg, O.kind, g0 + r, c * CH + 8 * qg, e, re, im);
-      if (stop) leave_sh = 1;
-      asm volatile("bar.sync 1, 256;" ::: "memory");   // its slots may be overwritten
-      if (leave_sh) break;                             // (all of them, after a timeout anywhere)
-      if (++c == nch) {
-        c = 0;
-        id += gridDim.x;
-        enter();
-      }
+      if (active) take8(reinterpret_cast<const double*>(raw + r), O.kind, part, g0 + r, c * CH, e, v);
+      if (stop) leave_sh[grp] = 1;
+      sync();                      // its slots may be overwritten
+      if (leave_sh[grp]) break;    // (all of the group, after a timeout anywhere)
+      advance();
+      advance();
       fetch();
-      if (g >= 2 && !mbar_wait(&empty[h], ((uint32_t)(g >> 1) & 1u) ^ 1u)) {
+      if (g >= NSLOT && !mbar_wait(&empty[h], ((uint32_t)(g / NSLOT) & 1u) ^ 1u)) {
         atomicOr(&st->bits, ST_TIMEOUT);   // (go on: every warp passes the same barriers)
         abort_sh = 1;
         ok = false;
       }
       if (active && ok) {
-        const int u = 4 * h + qg;
         if (is_b) {
-          put8<false, false>(re, rowp, u, rowp, u, sw, B_SLICE);
-          put8<false, false>(im, rowp, u + 2, rowp, u, sw, B_SLICE);
+          put8<false>(v, rowp, 2 * h + part, rowp, 0, 0u, sw, B_SLICE);
         } else {   // real rows [Ar | -Ai], imaginary rows [Ai | Ar]
-          unsigned char* rowi = rowp + 64 * ROW_BYTES;
-          put8<true, false>(re, rowp, u, rowi, u + 2, sw, A_SLICE);
-          put8<true, true>(im, rowi, u, rowp, u + 2, sw, A_SLICE);
+          unsigned char* rowi = rowp + 16 * ROW_BYTES;
+          put8<true>(v, part ? rowi : rowp, 2 * h, part ? rowp : rowi, 2 * h + 1, part ? 0x80008000u : 0u, sw, A_SLICE);
         }
       }
       fence_proxy_async_smem();
       mbar_arrive(&full[h]);
-      ++g;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-  } else {
-    // ---------------- epilogue: warp w reads TMEM lanes 32 (w % 4) .. and, per slab of 16 columns, 8 of
-    // them.  Warp 8 also issues the MMAs of a drain group, which cannot overlap a drain (the levels
-    // fill TMEM).
-    int g = 0;
-    auto issue = [&](int nc, int G) -> bool {
-      if (abort_sh || (G >= 1 && !mbar_wait(&acc_empty, (uint32_t)(G - 1) & 1u))) return false;
+  } else if (warp == MMA_WARP) {
+    // ---------------- the MMAs, from one lane; a drain group waits for the drain before it (the levels
+    // fill TMEM)
+    if (lane == 0) {
       const uint32_t a0 = ((smem_u32(sA) & 0x3FFFFu) >> 4) | (1u << 16);
       const uint32_t b0 = ((smem_u32(sB) & 0x3FFFFu) >> 4) | (1u << 16);
+      bool ok = true;
+      int g = 0, G = 0;
+      for (int id = blockIdx.x; id < n_tiles && ok; id += gridDim.x) {
+        if (skip(id)) continue;
+        for (int gi = 0; gi * GROUP < nch && ok; ++gi, ++G) {
+          const int nc = min(GROUP, nch - gi * GROUP);
+          ok = !abort_sh && (G == 0 || mbar_wait(&acc_empty, (uint32_t)(G - 1) & 1u));
+          tc_fence_after();
 #pragma unroll 1
-      for (int c = 0; c < nc; ++c, ++g) {
-        const uint32_t off = (uint32_t)(g & 1) * 4u;   // (64 bytes: the chunk's half of a row)
-        if (abort_sh || !mbar_wait(&full[g & 1], (uint32_t)(g >> 1) & 1u)) return false;
-        tc_fence_after();
-        if (c == 0) mma_step<NCP, true>(tmem, a0 + off, b0 + off);
-        else mma_step<NCP, false>(tmem, a0 + off, b0 + off);
-        mma_step<NCP, false>(tmem, a0 + off + 2, b0 + off + 2);
-        umma_commit(&empty[g & 1]);
+          for (int c = 0; c < nc && ok; ++c, ++g) {
+            const int h = g & (NSLOT - 1);
+            const uint32_t off = (uint32_t)h * 2u;   // (32 bytes: the chunk's quarter of a row)
+            ok = !abort_sh && mbar_wait(&full[h], (uint32_t)(g / NSLOT) & 1u);
+            if (!ok) break;
+            tc_fence_after();
+            if (c == 0) mma_step<NCP, true>(tmem, a0 + off, b0 + off);
+            else mma_step<NCP, false>(tmem, a0 + off, b0 + off);
+            umma_commit(&empty[h]);
+          }
+          if (ok) umma_commit(&acc_full);
+        }
       }
-      umma_commit(&acc_full);
-      return true;
-    };
-    const int quarter = warp & 3;
-    const int row = quarter * 32 + lane, cr = row & 63;
-    const int part = row >> 6;   // 0: real part, 1: imaginary part
-    const int half = (warp - 8) >> 2;
-    const int et = threadIdx.x - STAGE_THREADS;
+      if (!ok) {
+        atomicOr(&st->bits, ST_TIMEOUT);
+        abort_sh = 1;
+      }
+      umma_commit(&done_bar);   // all issued MMAs complete
+    }
+    __syncwarp();
+  } else {
+    // ---------------- epilogue: warp w reads the TMEM lanes 32 (w % 4) .., both parts of 16 complex rows,
+    // and every other slab of 8 columns, and writes it through shared memory of its own
+    const int quarter = warp & 3, half = (warp - STAGE_THREADS / 32) >> 2;
+    const int wr = lane >> 3, wc = lane & 7;   // writes rows wr + 4 q of a slab's column wc
+    double2* slab = slab0 + (warp - STAGE_THREADS / 32) * 16 * (SLAB + 1);
+    double* mine = reinterpret_cast<double*>(slab + (lane & 15) * (SLAB + 1)) + (lane >> 4);
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
     bool ok = true;
     int G = 0;
-    for (int64_t id = blockIdx.x; id < n_tiles && ok; id += gridDim.x) {
-      const int64_t k = id / per_k;
-      const int in = (int)(id - k * per_k);
-      if (skip(in)) continue;
-      const int r0 = (in / nrt) * rr, c0 = (in % nrt) * rr;
+    for (int id = blockIdx.x; id < n_tiles && ok; id += gridDim.x) {
+      const int64_t k = id >> (2 * lg);
+      if (skip(id)) continue;
+      const int r0 = row_of(id) * rr + 16 * quarter, c0 = col_of(id) * rr;
       const int ea = op_exp(A, k), eb = op_exp(B, k);
       const bool bad = ea >= ZEXP_BAD || eb >= ZEXP_BAD;
       const int es = bad ? 0 : ea + eb - 55;
-      const int nrow = min(rr, W - r0), ncol = min(rr, W - c0);
-      double2* Ck = C + k * (int64_t)W * W + (int64_t)r0 * W + c0;
+      const int nrow = min(rr - 16 * quarter, W - r0) - wr, ncol = min(rr, W - c0) - wc;
+      double2* Ck = C + k * (int64_t)W * W + (int64_t)(r0 + wr) * W + c0 + wc;
       unsigned mx = 0u;
       for (int gi = 0; gi * GROUP < nch; ++gi, ++G) {
-        if (warp == 8) {
-          if (lane == 0) ok = issue(min(GROUP, nch - gi * GROUP), G);
-          __syncwarp();
-        }
-        ok = ok && mbar_wait(&acc_full, (uint32_t)G & 1u);
+        ok = mbar_wait(&acc_full, (uint32_t)G & 1u);
         ok = __all_sync(0xffffffffu, ok && !abort_sh);   // tcgen05.ld is warp-collective
-        if (!ok) leave_epi_sh = 1;
-        asm volatile("bar.sync 2, 256;" ::: "memory");
-        if (leave_epi_sh) ok = false;
-        asm volatile("bar.sync 2, 256;" ::: "memory");   // (every epilogue warp leaves together)
         if (!ok) break;
         tc_fence_after();
         const bool add = accum || gi > 0, final_group = (gi + 1) * GROUP >= nch;
 #pragma unroll 1
-        for (int s0 = 0; s0 < NCP; s0 += SLAB) {
-          uint32_t x[NLEV][8];
+        for (int s0 = half * SLAB; s0 < NCP; s0 += 2 * SLAB) {
 #pragma unroll
-          for (int l = 0; l < NLEV; ++l) tmem_ld8_async(lane_addr + (uint32_t)(l * NCP + s0 + 8 * half), x[l]);
+          for (int b = 0; b < 2; ++b) {
+            uint32_t x[NLEV][4];
 #pragma unroll
-          for (int l = 0; l < NLEV; ++l) tmem_wait_ld8(x[l]);
-          if (s0 + SLAB >= NCP) {   // the thread's last TMEM read of this drain
-            tc_fence_before();
-            mbar_arrive(&acc_empty);
+            for (int l = 0; l < NLEV; ++l) tmem_ld4_async(lane_addr + (uint32_t)(l * NCP + s0 + 4 * b), x[l]);
+#pragma unroll
+            for (int l = 0; l < NLEV; ++l) tmem_wait_ld4(x[l]);
+            if (b == 1 && s0 + 2 * SLAB >= NCP) {   // the thread's last TMEM read of this drain
+              tc_fence_before();
+              mbar_arrive(&acc_empty);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              int I[NLEV];
+#pragma unroll
+              for (int l = 0; l < NLEV; ++l) I[l] = __float2int_rn(__uint_as_float(x[l][j]));
+              // sum_l I_l 2^(41 - 8 l), the levels 6 and 7 rounded to the unit 2^-55
+              const long long hi = (long long)I[0] * 65536 + ((long long)I[1] * 256 + I[2]);
+              const long long lo = (long long)I[3] * 65536 + ((long long)I[4] * 256 + I[5]);
+              const long long v = (hi << 25) + (lo << 1) + (((long long)I[6] * 256 + (I[7] + 16384)) >> 15);
+              mine[2 * (4 * b + j)] = bad ? __longlong_as_double(0x7FF8000000000000ll) : scaled_double(v, es);
+            }
           }
+          __syncwarp();
+          // the slab to global memory, 8 columns (128 bytes) of a row by 8 lanes
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            int I[NLEV];
-#pragma unroll
-            for (int l = 0; l < NLEV; ++l) I[l] = __float2int_rn(__uint_as_float(x[l][j]));
-            // sum_l I_l 2^(41 - 8 l), the levels 6 and 7 rounded to the unit 2^-55
-            const long long hi = (long long)I[0] * 65536 + ((long long)I[1] * 256 + I[2]);
-            const long long lo = (long long)I[3] * 65536 + ((long long)I[4] * 256 + I[5]);
-            const long long v = (hi << 25) + (lo << 1) + (((long long)I[6] * 256 + (I[7] + 16384)) >> 15);
-            reinterpret_cast<double*>(slab + cr * (SLAB + 1) + 8 * half + j)[part] =
-                bad ? __longlong_as_double(0x7FF8000000000000ll) : scaled_double(v, es);
-          }
-          asm volatile("bar.sync 2, 256;" ::: "memory");
-          // the slab to global memory, 16 columns (256 bytes) of a row by 16 lanes
-#pragma unroll
-          for (int q = 0; q < 64 * SLAB / EPI_THREADS; ++q) {
-            const int rw = (et >> 4) + q * (EPI_THREADS / SLAB), cl = et & 15;
-            if (rw < nrow && s0 + cl < ncol) {
-              double2 v = slab[rw * (SLAB + 1) + cl];
-              double2* dst = Ck + (int64_t)rw * W + s0 + cl;
+          for (int q = 0; q < 4; ++q)
+            if (4 * q < nrow && s0 < ncol) {
+              double2* dst = Ck + (int64_t)(4 * q) * W + s0;
+              double2 v = slab[(wr + 4 * q) * (SLAB + 1) + wc];
               if (add) {
                 const double2 o = *dst;
                 v.x += o.x;
@@ -415,8 +445,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               *dst = v;
               if (final_group) mx = max(mx, (unsigned)(max(mag_bits(v.x), mag_bits(v.y)) >> 32));
             }
-          }
-          asm volatile("bar.sync 2, 256;" ::: "memory");
+          __syncwarp();
         }
       }
       if (ec && ok) {
@@ -429,11 +458,10 @@ __global__ void __launch_bounds__(THREADS, 1)
       atomicOr(&st->bits, ST_TIMEOUT);
       abort_sh = 1;
     }
-    if (warp == 8 && lane == 0) umma_commit(&done_bar);   // all issued MMAs complete
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
+  if (warp == MMA_WARP) {
     if (lane == 0) mbar_wait(&done_bar, 0);
     __syncwarp();
     tc_fence_after();
@@ -543,7 +571,7 @@ cudaError_t launch_zgemm_tc64(const ZOp& A, const ZOp& B, double2* C, int* ec, i
   const int nt = (W + 63) / 64, rr = (W + nt - 1) / nt;
   const int ncp = (rr + 15) / 16 * 16;
   const size_t sm = (size_t)ND * A_SLICE + (size_t)ND * ncp * ROW_BYTES +
-                    ((size_t)8 * RAW_PITCH + 64 * (SLAB + 1)) * sizeof(double2) + 1024;
+                    ((size_t)2 * CH * RAW_PITCH + EPI_THREADS / 2 * (SLAB + 1)) * sizeof(double2) + 1024;
   int dev = 0, nsm = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   auto go = [&](auto kern) -> cudaError_t {

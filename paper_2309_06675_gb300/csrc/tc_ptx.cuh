@@ -178,6 +178,11 @@ __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* r) {
                  "=r"(r[7])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld4_async(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
 // completes the thread's outstanding TMEM loads; the loaded registers pass through so that no
 // use of them is scheduled before it
 __device__ __forceinline__ void tmem_wait_ld8(uint32_t* r) {
@@ -186,6 +191,9 @@ __device__ __forceinline__ void tmem_wait_ld8(uint32_t* r) {
                  "+r"(r[7])
                :
                : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld4(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
 }
 
 // 32 lanes x 16 consecutive 32-bit columns, registers -> TMEM
