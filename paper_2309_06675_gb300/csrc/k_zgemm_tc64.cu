@@ -83,15 +83,16 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src, bool on) {
                "r"(on ? BYTES : 0)
                : "memory");
 }
-// lanes along the inner index: rows (t / 8) + RS i, index t % 8; mask: rows inside the matrix
+// lanes along the inner index: rows (t / 8) + RS i, index t % 8; mask: rows inside the matrix; the steps
+// after an even and after an odd row
 template <int BYTES, int RS>
-__device__ __forceinline__ void fetch_rows(const char* src, int64_t step, const char* safe, double2* dst,
-                                           unsigned mask, bool on) {
+__device__ __forceinline__ void fetch_rows(const char* src, int64_t step0, int64_t step1, const char* safe,
+                                           double2* dst, unsigned mask, bool on) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const bool g = on && ((mask >> i) & 1u);
     cp_async<BYTES>(dst + i * RS, g ? src : safe, g);
-    src += step;
+    src += i & 1 ? step1 : step0;
   }
 }
 // lanes along the rows: row t % nrow, inner indices (t / nrow) + 2 i, nq of them inside the matrix
@@ -104,7 +105,9 @@ __device__ __forceinline__ void fetch_cols(const char* src, int64_t step, const 
     src += step;
   }
 }
-// chunk c of rows (columns) g0 .. glim - 1 of an operand, NROW of them per tile, by 2 NROW threads
+// chunk c of rows (columns) g0 .. glim - 1 of an operand, NROW of them per tile, by 2 NROW threads.  Sources:
+// A (r, q) of the matrix or, conjugated, (q, r); B (q, r) or, conjugated, (r, q); packed Hermitian rows (kind 2)
+// P(r, q) and P(q, r)
 template <int NROW>
 __device__ __forceinline__ void fetch_chunk(const ZOp& o, int64_t k, int W, bool is_b, int t, int g0, int glim,
                                             int c, double2* raw) {
@@ -117,24 +120,55 @@ __device__ __forceinline__ void fetch_chunk(const ZOp& o, int64_t k, int W, bool
   const unsigned mask = left <= 0 ? 0u : left > 3 * RS ? 0xFu : (1u << ((left + RS - 1) / RS)) - 1u;
   const bool ron = c * CH + rq < W;
   const int nq = g0 + cr < glim ? W - c * CH - cq : 0;
-  if (o.kind == 2) {   // packed Hermitian rows: (P(r, q), P(q, r))
+  if (o.kind == 2) {
     const double* P = reinterpret_cast<const double*>(o.p) + k * o.ld;
     const char* safe = reinterpret_cast<const char*>(P);
-    fetch_rows<8, RS>(reinterpret_cast<const char*>(P + (int64_t)(g0 + rr) * W + c * CH + rq), (int64_t)RS * W * 8,
-                      safe, rdst, mask, ron);
+    const int64_t step = (int64_t)RS * W * 8;
+    fetch_rows<8, RS>(reinterpret_cast<const char*>(P + (int64_t)(g0 + rr) * W + c * CH + rq), step, step, safe,
+                      rdst, mask, ron);
     fetch_cols<8>(reinterpret_cast<const char*>(P + (int64_t)(c * CH + cq) * W + g0 + cr), (int64_t)2 * W * 8,
                   safe, cdst + 8, nq);
     return;
   }
-  // A: (r, q) of the matrix or, conjugated, (q, r); B: (q, r) or, conjugated, (r, q)
   const double2* P = reinterpret_cast<const double2*>(o.p) + k * (int64_t)W * W;
   const char* safe = reinterpret_cast<const char*>(P);
+  const int64_t step = (int64_t)RS * W * 16;
   if ((o.kind == 0) != is_b)
-    fetch_rows<16, RS>(reinterpret_cast<const char*>(P + (int64_t)(g0 + rr) * W + c * CH + rq),
-                       (int64_t)RS * W * 16, safe, rdst, mask, ron);
+    fetch_rows<16, RS>(reinterpret_cast<const char*>(P + (int64_t)(g0 + rr) * W + c * CH + rq), step, step, safe,
+                       rdst, mask, ron);
   else
-    fetch_cols<16>(reinterpret_cast<const char*>(P + (int64_t)(c * CH + cq) * W + g0 + cr),
-                         (int64_t)2 * W * 16, safe, cdst, nq);
+    fetch_cols<16>(reinterpret_cast<const char*>(P + (int64_t)(c * CH + cq) * W + g0 + cr), (int64_t)2 * W * 16,
+                   safe, cdst, nq);
+}
+// the same for a tile of P matrices k .. k + P - 1 (below n), 64 / P of its rows (columns) each
+template <int P>
+__device__ __forceinline__ void fetch_chunk_packed(const ZOp& o, int64_t k, int n, int W, bool is_b, int t, int c,
+                                                   double2* raw) {
+  constexpr int RS = 16, SUB = 64 / P;
+  const int rr = t >> 3, rq = t & 7, cr = t & 63, cq = t >> 6;
+  const int csub = cr / SUB, cl = cr % SUB;
+  const int left = (int)min((int64_t)P, n - k);    // matrices of the tile that exist
+  unsigned mask = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) mask |= ((rr + RS * i) % SUB < W && (rr + RS * i) / SUB < left ? 1u : 0u) << i;
+  const bool ron = c * CH + rq < W;
+  const int nq = cl < W && csub < left ? W - c * CH - cq : 0;
+  const int64_t bytes = o.kind == 2 ? 8 : 16, mat = o.kind == 2 ? o.ld * 8 : (int64_t)W * W * 16;
+  const int64_t rows = (int64_t)RS * W * bytes;
+  const int64_t s0 = P == 4 ? mat : rows, s1 = P == 4 ? mat : mat - rows;
+  const char* base = reinterpret_cast<const char*>(o.p) + k * mat;
+  const char* rsrc = base + ((int64_t)rr * W + c * CH + rq) * bytes;
+  const char* csrc = base + csub * mat + ((int64_t)(c * CH + cq) * W + cl) * bytes;
+  double2* rdst = raw + rq * RAW_PITCH + rr;
+  char* cdst = reinterpret_cast<char*>(raw + cq * RAW_PITCH + cr);
+  if (o.kind == 2) {
+    fetch_rows<8, RS>(rsrc, s0, s1, base, rdst, mask, ron);
+    fetch_cols<8>(csrc, (int64_t)2 * W * 8, base, cdst + 8, nq);
+  } else if ((o.kind == 0) != is_b) {
+    fetch_rows<16, RS>(rsrc, s0, s1, base, rdst, mask, ron);
+  } else {
+    fetch_cols<16>(csrc, (int64_t)2 * W * 16, base, cdst, nq);
+  }
 }
 // round(x 2^(55 - e)) for |x| <= 2^e with e2 = e + 1030 and e above -900 (zeros and subnormals are then
 // far below the unit): the general form without its case distinctions
@@ -226,8 +260,9 @@ __device__ __forceinline__ void mma_step(uint32_t tmem, uint32_t alo, uint32_t b
 }
 
 // NCP: columns per tile; nrt, nct row and column tiles of rr rows and columns.  upper: tiles strictly
-// below the diagonal are left out.
-template <int NCP>
+// below the diagonal are left out.  P > 1 (NCP = 64): P matrices of up to 64 / P rows share a tile, whose P
+// diagonal blocks are drained.
+template <int NCP, int P>
 __global__ void __launch_bounds__(THREADS, 1)
     zgemm_tc64_kernel(ZOp A, ZOp B, double2* __restrict__ C, int* __restrict__ ec, int W, int n,
                       int nrt, int rr, int upper, int accum, DevStatus* st) {
@@ -244,7 +279,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   double2* slab0 = raw0 + 2 * CH * RAW_PITCH;   // per epilogue warp [16 rows][SLAB + 1]: a slab of output columns
   const int nch = (W + CH - 1) / CH;
   // tile id: k-point, then row and column tile (nrt = 1 or 2 of them)
-  const int lg = nrt - 1, n_tiles = n << (2 * lg);
+  const int lg = nrt - 1, n_tiles = P == 1 ? n << (2 * lg) : (n + P - 1) / P;
+  constexpr int SUB = 64 / P, DRAIN_COLS = P == 1 ? NCP : SUB;
   auto row_of = [&](int id) { return (id >> lg) & lg; };
   auto col_of = [&](int id) { return id & lg; };
 
@@ -288,14 +324,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     auto sync = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + grp) : "memory"); };
     bool ok = true;
     // the chunk being fetched: tile id, its matrix, the operand's first row there, exponent
+    const int sub = P == 1 ? 0 : r / SUB, rl = P == 1 ? r : r % SUB;   // matrix of the tile, row in it
     int id = blockIdx.x, k = 0;
     int g0 = 0, e = 0, c = 0;
     auto enter = [&]() {   // the next tile to be worked on, from id on
       while (id < n_tiles && skip(id)) id += gridDim.x;
       if (id >= n_tiles) return;
-      k = id >> (2 * lg);
+      k = (id >> (2 * lg)) * P;
       g0 = (is_b ? col_of(id) : row_of(id)) * rr;
-      e = op_exp(O, k);
+      e = op_exp(O, P == 1 ? k : min(k + sub, n - 1));
     };
     auto advance = [&]() {
       if (id < n_tiles && ++c == nch) {
@@ -306,7 +343,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     };
     auto fetch = [&]() {
       if (id < n_tiles && active) {
-        if (is_b) fetch_chunk<NCP>(O, k, W, true, t, g0, min(W, g0 + rr), c, raw);
+        if constexpr (P > 1) fetch_chunk_packed<P>(O, k, n, W, is_b, t, c, raw);
+        else if (is_b) fetch_chunk<NCP>(O, k, W, true, t, g0, min(W, g0 + rr), c, raw);
         else fetch_chunk<64>(O, k, W, false, t, g0, min(W, g0 + rr), c, raw);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -320,7 +358,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       sync();   // the chunk is complete
       const bool stop = abort_sh != 0;
-      if (active) take8(reinterpret_cast<const double*>(raw + r), O.kind, part, g0 + r, c * CH, e, v);
+      if (active) take8(reinterpret_cast<const double*>(raw + r), O.kind, part, g0 + rl, c * CH, e, v);
       if (stop) leave_sh[grp] = 1;
       sync();                      // its slots may be overwritten
       if (leave_sh[grp]) break;    // (all of the group, after a timeout anywhere)
@@ -386,17 +424,20 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int wr = lane >> 3, wc = lane & 7;   // writes rows wr + 4 q of a slab's column wc
     double2* slab = slab0 + (warp - STAGE_THREADS / 32) * 16 * (SLAB + 1);
     double* mine = reinterpret_cast<double*>(slab + (lane & 15) * (SLAB + 1)) + (lane >> 4);
-    const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
+    const int sub = P == 1 ? 0 : 16 * quarter / SUB;                  // matrix of the tile
+    const int ro = P == 1 ? 16 * quarter : (16 * quarter) % SUB;      // row in it
+    const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(sub * SUB);
     bool ok = true;
     int G = 0;
     for (int id = blockIdx.x; id < n_tiles && ok; id += gridDim.x) {
-      const int64_t k = id >> (2 * lg);
       if (skip(id)) continue;
-      const int r0 = row_of(id) * rr + 16 * quarter, c0 = col_of(id) * rr;
+      const int k1 = (id >> (2 * lg)) * P + sub;
+      const int64_t k = P == 1 ? k1 : min(k1, n - 1);
+      const int r0 = row_of(id) * rr + ro, c0 = col_of(id) * rr;
       const int ea = op_exp(A, k), eb = op_exp(B, k);
       const bool bad = ea >= ZEXP_BAD || eb >= ZEXP_BAD;
       const int es = bad ? 0 : ea + eb - 55;
-      const int nrow = min(rr - 16 * quarter, W - r0) - wr, ncol = min(rr, W - c0) - wc;
+      const int nrow = P == 1 || k1 < n ? min(rr - ro, W - r0) - wr : 0, ncol = min(rr, W - c0) - wc;
       double2* Ck = C + k * (int64_t)W * W + (int64_t)(r0 + wr) * W + c0 + wc;
       unsigned mx = 0u;
       for (int gi = 0; gi * GROUP < nch; ++gi, ++G) {
@@ -406,7 +447,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         tc_fence_after();
         const bool add = accum || gi > 0, final_group = (gi + 1) * GROUP >= nch;
 #pragma unroll 1
-        for (int s0 = half * SLAB; s0 < NCP; s0 += 2 * SLAB) {
+        for (int s0 = half * SLAB; s0 < DRAIN_COLS; s0 += 2 * SLAB) {
 #pragma unroll
           for (int b = 0; b < 2; ++b) {
             uint32_t x[NLEV][4];
@@ -414,7 +455,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int l = 0; l < NLEV; ++l) tmem_ld4_async(lane_addr + (uint32_t)(l * NCP + s0 + 4 * b), x[l]);
 #pragma unroll
             for (int l = 0; l < NLEV; ++l) tmem_wait_ld4(x[l]);
-            if (b == 1 && s0 + 2 * SLAB >= NCP) {   // the thread's last TMEM read of this drain
+            if (b == 1 && s0 + 2 * SLAB >= DRAIN_COLS) {   // the thread's last TMEM read of this drain
               tc_fence_before();
               mbar_arrive(&acc_empty);
             }
@@ -451,7 +492,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (ec && ok) {
         for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const int ex = (int)(mx >> 20);
-        if (lane == 0) atomicMax(&ec[k], ex == 0x7FF ? ZEXP_BAD : ex - 1022);
+        if (lane == 0 && (P == 1 || k1 < n)) atomicMax(&ec[k], ex == 0x7FF ? ZEXP_BAD : ex - 1022);
       }
     }
     if (!ok) {
@@ -569,7 +610,10 @@ cudaError_t launch_zgemm_tc64(const ZOp& A, const ZOp& B, double2* C, int* ec, i
   if (W < 1 || W > LARGE_W_MAX || B.kind == 2) return cudaErrorInvalidValue;
   // even split of W into tiles of at most 64
   const int nt = (W + 63) / 64, rr = (W + nt - 1) / nt;
-  const int ncp = (rr + 15) / 16 * 16;
+  // matrices per tile: an unshared tile of W = 32 leaves half of the MMA rows empty and its chunks, loads and
+  // drain take their latencies alone (gradient at W = 32, 9,216 k-points: adjoint 7.2 ms, two to a tile 5.3)
+  const int P = W <= 16 ? 4 : W <= 32 ? 2 : 1;
+  const int ncp = rr <= 32 || rr > 48 ? 64 : 48;
   const size_t sm = (size_t)ND * A_SLICE + (size_t)ND * ncp * ROW_BYTES +
                     ((size_t)2 * CH * RAW_PITCH + EPI_THREADS / 2 * (SLAB + 1)) * sizeof(double2) + 1024;
   int dev = 0, nsm = 152;
@@ -581,17 +625,14 @@ cudaError_t launch_zgemm_tc64(const ZOp& A, const ZOp& B, double2* C, int* ec, i
       e = cudaMemsetAsync(ec, 0xC0, sizeof(int) * (size_t)n, s);   // a large negative exponent
       if (e != cudaSuccess) return e;
     }
-    const int64_t tiles = (int64_t)n * nt * nt;
+    const int64_t tiles = ((int64_t)n + P - 1) / P * nt * nt;
     kern<<<(int)std::min<int64_t>(tiles, std::max(nsm, 1)), THREADS, sm, s>>>(A, B, C, ec, W, n, nt, rr,
                                                                               upper ? 1 : 0, accum ? 1 : 0, st);
     return cudaGetLastError();
   };
-  switch (ncp) {
-    case 16: return go(zgemm_tc64_kernel<16>);
-    case 32: return go(zgemm_tc64_kernel<32>);
-    case 48: return go(zgemm_tc64_kernel<48>);
-    default: return go(zgemm_tc64_kernel<64>);
-  }
+  if (P == 4) return go(zgemm_tc64_kernel<64, 4>);
+  if (P == 2) return go(zgemm_tc64_kernel<64, 2>);
+  return ncp == 48 ? go(zgemm_tc64_kernel<48, 1>) : go(zgemm_tc64_kernel<64, 1>);
 }
 
 cudaError_t launch_curvature64(const double* E, const double2* Vx, const double2* Vy, int W, int n,

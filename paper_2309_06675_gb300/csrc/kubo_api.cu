@@ -20,8 +20,9 @@ constexpr int MAX_W = LARGE_W_MAX;
 constexpr int SMALL_W_MAX = 64;      // beyond: the multi-pass eigenvector / rotation kernels
 constexpr int MAX_ETA = 8;
 // FP64 rotations: integer-pipe kernel (one launch, k-points packed in a CTA) up to this order, tensor-
-// core products above
-constexpr int FIX_W_MAX = 32;
+// core products above.  9,216 k-points, integer pipe and tensor cores: W = 24 1.25 and 1.31 ms, W = 28 2.10 and
+// 1.47, W = 32 2.43 and 1.53 (W = 16, 13,824: 0.54 and 1.13); 19 to 304 k-points at W = 25: 0.084 and 0.080
+constexpr int FIX_W_MAX = 24;
 // k-points per sub-batch of the latter: T, v^x and v^y of a sub-batch (192 KB each at W = 64) are
 // written and read while they are in L2
 constexpr int ZG_BATCH = 152 * 8;

@@ -1,6 +1,6 @@
 """Integer-pipe products of FP64 grade (rotations, U = Q D Z) against extended precision.
 
-Orders around the tiles (2 x 2 below 13, 4 x 2 to 32, tensor-core tiles of up to 64 above; 4 reflectors
+Orders around the tiles (2 x 2 below 13, 4 x 2 to 24, tensor-core tiles of up to 64 above; 4 reflectors
 per block), magnitudes far from
 1, eigenvectors that are not normalised, non-finite operands.
 """
@@ -134,3 +134,41 @@ def test_non_finite_matrix_leaves_the_others():
     ref = np.linalg.eigvalsh(A)
     assert np.isnan(E[1]).all()
     assert np.abs(E[[0, 2]] - ref[[0, 2]]).max() <= 80 * 2.0 ** -52 * np.abs(ref).max()
+
+
+def test_non_finite_operands_in_a_shared_tile():
+    # two matrices of order 25 .. 32 to a tensor-core tile: the other one is not affected
+    import torch
+    import paper_2309_06675_gb300 as kubo
+    A, E, U = _problem(30, 5, 2)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()   # noqa: E731
+    X = kubo.pack_hermitian(d(A[1]))
+    Y = kubo.pack_hermitian(d(A[2]))
+    ref = kubo.berry_batched(d(E), d(U), X, Y, eta=0.1).cpu().numpy()[0]
+    X[1, 7] = float("inf")
+    Ud = d(U)
+    Ud[2, 3, 4] = float("nan")
+    got = kubo.berry_batched(d(E), Ud, X, Y, eta=0.1).cpu().numpy()[0]
+    assert np.array_equal(got[[0, 3, 4]], ref[[0, 3, 4]])
+    assert np.isnan(got[1]).all() and np.isnan(got[2]).all()
+
+
+@pytest.mark.parametrize("W", [1, 5, 15, 16, 17, 31, 32, 33])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 6])
+def test_gradient_of_shared_tiles(W, n):
+    # Four (W <= 16) or two (W <= 32) k-points share a tile of the gradient's products, one by itself
+    # when the range is a single k-point.  The products of a k-point are the same numbers either way;
+    # the sum over k rounds its operands to 2^-55 of the largest of the range.
+    import torch
+    import tbgen
+    import paper_2309_06675_gb300 as kubo
+    m = tbgen.random_tb(W, 1, 1.0, W)
+    H, R = torch.from_numpy(m.H_R).cuda(), torch.from_numpy(m.R)
+    E_F = torch.zeros(1, dtype=torch.float64, device="cuda")
+    g = torch.ones(1, 1, dtype=torch.float64, device="cuda")
+    run = lambda a, b: kubo.ahc_grad(H, R, (4, 3, 2), E_F, g, etas=[0.05], kT=0.1, k_range=(a, b))   # noqa: E731
+    first = lambda x: x[0] if isinstance(x, tuple) else x   # noqa: E731
+    whole = first(run(3, 3 + n)).cpu().numpy()
+    parts = sum(first(run(3 + i, 4 + i)).cpu().numpy() for i in range(n))
+    assert np.isfinite(whole).all()
+    assert np.abs(whole - parts).max() <= 1e-12 * max(np.abs(parts).max(), 1e-300)
