@@ -553,13 +553,20 @@ kubo_status check_klist(Call& c, const int64_t* kidx, int64_t n) {
 
 // Prepare the model: status reset, Hermitian check (one host sync, which also gives max |H(R)|
 // and so the range exponent of the call), twiddles, packed basis (scaled by 2^escale).
-kubo_status prepare_model(Call& c, const double* H_R, const RInfo& ri) {
+// deferred: the verdict is left in the device status, for a caller whose outputs are written on success
+// only and who reads it at the end.
+kubo_status prepare_model(Call& c, const double* H_R, const RInfo& ri, bool deferred = false) {
   Plan& p = c.p;
   KCHECK(cudaMemsetAsync(c.at<char>(p.o_status), 0, sizeof(DevStatus), c.s));
-  KCHECK(cudaMemcpyAsync(c.at<int>(p.o_neg), ri.neg.data(), sizeof(int) * p.N_R, cudaMemcpyHostToDevice, c.s));
-  if (p.N_h > 0) {
-    KCHECK(cudaMemcpyAsync(c.at<int>(p.o_pairs), ri.pairs.data(), sizeof(int) * 2 * p.N_h, cudaMemcpyHostToDevice, c.s));
-    KCHECK(cudaMemcpyAsync(c.at<int>(p.o_Rh), ri.Rh.data(), sizeof(int) * 3 * p.N_h, cudaMemcpyHostToDevice, c.s));
+  {
+    // the three tables lie one behind the other: one upload
+    std::vector<char> tabs(p.o_Rh - p.o_neg + sizeof(int) * 3 * (size_t)std::max(1, p.N_h), 0);
+    std::memcpy(tabs.data(), ri.neg.data(), sizeof(int) * p.N_R);
+    if (p.N_h > 0) {
+      std::memcpy(tabs.data() + (p.o_pairs - p.o_neg), ri.pairs.data(), sizeof(int) * 2 * p.N_h);
+      std::memcpy(tabs.data() + (p.o_Rh - p.o_neg), ri.Rh.data(), sizeof(int) * 3 * p.N_h);
+    }
+    KCHECK(cudaMemcpyAsync(c.at<char>(p.o_neg), tabs.data(), tabs.size(), cudaMemcpyHostToDevice, c.s));
   }
   DevStatus* st = c.at<DevStatus>(p.o_status);
   {
@@ -567,10 +574,13 @@ kubo_status prepare_model(Call& c, const double* H_R, const RInfo& ri) {
     KCHECK(launch_check_hermitian((const double2*)H_R, c.at<int>(p.o_neg), p.N_R, p.W, st, c.s));
     KCHECK(launch_hermitian_verdict(st, c.s));
   }
-  DevStatus h;
-  kubo_status hv = read_status(c, &h);
-  if (hv != KUBO_OK) return hv;
-  p.escale = p.scale_ok ? range_exponent(herm_max(h)) : 0;
+  p.escale = 0;
+  if (!deferred || p.scale_ok) {
+    DevStatus h;
+    kubo_status hv = read_status(c, &h);
+    if (hv != KUBO_OK) return hv;
+    if (p.scale_ok) p.escale = range_exponent(herm_max(h));
+  }
   {
     StageTimer tm(c, KUBO_STAGE_PREP, 2);
     KCHECK(launch_twiddles(c.at<double2>(p.o_tab), p.mesh.N1, p.mesh.N2, p.mesh.N3, c.s));
@@ -589,7 +599,7 @@ kubo_status prepare_model(Call& c, const double* H_R, const RInfo& ri) {
     StageTimer tm(c, KUBO_STAGE_PREP, 2);
     KCHECK(launch_basis_split64(c.at<double>(p.o_Bp), c.at<int>(p.o_Rh), p.N_h, p.W, p.Npad, p.Kp, c.at<int>(p.o_cexp), c.at<char>(p.o_Bt), c.s));
   }
-  return read_status(c);
+  return KUBO_OK;
 }
 
 Model make_model(const Call& c) {
@@ -924,11 +934,17 @@ kubo_status fixup_batch(Call& c, const Model& md, const KList& kl, const double*
   return KUBO_OK;
 }
 
+// W^3 n up to which kubo_ahc does not wait for the model's verdict: about 3 ms (W = 16, 24^3 k-points: 5.7e7)
+constexpr double kDeferWork = 1e8;
+
 // Shared body of kubo_ahc and kubo_ahc_host (device pointers by now).
 kubo_status ahc_device(Call& c, const kubo_options& o, const double* H_R, const RInfo& ri,
                        const double* E_F, double eta, double* out, int64_t kb, int64_t ke) {
   Plan& p = c.p;
-  kubo_status r = prepare_model(c, H_R, ri);
+  // a call of a few milliseconds runs through without waiting for the Hermitian verdict (a model that fails
+  // it costs the call's time, and out stays untouched as before); longer ones ask first
+  const bool deferred = ke - kb <= p.chunk && (double)p.W * p.W * p.W * (double)(ke - kb) <= kDeferWork;
+  kubo_status r = prepare_model(c, H_R, ri, deferred);
   if (r != KUBO_OK) return r;
   r = upload_etas(c, o, eta);
   if (r != KUBO_OK) return r;
