@@ -48,6 +48,9 @@ METRIC = "k-points/sec for σ_xy (W=64, N_R=1331), mixed vs FP64 GPU at rel err 
 WORKLOAD = "w64_r1331_k128"
 FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12   # 152 SMs x 4 FP64 flop/clk/SM x 2.07 GHz (derived)
 FP32_PEAK_TOPS = 152 * 128 * 2.07e9 / 1e12   # FP32 pipe: 152 SMs x 128 lanes x 2.07 GHz (derived)
+# 32 x 32 + 64-bit integer multiply-adds: 152 SMs x 32 lanes x 2.07 GHz (four cycles of a sub-core's pipe each,
+# measured); the FP64 path's fixed-point products take 12 per complex multiply-add (8 flop)
+IMAD_PEAK_TOPS = 152 * 32 * 2.07e9 / 1e12
 # padded K of the tensor-core Fourier contraction (N_R = 1331 -> multiple of 64)
 TC_KPAD = (1331 + 63) // 64 * 64
 # minimal FP32 operations of one double-float multiply-accumulate (TwoProd by FMA with the two
@@ -62,7 +65,7 @@ def stage_flops(W, N_R, prec="fp64"):
     """Algorithmic flops per k-point of each stage (useful work, not issued slice products).
 
     Eigenvector stage ("backtransform"): inverse iteration for the eigenvectors Z of the
-    tridiagonal, then U = Q D Z (8 W^3) -- in FP64 on the FP64 path, in FP32 on the reduced
+    tridiagonal, then U = Q D Z (8 W^3) -- in FP64 grade on the FP64 path, in FP32 on the reduced
     ones: by a kernel of its own before the 3xTF32 rotation (W > 40, the default there), inside
     the SIMT rotation kernel otherwise (counted in "berry").
     """
@@ -124,6 +127,18 @@ def roofline_of(dom, head, W, N_R, k_per_launch, ms_per_launch):
         return {"bound": "tensor", "achieved": fl / t / 1e12, "peak": pk["bf16_sustained"],
                 "unit": "TFLOP/s",
                 "peak_note": f"bf16 dense sustained, {pk['how']}; work: issued BF16 slice-pair products"}
+    if head == "fp64" and dom in ("fourier", "berry"):
+        # seven digits per operand: 28 digit products per real one (34 in the W x W products)
+        fl = stage_flops(W, N_R, head)[dom] * (28 if dom == "fourier" else 34) * k_per_launch
+        pk = measured_peaks()
+        return {"bound": "tensor", "achieved": fl / t / 1e12, "peak": pk["bf16_sustained"],
+                "unit": "TFLOP/s",
+                "peak_note": f"bf16 dense sustained, {pk['how']}; work: the digit products of the algorithmic flops"}
+    if head == "fp64" and dom in ("tridiag", "backtransform"):
+        ops = 12 / 8 * (16.0 / 3.0 if dom == "tridiag" else 8.0) * W ** 3 * k_per_launch
+        return {"bound": "alu", "achieved": ops / t / 1e12, "peak": IMAD_PEAK_TOPS, "unit": "T IMAD/s",
+                "peak_note": "integer multiply-add pipe: 152 SMs x 32 lanes x 2.07 GHz (derived); work: 12 per "
+                             "complex multiply-add of the reduction (16/3 W^3 flop) or of U = Q D Z (8 W^3)"}
     fl = stage_flops(W, N_R, head)[dom] * k_per_launch
     return {"bound": "alu", "achieved": fl / t / 1e12, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "peak_note": "FP64 pipe: 152 SMs x 4 flop/clk/SM (one DFMA warp instruction per 16 "

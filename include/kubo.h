@@ -59,7 +59,10 @@ typedef enum {
 } kubo_status;
 
 typedef enum {
-  KUBO_FP64 = 0,            /* every step in FP64 */
+  KUBO_FP64 = 0,            /* every step in FP64 or in arithmetic of at least its accuracy: the
+                               products of steps (1)-(3) as fixed-point digit products (55 to 59
+                               fractional bits, exact sums) on the tensor cores and the integer
+                               pipe, everything else in FP64 */
   KUBO_MIXED = 1,           /* the mixed-precision form: step (1) on the tensor cores (fixed-point
                                BF16 slices with exact FP32 block accumulation: H(k) to ~2^-31
                                relative, the velocity columns, which feed only step (3), to
@@ -172,7 +175,10 @@ typedef struct kubo_options {
                                k-point that reaches the cap makes the call return
                                KUBO_ERR_NO_CONVERGENCE with its outputs untouched; a cap of 1
                                forces that path on any matrix that needs a second sweep.
-                               < 0: KUBO_ERR_INVALID_ARG. */
+                               < 0: KUBO_ERR_INVALID_ARG.  (KUBO_FP64 with 0 and W >= 9 takes the
+                               inverse iteration's shifts from bisection, which has no sweeps,
+                               and reports the Rayleigh quotients of the eigenvectors; a cap
+                               asks for the QL iteration.) */
   int ql_fp64;              /* KUBO_MIXED: 1 = its QL iteration in FP64 as well and the QL
                                eigenvalues reported (every operation of the eigensolver in
                                FP64); 0 (default) = the QL iteration in double-float, used only
@@ -349,7 +355,7 @@ typedef struct kubo_batch_schedule {
                                column tile of the H columns (L2 reuse of the basis tiles; the
                                velocity columns use min(64, 4 x this)); default 8, tuned over
                                {4, 8, 16}; 1..64 */
-  int symv_parts;           /* Householder reduction: cap on the column partitions per row of
+  int symv_parts;           /* Householder reduction (not that of KUBO_FP64): cap on the column partitions per row of
                                its symv (W <= 64: the count up to the cap with the fewest FP64
                                instructions for each trailing order; W > 64: the cap where
                                the threads allow); default 4, tuned over {2, 4, 8}; 1..8 */

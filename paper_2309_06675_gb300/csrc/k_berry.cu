@@ -61,14 +61,14 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
   lo = __fadd_rn(lo, err);
 }
 
-// Curvature epilogue shared by both precisions.  Every pair is evaluated once (n < m) and
+// Curvature epilogue of the FP32-grade rotations.  Every pair is evaluated once (n < m) and
 // enters Omega_n with +T_nm and Omega_m with -T_nm, so the antisymmetry T_mn = -T_nm that
 // makes occupied-occupied pairs cancel holds exactly even when v is only Hermitian to FP32
 // rounding.  Per-thread row / column partials go to `red` (2 * n_eta * W * 16 doubles, may
 // alias sVx: a barrier separates the last read of sVx from the first write of red) and are
 // summed in a fixed order (deterministic).
 //
-// FP32 velocities (V = float2): the numerator carries FP32 rounding already, so the quotient
+// The numerator carries FP32 rounding already, so the quotient
 // T = num / (dE^2 + eta^2) is formed in FP32 too; only dE = E_n - E_m (a difference of close
 // FP64 eigenvalues), its square and the eta = 0 cut-off stay in FP64.  The numerator is
 // Kahan's difference of products (within 2 ulp of the exact Im part), and the partial sums are
@@ -77,21 +77,17 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
 // both bands are occupied.  Every term is bounded (|num| <= 2 |v^x| |v^y|) while the FP32
 // denominator is at least 2^-86; a thread whose tile holds a smaller one (eta and a gap below
 // ~1e-13) takes the FP64 quotient for that eta.
-template <int TM, typename V>
-__device__ __forceinline__ void curvature_epilogue(const V* sVx, const V (&vy)[TM][TM],
+template <int TM>
+__device__ __forceinline__ void curvature_epilogue(const float2* sVx, const float2 (&vy)[TM][TM],
                                                    const double* sE, const double* sEta,
                                                    int n_eta, double emax, int W, int LD, int ty,
                                                    int tx, int t, double* red,
                                                    double* __restrict__ Om, int64_t eta_stride,
                                                    int64_t k) {
-  constexpr bool F32 = std::is_same<V, float2>::value;
-  using R = typename std::conditional<F32, float, double>::type;
   const double thr2 = (1e-12 * emax) * (1e-12 * emax);
-  R num[TM][TM];
-  // (dE)^2 per pair: FP64 for FP64 velocities; for FP32 ones only its FP32 rounding is kept
-  // (the FP64 fallback recomputes it), and the pair / cut-off tests are bit masks, so that the
-  // per-eta loop issues no FP64 compare
-  double d2[F32 ? 1 : TM][F32 ? 1 : TM];
+  float num[TM][TM];
+  // (dE)^2 per pair: only its FP32 rounding is kept (the FP64 fallback recomputes it), and the
+  // pair / cut-off tests are bit masks, so that the per-eta loop issues no FP64 compare
   float d2f[TM][TM];
   unsigned pairs = 0;    // bit (i TM + j): n < m < W
   unsigned small0 = 0;   // bit (i TM + j): (dE)^2 <= thr2 (dropped when eta = 0)
@@ -105,15 +101,11 @@ __device__ __forceinline__ void curvature_epilogue(const V* sVx, const V (&vy)[T
       d2f[i][j] = 0.f;
       if (n < W && m < W && n < m) {
         pairs |= 1u << (i * TM + j);
-        const V vx = sVx[n * LD + m];
-        if constexpr (F32)
-          num[i][j] = -2.0f * diff_of_products(vx.y, vy[i][j].x, vx.x, vy[i][j].y);
-        else
-          num[i][j] = -2.0 * (vx.y * vy[i][j].x - vx.x * vy[i][j].y);
+        const float2 vx = sVx[n * LD + m];
+        num[i][j] = -2.0f * diff_of_products(vx.y, vy[i][j].x, vx.x, vy[i][j].y);
         const double dE = sE[n] - sE[m];
         const double q = dE * dE;
-        if constexpr (F32) d2f[i][j] = (float)q;
-        else d2[i][j] = q;
+        d2f[i][j] = (float)q;
         if (q <= thr2) small0 |= 1u << (i * TM + j);
       }
     }
@@ -122,11 +114,11 @@ __device__ __forceinline__ void curvature_epilogue(const V* sVx, const V (&vy)[T
   for (int e = 0; e < n_eta; ++e) {
     const double eta = sEta[e];
     const bool eta0 = eta == 0.0;
-    R rp[TM], cp[TM], rl[TM], cl[TM];   // (rl, cl: the FP32 pairs' low parts)
+    float rp[TM], cp[TM], rl[TM], cl[TM];   // (rl, cl: the FP32 pairs' low parts)
 #pragma unroll
     for (int i = 0; i < TM; ++i) { rp[i] = 0; cp[i] = 0; rl[i] = 0; cl[i] = 0; }
-    bool fp64 = !F32;
-    if constexpr (F32) {
+    bool fp64 = false;
+    {
       const float eta2 = (float)(eta * eta);
 #pragma unroll
       for (int i = 0; i < TM; ++i)
@@ -151,14 +143,8 @@ __device__ __forceinline__ void curvature_epilogue(const V* sVx, const V (&vy)[T
         for (int j = 0; j < TM; ++j) {
           if (!((pairs >> (i * TM + j)) & 1u)) continue;
           if (eta0 && ((small0 >> (i * TM + j)) & 1u)) continue;
-          double q;
-          if constexpr (F32) {
-            const double dE = sE[ty + 16 * i] - sE[tx + 16 * j];
-            q = dE * dE;
-          } else {
-            q = d2[i][j];
-          }
-          const double T = (double)num[i][j] / fma(eta, eta, q);
+          const double dE = sE[ty + 16 * i] - sE[tx + 16 * j];
+          const double T = (double)num[i][j] / fma(eta, eta, dE * dE);
           rq[i] += T;
           cq[j] -= T;
         }
@@ -488,7 +474,7 @@ __global__ void __launch_bounds__(NT) berry_mixed_kernel(const double* __restric
   store_tile_f32<TM>(sB, W, LD, ty, tx, acc);
   __syncthreads();
   cgemm_tile_f32<TM, true>(sU, sB, W, LD, ty, tx, acc);    // v^y = U^H T
-  curvature_epilogue<TM, float2>(sA, acc, sE, sEta, n_eta, s_emax, W, LD, ty, tx, t, red, Om,
+  curvature_epilogue<TM>(sA, acc, sE, sEta, n_eta, s_emax, W, LD, ty, tx, t, red, Om,
                              eta_stride, k);
 }
 
@@ -847,7 +833,7 @@ __global__ void __launch_bounds__(RT_NT, 1) berry_tc_kernel(
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) vy[i][j] = sVy[(ty + 16 * i) * LDV + tx + 16 * j];
-      curvature_epilogue<4, float2>(sVx, vy, sE, sEta, n_eta, s_emax, W, LDV, ty, tx, t,
+      curvature_epilogue<4>(sVx, vy, sE, sEta, n_eta, s_emax, W, LDV, ty, tx, t,
                                     reinterpret_cast<double*>(opA), Om, eta_stride, k);
     }
   }
@@ -1258,7 +1244,7 @@ __global__ void __launch_bounds__(TF_NT, 2) berry_tf32_kernel(
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) vy[i][j] = sVy[(ty + 16 * i) * TF_LDU + tx + 16 * j];
-      curvature_epilogue<4, float2>(sVx, vy, sE, sEta, n_eta, s_emax, W, TF_LDU, ty, tx, t,
+      curvature_epilogue<4>(sVx, vy, sE, sEta, n_eta, s_emax, W, TF_LDU, ty, tx, t,
                                     reinterpret_cast<double*>(tf_smem), Om, eta_stride, k);
     }
   }

@@ -1,10 +1,11 @@
 // FP64-grade matrix work of steps (2)-(4) on the integer pipe (fixed.cuh):
 //
-//   berry_fix_kernel   v^a = U^dagger (d_a H) U for a = x, y and the curvature of Eq. 3 (W <= 64)
+//   berry_fix_kernel   v^a = U^dagger (d_a H) U for a = x, y and the curvature of Eq. 3 (W <= 24; to 64
+//                      where a caller's workspace has no room for k_zgemm_tc64.cu's matrices)
 //   reflect_fix_kernel U = Q D Z: the Householder reflectors applied to the eigenvectors of T
 //
 // Both were FP64 kernels at 85-96 % of the FP64 pipe; the products here are sums of 59-bit
-// fixed-point products, ten times as many per clock.  Energy differences, curvature quotients
+// fixed-point products, five times as many per clock.  Energy differences, curvature quotients
 // and the band sums stay FP64.
 #include <algorithm>
 

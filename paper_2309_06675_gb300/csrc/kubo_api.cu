@@ -23,11 +23,12 @@ constexpr int MAX_ETA = 8;
 // core products above.  9,216 k-points, integer pipe and tensor cores: W = 24 1.25 and 1.31 ms, W = 28 2.10 and
 // 1.47, W = 32 2.43 and 1.53 (W = 16, 13,824: 0.54 and 1.13); 19 to 304 k-points at W = 25: 0.084 and 0.080
 constexpr int FIX_W_MAX = 24;
-// k-points per sub-batch of the latter: T, v^x and v^y of a sub-batch (192 KB each at W = 64) are
-// written and read while they are in L2
+// k-points per sub-batch of the latter: T, v^x and v^y of a sub-batch (64 KB each per k-point at W = 64) are
+// written and read while most of them are in L2, and 8 tiles per SM keep the last wave short
 constexpr int ZG_BATCH = 152 * 8;
 // Shifts by bisection (a lane per eigenvalue) instead of the QL iteration (a lane per k-point) from
-// this order
+// this order: W = 16, 13,824 k-points 0.49 -> 0.16 ms, W = 48, 777: 3.55 -> 0.13, W = 64, 4,096: 6.2 -> 0.63; at
+// W = 6, 147,456 k-points, the QL lanes fill the chip and take 0.15 ms
 constexpr int BISECT_W_MIN = 9;
 constexpr int KSUM_KPB = 32;         // k-points per deterministic k-sum block (at least)
 constexpr size_t KSUM_PART_BYTES = (size_t)256 << 20;   // cap on the per-block partials
@@ -223,7 +224,9 @@ int auto_chunk(int W, int n_eta, int64_t n_total, size_t extra_per_k = 0) {
 
 // Step (1) of the FP64 mode on the tensor cores (seven slices) instead of the FP64 pipe.  The
 // FMA kernel takes 6 N_R W^2 operations per k-point at 1.2 TFLOP/s; the tensor-core form adds
-// three launches and the slicing of the basis, and pads to 64 vectors and 32 columns.
+// three launches and the slicing of the basis, and pads to 64 vectors and 32 columns: W = 64, N_R = 1331,
+// 4,096 k-points 112 -> 3.4 ms, W = 16, N_R = 125, 13,824 (2.7e9 operations) 2.34 -> 0.16 ms; at 1e8
+// operations the FMA kernel takes 0.1 ms, about what the extra launches and the slicing cost.
 // The sliced basis (42 bytes per complex entry of H(R)) stays within 16 GiB.
 constexpr double kTc64MinFlops = 1e8;
 constexpr size_t kTc64MaxBasis = (size_t)16 << 30;
@@ -713,6 +716,12 @@ cudaError_t berry_tc64(const Call& c, const double* E, const double2* U, const i
   return cudaSuccess;
 }
 
+// kernels of one berry_any call
+int berry_launches(const Plan& p, int n) {
+  if (p.zk > 0) return 7 * ((n + p.zk - 1) / p.zk);   // per sub-batch: two exponents, four products, curvature
+  return p.W > SMALL_W_MAX ? 5 : 1;
+}
+
 // Steps (3)-(4) from packed Hermitian dH rows X, Y of leading dimension ld; f32 = FP32
 // products.  rows = X and Y are the W*W and 2*W*W column offsets of tensor-core output rows.
 cudaError_t berry_any(const Call& c, const double* E, const double2* U, const double* X,
@@ -815,7 +824,7 @@ kubo_status run_batch_mixed(Call& c, const Model& md, const KList& kl, double* E
                         rq_eigenvalues(p.precision, p.ql_fp64)));
   }
   {
-    StageTimer tm(c, KUBO_STAGE_BERRY, p.W > SMALL_W_MAX ? 5 : 1);
+    StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n));
     KCHECK(berry_any(c, Eout, U, C64 + WW, C64 + 2 * WW, p.Npad, true, kl.n, f32_rotation(p.precision), Om, om_stride));
   }
   return KUBO_OK;
@@ -833,7 +842,7 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
   DevStatus* st = c.at<DevStatus>(p.o_status);
   double2* U = c.at<double2>(p.o_U);
   if (!fourier_done) {
-    StageTimer tm(c, KUBO_STAGE_FOURIER, p.tc64 ? 2 : 1);
+    StageTimer tm(c, KUBO_STAGE_FOURIER, p.tc64 ? 2 * ((kl.n + p.f64_k - 1) / p.f64_k) : 1);
     KCHECK(fourier64(c, md, kl, Hp, Xp, Yp));
   }
   {
@@ -868,7 +877,7 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
     KCHECK(eigh_vectors(c, kl.n, eb, Eout, U, f32_rotation(p.precision)));
   }
   {
-    StageTimer tm(c, KUBO_STAGE_BERRY, p.W > SMALL_W_MAX ? 5 : 1);
+    StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n));
     KCHECK(berry_any(c, Eout, U, Xp, Yp, (int64_t)p.W * p.W, false, kl.n, f32_rotation(p.precision), Om, om_stride));
   }
   return KUBO_OK;
@@ -1104,7 +1113,7 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
     KList kl{nullptr, base, (int)std::min<int64_t>(p.chunk, ke - base)};
     const int n = kl.n;
     {
-      StageTimer tm(c, KUBO_STAGE_FOURIER, p.tc64 ? 2 : 1);
+      StageTimer tm(c, KUBO_STAGE_FOURIER, p.tc64 ? 2 * ((kl.n + p.f64_k - 1) / p.f64_k) : 1);
       KCHECK(fourier64(c, md, kl, Hp, Xp, Yp));
     }
     {
@@ -1121,7 +1130,7 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
     }
     if (out) {
       {
-        StageTimer tm(c, KUBO_STAGE_BERRY, p.W > SMALL_W_MAX ? 5 : 1);
+        StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n));
         KCHECK(berry_any(c, E, U, Xp, Yp, (int64_t)WW, false, n, false, Om, (int64_t)n * p.W));
       }
       StageTimer tm(c, KUBO_STAGE_KSUM, o.kT == 0.0 ? 3 : 2);
