@@ -222,18 +222,23 @@ int auto_chunk(int W, int n_eta, int64_t n_total, size_t extra_per_k = 0) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(c, n_total));
 }
 
-// Step (1) of the FP64 mode on the tensor cores (seven slices) instead of the FP64 pipe.  The
-// FMA kernel takes 6 N_R W^2 operations per k-point at 1.2 TFLOP/s; the tensor-core form adds
-// three launches and the slicing of the basis, and pads to 64 vectors and 32 columns: W = 64, N_R = 1331,
-// 4,096 k-points 112 -> 3.4 ms, W = 16, N_R = 125, 13,824 (2.7e9 operations) 2.34 -> 0.16 ms; at 1e8
-// operations the FMA kernel takes 0.1 ms, about what the extra launches and the slicing cost.
-// The sliced basis (42 bytes per complex entry of H(R)) stays within 16 GiB.
+// Step (1) of the FP64 mode on the tensor cores (seven slices) instead of the FP64 pipe.  The tensor-core form
+// adds three launches and the slicing of the basis, and pads to 64 vectors and 32 columns; the FMA kernel takes
+// 6 N_R W^2 operations per k-point at 1.2 TFLOP/s, and not less than the 1.7 us a vector takes its CTA
+// (preparation and sum in ms, FMA -> tensor cores: one k-point of W = 16, N_R = 27 0.077 -> 0.062, N_R = 125 0.242 ->
+// 0.071; W = 32, N_R = 729 1.30 -> 0.157; W = 64, N_R = 1331 2.56 -> 0.465; the sum alone at W = 64, N_R = 1331, 4,096
+// k-points 112 -> 3.4).  So: from 24 vectors, fewer (from 16) where there are 1e8 operations.
+// The sliced basis (42 bytes per complex entry of H(R)) stays within 16 GiB, and 256 MiB below 1e8 operations.
 constexpr double kTc64MinFlops = 1e8;
 constexpr size_t kTc64MaxBasis = (size_t)16 << 30;
+constexpr int kTc64MinVectors = 24;
+constexpr size_t kTc64SmallBasis = (size_t)256 << 20;
 constexpr size_t kTc64CoefBytes = (size_t)2 << 30;   // coefficient slices of a sub-batch
 bool use_tc64(int W, int N_R, int64_t n) {
   const size_t basis = (size_t)2 * tc64_slices() * tc64_pad_n(W) * tc_pad_k(N_R);
-  return W >= 4 && N_R >= 16 && 6.0 * N_R * W * W * (double)n >= kTc64MinFlops && basis <= kTc64MaxBasis;
+  if (W < 4 || N_R < 16) return false;
+  if (6.0 * N_R * W * W * (double)n >= kTc64MinFlops) return basis <= kTc64MaxBasis;
+  return N_R >= kTc64MinVectors && basis <= kTc64SmallBasis;
 }
 
 void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
