@@ -129,36 +129,65 @@ __global__ void band_prefix_kernel(double* __restrict__ Om, int W, int n, int n_
 
 constexpr int KS_MAXE = 8;
 
-// kT = 0: thread per E_F (all etas), k-range of the block in order
-__global__ void ksum_step_kernel(const double* __restrict__ E, const double* __restrict__ P,
-                                 int W, int n, int n_eta, int64_t eta_stride,
-                                 const double* __restrict__ E_F, int n_EF,
-                                 double2* __restrict__ part, int kpb) {
-  const int b = blockIdx.x;
+// kT = 0: a CTA's threads are TJ Fermi levels x KG groups of its k-points, every thread all etas; group kg takes
+// the k-points kg, kg + KG, ... in order and the groups are added in order (Neumaier).  A k-point is a
+// chain of log2 W dependent loads, and one thread per Fermi level walked a block's 32 of them in turn.  k-sum stage
+// (three launches) with one level: W = 2, 576 k-points 81 -> 33 us; W = 16, 13,824 126 -> 52 us; W = 6, 147,456 and
+// four etas 0.53 -> 0.42 ms; 64 levels, W = 64, 4,096: 0.18 -> 0.115 ms.
+constexpr int KS_NT = 256;
+__global__ void __launch_bounds__(KS_NT) ksum_step_kernel(const double* __restrict__ E,
+                                                          const double* __restrict__ P, int W, int n,
+                                                          int n_eta, int64_t eta_stride,
+                                                          const double* __restrict__ E_F, int n_EF,
+                                                          double2* __restrict__ part, int kpb, int TJ,
+                                                          int KG) {
+  __shared__ double2 red[KS_NT];
+  const int b = blockIdx.x, t = threadIdx.x;
+  const int tj = t % TJ, kg = t / TJ;
   const int kb = b * kpb, ke = min(n, kb + kpb);
   const int n_out = n_eta * n_EF;
-  for (int j = threadIdx.x; j < n_EF; j += blockDim.x) {
-    const double ef = E_F[j];
+  for (int j0 = 0; j0 < n_EF; j0 += TJ) {
+    const int j = j0 + tj;
+    const bool on = j < n_EF;
+    const double ef = on ? E_F[j] : 0.0;
     double s[KS_MAXE], c[KS_MAXE];
 #pragma unroll
     for (int e = 0; e < KS_MAXE; ++e) { s[e] = 0.0; c[e] = 0.0; }
-    for (int k = kb; k < ke; ++k) {
-      const double* Ek = E + (size_t)k * W;
-      int lo = 0, hi = W;   // number of levels strictly below E_F
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (Ek[mid] < ef) lo = mid + 1;
-        else hi = mid;
+    if (on)
+      for (int k = kb + kg; k < ke; k += KG) {
+        const double* Ek = E + (size_t)k * W;
+        int lo = 0, hi = W;   // number of levels strictly below E_F
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (Ek[mid] < ef) lo = mid + 1;
+          else hi = mid;
+        }
+        if (lo == 0) continue;
+        const double* Pk = P + (size_t)k * W + (lo - 1);
+#pragma unroll
+        for (int e = 0; e < KS_MAXE; ++e)
+          if (e < n_eta) neumaier_add(s[e], c[e], Pk[e * eta_stride]);
       }
-      if (lo == 0) continue;
-      const double* Pk = P + (size_t)k * W + (lo - 1);
 #pragma unroll
-      for (int e = 0; e < KS_MAXE; ++e)
-        if (e < n_eta) neumaier_add(s[e], c[e], Pk[e * eta_stride]);
+    for (int e = 0; e < KS_MAXE; ++e) {
+      if (e >= n_eta) break;
+      if (KG == 1) {
+        if (on) part[(size_t)b * n_out + e * n_EF + j] = make_double2(s[e], c[e]);
+        continue;
+      }
+      __syncthreads();
+      red[t] = make_double2(s[e], c[e]);
+      __syncthreads();
+      if (on && kg == 0) {
+        double s2 = 0.0, c2 = 0.0;
+        for (int g = 0; g < KG; ++g) {
+          const double2 r = red[g * TJ + tj];
+          neumaier_add(s2, c2, r.x);
+          c2 += r.y;
+        }
+        part[(size_t)b * n_out + e * n_EF + j] = make_double2(s2, c2);
+      }
     }
-#pragma unroll
-    for (int e = 0; e < KS_MAXE; ++e)
-      if (e < n_eta) part[(size_t)b * n_out + e * n_EF + j] = make_double2(s[e], c[e]);
   }
 }
 
@@ -323,8 +352,10 @@ cudaError_t launch_ksum_partial(const double* E, double* Om, int W, int n, int n
     const int64_t rows = (int64_t)n_eta * n;
     const int pb = (int)std::min<int64_t>((rows + 127) / 128, 152 * 16);
     band_prefix_kernel<<<pb, 128, 0, s>>>(Om, W, n, n_eta, eta_stride);
-    const int nt = std::min(256, (n_EF + 31) / 32 * 32);
-    ksum_step_kernel<<<nb, nt, 0, s>>>(E, Om, W, n, n_eta, eta_stride, E_F, n_EF, part, kpb);
+    int TJ = 1, KG = 1;   // powers of two: TJ covers the Fermi levels, KG the k-points of a block, TJ KG <= 256
+    while (TJ < n_EF && TJ < KS_NT) TJ *= 2;
+    while (KG < kpb && KG < 32 && TJ * KG < KS_NT) KG *= 2;
+    ksum_step_kernel<<<nb, TJ * KG, 0, s>>>(E, Om, W, n, n_eta, eta_stride, E_F, n_EF, part, kpb, TJ, KG);
   } else {
     const int TJ = std::min(n_EF, FD_NT), KT = std::min(kpb, std::max(1, FD_LEVELS / W));
     const size_t sm = (size_t)KT * W * (sizeof(double) + sizeof(int));

@@ -172,3 +172,27 @@ def test_gradient_of_shared_tiles(W, n):
     parts = sum(first(run(3 + i, 4 + i)).cpu().numpy() for i in range(n))
     assert np.isfinite(whole).all()
     assert np.abs(whole - parts).max() <= 1e-12 * max(np.abs(parts).max(), 1e-300)
+
+
+@pytest.mark.parametrize("n_EF", [1, 2, 3, 31, 33, 255, 256, 257])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 70])
+def test_step_occupation_sum(n_EF, n):
+    # Fermi levels x groups of k-points of a block (32 k-points): against an exact sum of the same
+    # curvatures; a compensated sum of at most 70 terms of one rounding each (the prefix over bands: W of them)
+    import math
+    import torch
+    import tbgen
+    import paper_2309_06675_gb300 as kubo
+    W, mesh, etas = 5, (5, 7, 2), [0.05, 0.3]
+    m = tbgen.random_tb(W, 1, 1.0, 3)
+    H, R = torch.from_numpy(m.H_R).cuda(), torch.from_numpy(m.R)
+    ef = np.linspace(-1.5, 1.5, n_EF)
+    got = kubo.ahc(H, R, mesh, torch.from_numpy(ef).cuda(), etas=etas, k_range=(0, n)).cpu().numpy()
+    E, Om = kubo.ahc_k(H, R, mesh, torch.arange(n, dtype=torch.int64).cuda(), etas=etas)
+    E, Om = E.cpu().numpy(), Om.cpu().numpy()
+    for e in range(2):
+        for j in range(n_EF):
+            occ = E < ef[j]
+            ref = math.fsum(Om[e][occ]) / np.prod(mesh)
+            bound = (W + 2) * 2.0 ** -52 * np.abs(Om[e][occ]).sum() / np.prod(mesh)
+            assert abs(got[e, j] - ref) <= bound, (e, j)
