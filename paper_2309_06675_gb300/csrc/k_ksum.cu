@@ -130,10 +130,11 @@ __global__ void band_prefix_kernel(double* __restrict__ Om, int W, int n, int n_
 constexpr int KS_MAXE = 8;
 
 // kT = 0: a CTA's threads are TJ Fermi levels x KG groups of its k-points, every thread all etas; group kg takes
-// the k-points kg, kg + KG, ... in order and the groups are added in order (Neumaier).  A k-point is a
+// the k-points kg, kg + KG, ... in order and the groups are added in a fixed tree (Neumaier).  A k-point is a
 // chain of log2 W dependent loads, and one thread per Fermi level walked a block's 32 of them in turn.  k-sum stage
-// (three launches) with one level: W = 2, 576 k-points 81 -> 33 us; W = 16, 13,824 126 -> 52 us; W = 6, 147,456 and
-// four etas 0.53 -> 0.42 ms; 64 levels, W = 64, 4,096: 0.18 -> 0.115 ms.
+// (three launches) with one level: W = 2, 576 k-points 81 -> 25 us; W = 16, 13,824 126 -> 43 us; W = 6, 147,456 and
+// four etas 0.53 -> 0.155 ms (0.42 with the groups added one after the other by one thread: FP64 additions of
+// single lanes); 64 levels, W = 64, 4,096: 0.18 -> 0.112 ms.
 constexpr int KS_NT = 256;
 __global__ void __launch_bounds__(KS_NT) ksum_step_kernel(const double* __restrict__ E,
                                                           const double* __restrict__ P, int W, int n,
@@ -178,15 +179,16 @@ __global__ void __launch_bounds__(KS_NT) ksum_step_kernel(const double* __restri
       __syncthreads();
       red[t] = make_double2(s[e], c[e]);
       __syncthreads();
-      if (on && kg == 0) {
-        double s2 = 0.0, c2 = 0.0;
-        for (int g = 0; g < KG; ++g) {
-          const double2 r = red[g * TJ + tj];
-          neumaier_add(s2, c2, r.x);
-          c2 += r.y;
+      for (int h = KG / 2; h > 0; h >>= 1) {
+        if (kg < h) {
+          const double2 x = red[t], y = red[t + h * TJ];
+          double s2 = x.x, c2 = x.y;
+          neumaier_add(s2, c2, y.x);
+          red[t] = make_double2(s2, c2 + y.y);
         }
-        part[(size_t)b * n_out + e * n_EF + j] = make_double2(s2, c2);
+        __syncthreads();
       }
+      if (on && kg == 0) part[(size_t)b * n_out + e * n_EF + j] = red[t];
     }
   }
 }
