@@ -204,19 +204,6 @@ __device__ __forceinline__ long long pf_fixed31(float h, float l) {
   const long long r = (aq + (1ll << 30)) >> 31;
   return q < 0 ? -r : r;
 }
-// x mod d in [0, d) for |x| < 2^32, by the multiply-high division
-__device__ __forceinline__ int posmod(long long x, const FastDiv& f) {
-  const unsigned long long ax = x < 0 ? (unsigned long long)(-x) : (unsigned long long)x;
-  uint32_t r;
-  if (ax < 0x100000000ull) {
-    const uint32_t a = (uint32_t)ax;
-    r = a - f.div(a) * f.d;
-  } else {
-    r = (uint32_t)(ax % f.d);
-  }
-  return (x < 0 && r) ? (int)(f.d - r) : (int)r;
-}
-
 // A[s][m][k] for m < Mpad (rows >= n are zero), k < Kp.  Persistent CTAs over the rows
 // (k-points); a row's mesh coordinates once per row, then per (m, h) the three per-axis
 // twiddles by exact integer argument reduction (multiply-high modulo) and their product as two

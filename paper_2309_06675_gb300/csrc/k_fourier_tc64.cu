@@ -156,18 +156,6 @@ __global__ void basis_pad7_kernel(int n0, int Npad, int Kp, __nv_bfloat16* __res
     reinterpret_cast<uint32_t*>(Bt + (t / cnt) * plane + (size_t)n0 * Kp)[t % cnt] = 0u;
 }
 
-__device__ __forceinline__ int posmod(long long x, const FastDiv& f) {
-  const unsigned long long ax = x < 0 ? (unsigned long long)(-x) : (unsigned long long)x;
-  uint32_t r;
-  if (ax < 0x100000000ull) {
-    const uint32_t a = (uint32_t)ax;
-    r = a - f.div(a) * f.d;
-  } else {
-    r = (uint32_t)(ax % f.d);
-  }
-  return (x < 0 && r) ? (int)(f.d - r) : (int)r;
-}
-
 // A[s][m][k] for m < Mpad (rows >= n zero), k < Kp: the phases are those of mesh_phase (FP64
 // products of the three twiddles), rounded to 55 fractional bits.
 __global__ void __launch_bounds__(256) coef_slice7_kernel(Model md, Mesh mesh, KList kl, int Mpad,
@@ -180,8 +168,15 @@ __global__ void __launch_bounds__(256) coef_slice7_kernel(Model md, Mesh mesh, K
   for (int64_t i0 = (int64_t)blockIdx.x * 256; i0 < total; i0 += (int64_t)gridDim.x * 256) {
     const int64_t idx = i0 + threadIdx.x;
     if (idx >= total) break;
-    const int m = idx < 0x100000000ll ? (int)fp.div((uint32_t)idx) : (int)(idx / npair);
-    const int h = (int)(idx - (int64_t)m * npair);
+    int m, h;   // (idx npair is beyond 2^32 from some 10,000 rows at N_R = 1331)
+    if (idx < 0x100000000ll) {
+      uint32_t rem;
+      m = (int)fp.divmod((uint32_t)idx, rem);
+      h = (int)rem;
+    } else {
+      m = (int)(idx / npair);
+      h = (int)(idx - (int64_t)m * npair);
+    }
     uint32_t dc[NS], ds[NS];
 #pragma unroll
     for (int i = 0; i < NS; ++i) dc[i] = ds[i] = 0u;

@@ -137,9 +137,31 @@ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
 struct FastDiv {
   uint32_t d, mag;
   __host__ __device__ static uint32_t magic(uint32_t dd) { return dd > 1 ? 0xFFFFFFFFu / dd + 1u : 0u; }
-  __device__ explicit FastDiv(uint32_t dd) : d(dd), mag(magic(dd)) {}
-  __device__ __forceinline__ uint32_t div(uint32_t a) const { return mag ? __umulhi(a, mag) : a; }
+  __host__ __device__ explicit FastDiv(uint32_t dd) : d(dd), mag(magic(dd)) {}
+  __host__ __device__ __forceinline__ uint32_t div(uint32_t a) const {
+    return mag ? (uint32_t)(((uint64_t)a * mag) >> 32) : a;
+  }
+  // floor(a / d) and the remainder for any a < 2^32 and d < 2^31: where a d >= 2^32 the
+  // multiply-high may be one too large, and a - q d is then negative (in [-d, 0))
+  __host__ __device__ __forceinline__ uint32_t divmod(uint32_t a, uint32_t& r) const {
+    uint32_t q = div(a);
+    r = a - q * d;
+    if ((int32_t)r < 0) {
+      r += d;
+      --q;
+    }
+    return q;
+  }
 };
+
+// x mod f.d in [0, f.d): exact for every x (64-bit division beyond |x| = 2^32)
+__host__ __device__ __forceinline__ int posmod(long long x, const FastDiv& f) {
+  const unsigned long long ax = x < 0 ? (unsigned long long)(-x) : (unsigned long long)x;
+  uint32_t r;
+  if (ax < 0x100000000ull) f.divmod((uint32_t)ax, r);
+  else r = (uint32_t)(ax % f.d);
+  return (x < 0 && r) ? (int)(f.d - r) : (int)r;
+}
 
 // e^{i k.R} from per-axis twiddle tables with exact integer argument reduction.
 __device__ __forceinline__ double2 mesh_phase(const double2* __restrict__ tab, const int* off,
