@@ -1201,6 +1201,7 @@ struct Job {
   Plan p;
   double cost = 0.0;    // estimated device work (LPT order)
   int stream = 0;
+  bool skip = false;    // its H(R) failed the device check: keeps its place in the layout, is not run
   size_t o_tables = 0;  // offset of neg / pairs / Rh / status in the tables region
 };
 
@@ -1355,6 +1356,7 @@ kubo_status issue_batch(const BatchRun& br, const std::vector<kubo_problem>& pro
     if (cudaStreamWaitEvent(streams[q], evs[0], 0) != cudaSuccess) r = KUBO_ERR_CUDA;
   for (size_t i = 0; i < br.jobs.size() && r == KUBO_OK; ++i) {
     const Job& j = br.jobs[i];
+    if (j.skip) continue;
     Call c;
     c.p = j.p;
     c.s = streams[j.stream];
@@ -1776,29 +1778,30 @@ kubo_status kubo_ahc_batched(kubo_problem* probs, int n_probs, const kubo_option
     for (size_t i = 0; i < br.jobs.size(); ++i)
       BCHECK(cudaMemcpyAsync(&hs[i], job_tables(ws, br.jobs[i]).st, sizeof(DevStatus), cudaMemcpyDeviceToHost, origin));
     BCHECK(cudaStreamSynchronize(origin));
-    {
-      std::vector<Job> ok;
-      for (size_t i = 0; i < br.jobs.size(); ++i) {
-        const kubo_status r = bits_to_status(hs[i].bits);
-        if (r != KUBO_OK) {
-          probs[br.jobs[i].idx].status = r;
-          if (first == KUBO_OK) first = r;
-        } else {
-          // a model outside the FP32 steps' comfortable range is scaled by a power of two
-          // (basis and broadenings; its eigenvalues are scaled back per batch)
-          Job& j = br.jobs[i];
-          j.p.escale = j.p.scale_ok ? range_exponent(herm_max(hs[i])) : 0;
-          if (j.p.escale != 0) {
-            for (double& x : eta_h[i]) x = std::ldexp(x, j.p.escale);
-            BCHECK(cudaMemcpyAsync(job_tables(ws, j).etas, eta_h[i].data(), sizeof(double) * MAX_ETA,
-                                   cudaMemcpyHostToDevice, origin));
-          }
-          ok.push_back(std::move(j));
-        }
+    // A model that fails is skipped but stays in the layout: the allocation above was sized with every
+    // model, and a layout of the others alone (larger batches on fewer streams, another assignment) can
+    // be larger than that.
+    int n_run = 0;
+    for (size_t i = 0; i < br.jobs.size(); ++i) {
+      Job& j = br.jobs[i];
+      const kubo_status r = bits_to_status(hs[i].bits);
+      if (r != KUBO_OK) {
+        probs[j.idx].status = r;
+        if (first == KUBO_OK) first = r;
+        j.skip = true;
+        continue;
       }
-      br.jobs.swap(ok);
+      ++n_run;
+      // a model outside the FP32 steps' comfortable range is scaled by a power of two
+      // (basis and broadenings; its eigenvalues are scaled back per batch)
+      j.p.escale = j.p.scale_ok ? range_exponent(herm_max(hs[i])) : 0;
+      if (j.p.escale != 0) {
+        for (double& x : eta_h[i]) x = std::ldexp(x, j.p.escale);
+        BCHECK(cudaMemcpyAsync(job_tables(ws, j).etas, eta_h[i].data(), sizeof(double) * MAX_ETA,
+                               cudaMemcpyHostToDevice, origin));
+      }
     }
-    if (br.jobs.empty()) return finish(first);
+    if (n_run == 0) return finish(first);
     std::vector<kubo_problem> PP(probs, probs + n_probs);
     double* probe_out = (double*)(ws + probe_off);
     // ---- autotune: time every candidate schedule on a probe of each model's first k-points
@@ -1810,7 +1813,7 @@ kubo_status kubo_ahc_batched(kubo_problem* probs, int n_probs, const kubo_option
       int bS = cand_S[0], bC = cand_C[0];
       for (int cs : cand_S)
         for (int cc : cand_C) {
-          layout_batch(br, std::min(cs, (int)br.jobs.size()), cc, n_eta);
+          layout_batch(br, cs, cc, n_eta);
           float ms = 0.f;
           kubo_status r = run_batch_once(br, PP, o, ws, origin, streams, graph, probe_out, probe_nk, &ms);
           if (r != KUBO_OK) return finish(r);
@@ -1821,11 +1824,11 @@ kubo_status kubo_ahc_batched(kubo_problem* probs, int n_probs, const kubo_option
       chunk = bC;
       // then the kernel parameters, one at a time from the defaults (coordinate search), on
       // the chosen schedule
-      layout_batch(br, std::min(S, (int)br.jobs.size()), chunk, n_eta);
+      layout_batch(br, S, chunk, n_eta);
       auto try_params = [&](KernelParams kp) -> kubo_status {
         const KernelParams keep = br.kp;
         br.kp = kp;
-        layout_batch(br, std::min(S, (int)br.jobs.size()), chunk, n_eta);
+        layout_batch(br, S, chunk, n_eta);
         float ms = 0.f;
         kubo_status r = run_batch_once(br, PP, o, ws, origin, streams, graph, probe_out, probe_nk, &ms);
         if (r != KUBO_OK) return r;
@@ -1863,13 +1866,14 @@ kubo_status kubo_ahc_batched(kubo_problem* probs, int n_probs, const kubo_option
       chunk = cand_C[0];
     }
     // ---- the real run
-    layout_batch(br, std::min(S, (int)br.jobs.size()), chunk, n_eta);
+    layout_batch(br, S, chunk, n_eta);
     kubo_status r = run_batch_once(br, PP, o, ws, origin, streams, graph, nullptr, {}, nullptr);
     if (r != KUBO_OK) return finish(r);
     for (size_t i = 0; i < br.jobs.size(); ++i)
       BCHECK(cudaMemcpyAsync(&hs[i], job_tables(ws, br.jobs[i]).st, sizeof(DevStatus), cudaMemcpyDeviceToHost, origin));
     BCHECK(cudaStreamSynchronize(origin));
     for (size_t i = 0; i < br.jobs.size(); ++i) {
+      if (br.jobs[i].skip) continue;
       const kubo_status rj = bits_to_status(hs[i].bits);
       probs[br.jobs[i].idx].status = rj;
       if (rj != KUBO_OK && first == KUBO_OK) first = rj;
