@@ -8,6 +8,7 @@
 // O(W).  The prefix is accumulated in band order, so the per-k term is bit-identical to the
 // direct sum over occupied bands.
 #include <algorithm>
+#include <type_traits>
 
 #include "kubo_internal.cuh"
 
@@ -22,23 +23,37 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
   s = t;
 }
 
-// exp(x / kT) as mantissa (0.7 .. 1.5) and power of two, |power| <= 2^26: Cody-Waite reduction by
+// occupation of a level at energy E for Fermi level EF at kT > 0
+__device__ __forceinline__ double fermi_dirac(double E, double EF, double kT) {
+  const double x = (E - EF) / kT;
+  const double ex = exp(-fabs(x));
+  return x > 0.0 ? ex / (1.0 + ex) : 1.0 / (1.0 + ex);
+}
+
+// exp(x / kT) as mantissa (0.7 .. 1.5) and power of two for |x / kT| <= FD_QMAX: Cody-Waite reduction by
 // ln 2 = LN2 + LN2L, with the division's remainder carried along, so that the error stays a few ulp
-// for any x / kT (products of two of these never lose what (E - E_F) / kT would keep)
+// up to there (products of two of these never lose what (E - E_F) / kT would keep).  Beyond (power FD_FAR)
+// the power of two would leave its range: the caller takes the difference E - E_F instead.
+constexpr double FD_QMAX = 3.7e8;        // powers below 2^29.0
+constexpr int FD_FAR = 1 << 30;
 __device__ __forceinline__ double exp_parts(double x, double kT, int& p2) {
   constexpr double LN2 = 0.69314718055994530942, LN2L = 2.3190468138462995584e-17;
   const double q = x / kT;
+  if (fabs(q) > FD_QMAX) {   // (infinities too; a NaN goes on and stays one)
+    p2 = FD_FAR;
+    return 1.0;
+  }
   const double lo = fma(-q, kT, x) / kT;
-  const double n = fmin(fmax(rint(q * 1.4426950408889634074), -6e7), 6e7);
-  p2 = (int)n;
-  if (fabs(q) > 4e7) return q == q ? 1.0 : q;   // (also where the remainder overflows)
+  const double n = rint(q * 1.4426950408889634074);
+  p2 = q == q ? (int)n : 0;
   return exp(fma(-n, LN2L, fma(-n, LN2, q)) + lo);
 }
 
 // kT > 0.  f(E, E_F) = 1 / (1 + exp(E / kT) exp(-E_F / kT)): the exponentials are formed once per level
 // and once per Fermi level, and a (level, Fermi level) pair takes a product, a power of two from
 // integer instructions, a multiply-add and a reciprocal (7 FP64 instructions where an exp, a division by
-// kT and one by 1 + exp took about 45), shared by all broadenings.  A CTA's 256 threads are TJ Fermi levels
+// kT and one by 1 + exp took about 45), shared by all broadenings.  A pair of which either exponential is out of
+// range (energies beyond 3.7e8 kT) takes the direct form.  A CTA's 256 threads are TJ Fermi levels
 // x KG groups of k-points (one Fermi level: 256 k-points at a time instead of one thread);
 // KT k-points' levels are staged in shared memory.  Sums in a fixed order (Neumaier).
 constexpr int FD_NT = 256;
@@ -63,25 +78,35 @@ __global__ void __launch_bounds__(FD_NT) ksum_fd_kernel(const double* __restrict
     const int j = j0 + tj;
     const bool on = j < n_EF && kg < KG;
     int pb = 0;
-    const double mb = on ? exp_parts(-E_F[j], kT, pb) : 1.0;
+    const double ef = on ? E_F[j] : 0.0;
+    const double mb = on ? exp_parts(-ef, kT, pb) : 1.0;
     double s[FD_MAXE], c[FD_MAXE];
 #pragma unroll
     for (int e = 0; e < FD_MAXE; ++e) { s[e] = 0.0; c[e] = 0.0; }
     for (int k0 = kb; k0 < ke; k0 += KT) {
       const int nk = min(KT, ke - k0);
       __syncthreads();
-      for (int i = t; i < nk * W; i += FD_NT) sa[i] = exp_parts(E[(size_t)k0 * W + i], kT, se[i]);
-      __syncthreads();
-      if (on)
+      int far = pb == FD_FAR;
+      for (int i = t; i < nk * W; i += FD_NT) {
+        sa[i] = exp_parts(E[(size_t)k0 * W + i], kT, se[i]);
+        far |= se[i] == FD_FAR;
+      }
+      far = __syncthreads_or(far);   // (the same for the CTA: the usual loop has no test per pair)
+      auto sum = [&](auto any_far) {
         for (int kk = kg; kk < nk; kk += KG) {
           const double* O = Om + (size_t)(k0 + kk) * W;
           double v[FD_MAXE];
 #pragma unroll
           for (int e = 0; e < FD_MAXE; ++e) v[e] = 0.0;
           for (int q = 0; q < W; ++q) {
-            const int p2 = max(-1022, min(1000, se[kk * W + q] + pb));
-            const double y = fma(sa[kk * W + q] * mb, __longlong_as_double((long long)(1023 + p2) << 52), 1.0);
-            const double f = recip_nr(y);
+            const int pa = se[kk * W + q];
+            double f;
+            if (decltype(any_far)::value && (pa == FD_FAR || pb == FD_FAR)) {
+              f = fermi_dirac(E[(size_t)(k0 + kk) * W + q], ef, kT);
+            } else {
+              const int p2 = max(-1022, min(1000, pa + pb));
+              f = recip_nr(fma(sa[kk * W + q] * mb, __longlong_as_double((long long)(1023 + p2) << 52), 1.0));
+            }
 #pragma unroll
             for (int e = 0; e < FD_MAXE; ++e)
               if (e < n_eta) v[e] = fma(f, O[e * eta_stride + q], v[e]);
@@ -90,6 +115,11 @@ __global__ void __launch_bounds__(FD_NT) ksum_fd_kernel(const double* __restrict
           for (int e = 0; e < FD_MAXE; ++e)
             if (e < n_eta) neumaier_add(s[e], c[e], v[e]);
         }
+      };
+      if (on) {
+        if (far) sum(std::true_type{});
+        else sum(std::false_type{});
+      }
     }
 #pragma unroll
     for (int e = 0; e < FD_MAXE; ++e) {
