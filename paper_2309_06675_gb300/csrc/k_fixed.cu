@@ -264,8 +264,11 @@ __global__ void __launch_bounds__(512, 1)
   }
 }
 
-// per-matrix exponent with every column norm of U below 2^ue (0 for norms up to 1 + 2^-10), for
-// eigenvectors supplied by the caller; warp per column in turn, CTA per matrix
+// per-matrix exponent with every column norm of U below 2^ue (1 + 2^-34), for eigenvectors supplied by the
+// caller; warp per column in turn, CTA per matrix.  (The tolerance keeps ue = 0, and with it the last bit, for
+// unit columns with the rounding of any eigensolver.  It is below what dH's scale leaves over: the leading 15
+// bits of one dominating diagonal entry and a unit for each other one keep a row's norm below 1 - 2^-31, and rows
+// of several large entries stay further below their matrix's Frobenius norm, so |T| < 1.)
 __global__ void __launch_bounds__(256) unorm_kernel(const double2* __restrict__ U, int W,
                                                     int* __restrict__ ue) {
   __shared__ int s_e;
@@ -294,7 +297,7 @@ __global__ void __launch_bounds__(256) unorm_kernel(const double2* __restrict__ 
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     // norm = sqrt(s) 2^(ex - 1023)
     int f = 0;
-    frexp(sqrt(s) * (1.0 - 0x1p-10), &f);   // < 2^f
+    frexp(sqrt(s) * (1.0 - 0x1p-34), &f);   // < 2^f
     em = max(em, f + ex - 1023);
   }
   if (lane == 0) atomicMax(&s_e, em);
