@@ -165,7 +165,7 @@ struct Plan {
   bool lbuf = false;    // W > SMALL_W_MAX: scratch of the multi-pass kernels
   bool grad = false;    // reverse-mode buffers (kubo_ahc_grad)
   bool iit = false;     // inverse-iteration scratch (separate eigenvector kernel)
-  int zk = 0;           // k-points per sub-batch of the tensor-core rotations (FP64, W > FIX_W_MAX)
+  int zk = 0;           // k-points per sub-batch of the tensor-core FP64 rotations (W > FIX_W_MAX)
   bool lean = false;    // a caller's workspace too small for Z, the iteration scratch and zg (W <= 64)
   bool bisect = false;  // FP64 with eigenvectors: shifts by bisection, eigenvalues as Rayleigh quotients
   bool user_u = false;  // eigenvectors from the caller (kubo_berry_batched): column norms on the device
@@ -193,7 +193,8 @@ struct Plan {
 };
 
 // Per k-point scratch of the W > SMALL_W_MAX kernels, reused by stage: the eigenvectors Z of
-// the tridiagonal, then the FP64 rotation products T, V^x, V^y (the larger of the two).
+// the tridiagonal (with the FP32 modes' compact-WY factors), then the rotation products T, V^x, V^y
+// (FP32, or FP64 for the k-points of a sub-batch).
 size_t large_region_bytes(int W) {
   const size_t WW = (size_t)W * W;
   // (Z and the FP32 compact-WY factors of the U assembly, 256 bytes of alignment per batch
@@ -318,10 +319,13 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
     else if (!p.lean && (!p.model || p.fixup || !f32_rotation(p.precision)))
       p.o_Z = b.take(sizeof(double) * WW * (size_t)std::max(1, p.chunk));
   }
+  // FP64 rotations on the tensor cores: the FP64 modes', and above W = 64 (where berry_fix_kernel ends) the
+  // FP64 redo of the mixed ones.  There T, v^x, v^y lie in the large region, whose Z is not read once U is formed.
   p.zk = 0;
-  if ((p.berry || p.user_u) && !f32_rotation(p.precision) && p.W > FIX_W_MAX && !p.lean) {
+  if ((p.berry || p.user_u) && (!f32_rotation(p.precision) || (p.fixup && p.W > SMALL_W_MAX)) &&
+      p.W > FIX_W_MAX && !p.lean) {
     p.zk = std::min(std::max(1, p.chunk), ZG_BATCH);
-    p.o_zg = b.take(3 * sizeof(double2) * WW * (size_t)p.zk);
+    p.o_zg = p.lbuf ? p.o_L : b.take(3 * sizeof(double2) * WW * (size_t)p.zk);
     p.o_ze = b.take(3 * sizeof(int) * (size_t)p.zk);
   }
   // column norms of the caller's U (up to 48 of them in the unused part of the broadenings' block)
@@ -722,8 +726,8 @@ cudaError_t berry_tc64(const Call& c, const double* E, const double2* U, const i
 }
 
 // kernels of one berry_any call
-int berry_launches(const Plan& p, int n) {
-  if (p.zk > 0) return 7 * ((n + p.zk - 1) / p.zk);   // per sub-batch: two exponents, four products, curvature
+int berry_launches(const Plan& p, int n, bool f32 = false) {
+  if (!f32 && p.zk > 0) return 7 * ((n + p.zk - 1) / p.zk);   // per sub-batch: two exponents, four products, curvature
   return p.W > SMALL_W_MAX ? 5 : 1;
 }
 
@@ -829,7 +833,7 @@ kubo_status run_batch_mixed(Call& c, const Model& md, const KList& kl, double* E
                         rq_eigenvalues(p.precision, p.ql_fp64)));
   }
   {
-    StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n));
+    StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n, f32_rotation(p.precision)));
     KCHECK(berry_any(c, Eout, U, C64 + WW, C64 + 2 * WW, p.Npad, true, kl.n, f32_rotation(p.precision), Om, om_stride));
   }
   return KUBO_OK;
@@ -882,7 +886,7 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
     KCHECK(eigh_vectors(c, kl.n, eb, Eout, U, f32_rotation(p.precision)));
   }
   {
-    StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n));
+    StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n, f32_rotation(p.precision)));
     KCHECK(berry_any(c, Eout, U, Xp, Yp, (int64_t)p.W * p.W, false, kl.n, f32_rotation(p.precision), Om, om_stride));
   }
   return KUBO_OK;
@@ -936,7 +940,7 @@ kubo_status fixup_batch(Call& c, const Model& md, const KList& kl, const double*
   for (int c0 = 0; c0 < cnt; c0 += p.fix_cap) {
     const int nf = std::min(p.fix_cap, cnt - c0);
     KList fl{kid + c0, 0, nf};
-    StageTimer tm(c, KUBO_STAGE_FIXUP, p.W > SMALL_W_MAX ? 11 : 7);
+    StageTimer tm(c, KUBO_STAGE_FIXUP, 6 + berry_launches(p, nf));
     KCHECK(launch_fourier_fp64(md, p.mesh, fl, c.at<double>(p.o_fHp), c.at<double>(p.o_fXp), c.at<double>(p.o_fYp), c.s));
     KCHECK(launch_tridiag(c.at<double>(p.o_fHp), p.W, nf, eb, c.s));
     KCHECK(launch_ql(p.W, nf, eb, st, c.s));
