@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include <array>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -156,6 +157,8 @@ struct Plan {
   bool tc64 = false;                // FP64: step (1) as seven-slice products on the tensor cores
   int fourier_n = 0;                // its k-points when the call has no batch buffers (kubo_bloch)
   int f64_k = 0;                    // k-points per sub-batch of its coefficient slices
+  int f64_cap = INT_MAX;            // the most that leaves the layout within a caller's workspace
+  bool no_tc64 = false;             // its slices do not fit: the FP64-pipe kernel
   int group_m = 8;                  // tensor-core Fourier sum: M tiles rasterised together
   int symv_parts = 4;               // Householder reduction: column partitions of its symv
   bool model = false;   // needs the prepared Fourier basis
@@ -273,12 +276,12 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
       p.o_Xp = b.take(sizeof(double) * (size_t)p.chunk * WW);
       p.o_Yp = b.take(sizeof(double) * (size_t)p.chunk * WW);
       const int nf = std::max(p.chunk, p.fourier_n);
-      p.tc64 = p.precision == KUBO_FP64 && !p.sep && use_tc64(p.W, p.N_R, nf);
+      p.tc64 = p.precision == KUBO_FP64 && !p.sep && !p.no_tc64 && use_tc64(p.W, p.N_R, nf);
       if (p.tc64) {
         p.Npad = tc64_pad_n(p.W);
         p.Kp = tc_pad_k(p.N_R);
         const size_t per_k = (size_t)2 * tc64_slices() * p.Kp;
-        p.f64_k = (int)std::max<size_t>(128, std::min<size_t>((size_t)nf, kTc64CoefBytes / per_k / 128 * 128));
+        p.f64_k = (int)std::max<size_t>(128, std::min<size_t>((size_t)std::min(nf, p.f64_cap), kTc64CoefBytes / per_k / 128 * 128));
         p.o_Bt = b.take((size_t)2 * tc64_slices() * p.Npad * p.Kp);
         p.o_cexp = b.take(sizeof(int) * (size_t)p.Npad);
         p.o_A = b.take(per_k * (size_t)tc_pad_m(p.f64_k));
@@ -382,6 +385,19 @@ void fit_workspace(Plan& p, const kubo_options& o) {
   p.chunk = chunk;
   plan_layout(p, false, 0);
   fit_workspace(p, o);
+}
+
+// kubo_bloch with a caller's workspace, whose size does not depend on its list: the coefficient slices' sub-batch
+// is cut to what is left (the same bits: a row is one k-point), and the FP64-pipe kernel taken where less
+// than a tile per SM would be left of it or the sliced basis alone does not fit.
+void fit_fourier(Plan& p, const kubo_options& o) {
+  if (!o.workspace || p.total <= o.workspace_bytes || !p.tc64) return;
+  const size_t per_k = (size_t)2 * tc64_slices() * p.Kp;
+  const size_t rest = p.total - per_k * (size_t)tc_pad_m(p.f64_k);   // (up to the alignment, which 128 rows keep)
+  const size_t left = o.workspace_bytes > rest ? (o.workspace_bytes - rest) / per_k / 128 * 128 : 0;
+  if (left / 128 * (size_t)(p.Npad / 32) >= 152) p.f64_cap = (int)std::min<size_t>(left, INT_MAX);
+  else p.no_tc64 = true;
+  plan_layout(p, false, 0);
 }
 
 // ------------------------------------------------------------------ device allocations
@@ -1990,6 +2006,7 @@ kubo_status kubo_bloch(const double* H_R, const int32_t* R_vecs, int W, int N_R,
     p.fourier_n = (int)std::min<int64_t>(n_k, 1 << 19);
     p.model = true;
     plan_layout(p, false, 0);
+    fit_fourier(p, o);
     c.s = (cudaStream_t)o.stream;
     c.prof = o.profile;
     r = c.acquire(o);
