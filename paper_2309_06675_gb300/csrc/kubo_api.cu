@@ -159,6 +159,8 @@ struct Plan {
   int f64_k = 0;                    // k-points per sub-batch of its coefficient slices
   int f64_cap = INT_MAX;            // the most that leaves the layout within a caller's workspace
   bool no_tc64 = false;             // its slices do not fit: the FP64-pipe kernel
+  size_t slice_bytes = 0;           // slices of either Fourier sum that no_tc64 does without
+  bool host_io = false;             // buffers for host inputs and outputs (plan_layout's argument)
   int group_m = 8;                  // tensor-core Fourier sum: M tiles rasterised together
   int symv_parts = 4;               // Householder reduction: column partitions of its symv
   bool model = false;   // needs the prepared Fourier basis
@@ -238,6 +240,7 @@ constexpr size_t kTc64MaxBasis = (size_t)16 << 30;
 constexpr int kTc64MinVectors = 24;
 constexpr size_t kTc64SmallBasis = (size_t)256 << 20;
 constexpr size_t kTc64CoefBytes = (size_t)2 << 30;   // coefficient slices of a sub-batch
+constexpr size_t kSliceRetryBytes = (size_t)64 << 20;
 bool use_tc64(int W, int N_R, int64_t n) {
   const size_t basis = (size_t)2 * tc64_slices() * tc64_pad_n(W) * tc_pad_k(N_R);
   if (W < 4 || N_R < 16) return false;
@@ -247,6 +250,8 @@ bool use_tc64(int W, int N_R, int64_t n) {
 
 void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
   (void)n_list_outputs_unused;
+  p.host_io = host_io;
+  p.slice_bytes = 0;
   Bump b;
   const size_t WW = (size_t)p.W * p.W;
   p.o_status = b.take(sizeof(DevStatus));
@@ -285,6 +290,7 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
         p.o_Bt = b.take((size_t)2 * tc64_slices() * p.Npad * p.Kp);
         p.o_cexp = b.take(sizeof(int) * (size_t)p.Npad);
         p.o_A = b.take(per_k * (size_t)tc_pad_m(p.f64_k));
+        p.slice_bytes += (size_t)2 * tc64_slices() * p.Npad * p.Kp + per_k * (size_t)tc_pad_m(p.f64_k);
       }
     }
   }
@@ -346,10 +352,12 @@ void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
     p.o_Ebar = b.take(sizeof(double) * ch * p.W);
     p.o_Mbar = b.take(3 * sizeof(double) * ch * WW);
     p.o_ge = b.take(8 * sizeof(int) * ch);
-    // digit slices of the transposed sum's operands, k-points as its inner index: within 2 GiB
+    // digit slices of the transposed sum's operands, k-points as its inner index: within 2 GiB (no_tc64: 64 MiB)
     const size_t t_row = (size_t)2 * tc64_slices() * (tc64_pad_n(p.W) + tc_pad_m(2 * p.N_h + 1));
-    p.t_k = (int)std::max<size_t>(64, std::min<size_t>(std::min<size_t>(ch, 8192), kTc64CoefBytes / t_row / 64 * 64));
+    const size_t t_max = p.no_tc64 ? kSliceRetryBytes : kTc64CoefBytes;
+    p.t_k = (int)std::max<size_t>(64, std::min<size_t>(std::min<size_t>(ch, 8192), t_max / t_row / 64 * 64));
     const size_t t_cols = (size_t)tc_pad_k(p.t_k);
+    p.slice_bytes += t_row * t_cols;
     p.o_tA = b.take((size_t)2 * tc64_slices() * tc_pad_m(2 * p.N_h + 1) * t_cols);
     p.o_tB = b.take((size_t)2 * tc64_slices() * tc64_pad_n(p.W) * t_cols);
     p.o_texp = b.take(sizeof(int) * (size_t)tc64_pad_n(p.W));
@@ -398,6 +406,16 @@ void fit_fourier(Plan& p, const kubo_options& o) {
   if (left / 128 * (size_t)(p.Npad / 32) >= 152) p.f64_cap = (int)std::min<size_t>(left, INT_MAX);
   else p.no_tc64 = true;
   plan_layout(p, false, 0);
+}
+
+// After a failed allocation: the layout without the tensor-core Fourier sums' slices, if they were enough of it
+// to be worth another attempt (64 MiB); the FP64-pipe kernel, and short sub-batches of the transposed sum, take
+// their place.  False: nothing to gain.
+bool drop_slices(Plan& p) {
+  if (p.no_tc64 || p.slice_bytes < kSliceRetryBytes) return false;
+  p.no_tc64 = true;
+  plan_layout(p, p.host_io, 0);
+  return true;
 }
 
 // ------------------------------------------------------------------ device allocations
@@ -478,12 +496,13 @@ struct Call {
       ws = (char*)o.workspace;
       return KUBO_OK;
     }
-    retain_pool_memory(p.total);
-    if (lib_malloc_async((void**)&ws, p.total, s) != cudaSuccess) {
+    if (lib_malloc_async((void**)&ws, p.total, s) != cudaSuccess && !(drop_slices(p) && lib_malloc_async((void**)&ws, p.total, s) == cudaSuccess)) {
       cudaGetLastError();
       ws = nullptr;
       return KUBO_ERR_OOM;
     }
+    cudaGetLastError();
+    retain_pool_memory(p.total);
     owned = true;
     return KUBO_OK;
   }
@@ -1732,15 +1751,18 @@ kubo_status kubo_ahc_batched(kubo_problem* probs, int n_probs, const kubo_option
       cand_C.push_back(chunk > 0 ? chunk : 65536);
     }
     layout_tables(br);
-    size_t need = 0;
-    for (int cs : cand_S)
-      for (int cc : cand_C) {
-        layout_batch(br, cs, cc, n_eta);
-        need = std::max(need, br.total);
-      }
-    size_t probe_doubles = 0;
+    size_t need = 0, probe_doubles = 0, probe_off = 0;
     for (const auto& j : br.jobs) probe_doubles += (size_t)j.p.n_eta * j.p.n_EF;
-    const size_t probe_off = align_up(need);
+    auto size_layouts = [&]() {
+      need = 0;
+      for (int cs : cand_S)
+        for (int cc : cand_C) {
+          layout_batch(br, cs, cc, n_eta);
+          need = std::max(need, br.total);
+        }
+      probe_off = align_up(need);
+    };
+    size_layouts();
     // the batch runs behind the caller's stream on a stream of its own (the legacy default
     // stream cannot be captured), and the call returns when it is done
     {
@@ -1759,8 +1781,16 @@ kubo_status kubo_ahc_batched(kubo_problem* probs, int n_probs, const kubo_option
     }
     if (lib_malloc_async((void**)&ws, probe_off + sizeof(double) * probe_doubles, origin) != cudaSuccess) {
       cudaGetLastError();
-      ws = nullptr;
-      return finish(KUBO_ERR_OOM);
+      // once more without the slices of the FP64 Fourier sums, if they were a good part of it
+      const size_t with = need;
+      for (auto& j : br.jobs) j.p.no_tc64 = true;
+      size_layouts();
+      if (with < need + kSliceRetryBytes ||
+          lib_malloc_async((void**)&ws, probe_off + sizeof(double) * probe_doubles, origin) != cudaSuccess) {
+        cudaGetLastError();
+        ws = nullptr;
+        return finish(KUBO_ERR_OOM);
+      }
     }
     const int max_S = *std::max_element(cand_S.begin(), cand_S.end());
     streams.assign(max_S, nullptr);
