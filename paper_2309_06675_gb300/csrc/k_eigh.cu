@@ -634,11 +634,6 @@ __global__ void __launch_bounds__(32) ql_kernel(int W, int n, EighBufs b, DevSta
 //     previous vectors, normalisation.  Coincident eigenvalues are separated by 10 eps ||T||_1.
 //   * a warp at a time: the factors of 32 vectors live lane-interleaved in the U region;
 //     the iterate lives in its column of Z.
-__device__ __forceinline__ unsigned long long order_key(double x) {
-  unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
-
 // double2 slots of the U region: the W x (W+1) matrix, or the inverse-iteration factors of
 // 32 vectors (4 arrays of W x 32 doubles)
 __host__ __device__ __forceinline__ size_t bt_u_slots(int W) {
@@ -669,12 +664,7 @@ __global__ void __launch_bounds__(NT) backtransform_kernel(int W, EighBufs b, do
   // ascending order of the eigenvalues (ties broken by index)
   for (int j = t; j < W; j += NT) {
     const double lj = lk[j];
-    const unsigned long long kj = order_key(lj);
-    int rnk = 0;
-    for (int i = 0; i < W; ++i) {
-      const unsigned long long ki = order_key(lk[i]);
-      rnk += (ki < kj) || (ki == kj && i < j);
-    }
+    const int rnk = sorted_rank(lk, W, j);
     rank[j] = rnk;
     ws[rnk] = lj;
     Eout[k * W + rnk] = lj;

@@ -601,11 +601,6 @@ __global__ void __launch_bounds__(32) ql_df_kernel(int W, int n, EighBufs b, Dev
 }
 
 // ------------------------------------------------------------------ inverse iteration in double-float
-__device__ __forceinline__ unsigned long long order_key(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
-
 // deterministic start vector in [0.5, 1.5) from an integer hash of (row, vector): 23 hash bits
 // as the mantissa of a number in [1, 2), minus 1/2
 __device__ __forceinline__ float iit_start_f(int i, int j) {
@@ -653,12 +648,7 @@ __global__ void __launch_bounds__(128) iit_df_kernel(int W, int n, EighBufs b,
     const double* lk = b.lam + k * W;
     if (t < W) {
       const double lj = lk[t];
-      const unsigned long long kj = order_key(lj);
-      int rnk = 0;
-      for (int i = 0; i < W; ++i) {
-        const unsigned long long ki = order_key(lk[i]);
-        rnk += (ki < kj) || (ki == kj && i < t);
-      }
+      const int rnk = sorted_rank(lk, W, t);
       ws[rnk] = df_split_bits(lj);
       Eout[k * W + rnk] = lj;
       dd[t] = df_split_bits(b.d[k * W + t]);

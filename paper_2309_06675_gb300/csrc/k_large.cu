@@ -27,11 +27,6 @@ constexpr int IIT_SOLVES = 2;
 constexpr int MAXE = 8;
 constexpr int IIT_SMS = 152;   // GB300 SM count: persistent inverse-iteration grid
 
-__device__ __forceinline__ unsigned long long order_key(double x) {
-  unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
-
 // ------------------------------------------------------------------ inverse iteration
 // Persistent: CTA b handles the k-points kpc b .. kpc b + kpc - 1, then kpc gridDim.x further on;
 // kpc = blockDim / W k-points share the CTA (128 threads up to W = 64, W rounded up to a warp above:
@@ -70,12 +65,7 @@ __global__ void __launch_bounds__(LW_MAX, 8) iit_kernel(int W, int n, EighBufs b
     if (live) {
       const double* lam = b.lam + k * W;
       const double lj = lam[j];
-      const unsigned long long kj = order_key(lj);
-      int rnk = 0;
-      for (int i = 0; i < W; ++i) {
-        const unsigned long long ki = order_key(lam[i]);
-        rnk += (ki < kj) || (ki == kj && i < j);
-      }
+      const int rnk = sorted_rank(lam, W, j);
       ws[rnk] = lj;
       Eout[k * W + rnk] = lj;
       dd[j] = b.d[k * W + j];

@@ -343,7 +343,8 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
           a = a2 * ra;
           u[q] = make_double2(bj.x * ra, bj.y * ra);
         }
-        b.e[kw * W + j] = badk ? nan : fx::scale_pow2(a, ek - fx::BITS);
+        // (an infinite or NaN entry: T = NaN I, which the QL iteration leaves as it is)
+        b.e[kw * W + j] = badk ? 0.0 : fx::scale_pow2(a, ek - fx::BITS);
       }
       pr = cmul(pr, u[q]);
     }

@@ -112,6 +112,24 @@ __device__ __forceinline__ double recip_nr(double d) {
   return fma(r, e, r);
 }
 
+// Position of x[j] among x[0 .. W - 1] in ascending order, equal ones by their index: a permutation for any
+// contents, NaN included.  The numbers are read and compared as integers throughout.  (Loaded as doubles and
+// reinterpreted afterwards, NaNs of the same bits were not found equal in the compiled kernels: all of them
+// took position 0 and the other positions were left unwritten.)
+__device__ __forceinline__ int sorted_rank(const double* __restrict__ x, int W, int j) {
+  const unsigned long long* u = reinterpret_cast<const unsigned long long*>(x);
+  auto key = [](unsigned long long v) {
+    return v ^ ((unsigned long long)((long long)v >> 63) | 0x8000000000000000ull);
+  };
+  const unsigned long long kj = key(u[j]);
+  int r = 0;
+  for (int i = 0; i < W; ++i) {
+    const unsigned long long ki = key(u[i]);
+    r += (ki < kj) || (ki == kj && i < j);
+  }
+  return r;
+}
+
 // start vector of the inverse iterations: 0.5 + (h >> 8) 2^-24 in [0.5, 1.5) from an integer hash
 // of (row, vector); 1 + (h >> 8) 2^-24 is assembled from its bits (exponent of 1, the 24-bit
 // integer as the leading mantissa bits) and 0.5 subtracted exactly, instead of an integer ->
