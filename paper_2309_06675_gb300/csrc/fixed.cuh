@@ -21,6 +21,8 @@ namespace fx {
 constexpr int BITS = 59;   // fractional bits of a full-scale operand
 constexpr int LB = 28;     // bits of the low limb
 
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
+
 // round(x 2^s) for |x| 2^s < 2^60, from the bit pattern (round half up of the magnitude)
 __device__ __forceinline__ long long from_double(double x, int s) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);

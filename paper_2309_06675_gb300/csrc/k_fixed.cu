@@ -341,7 +341,8 @@ __global__ void __launch_bounds__(RF_NT, 2)
     sp[j] = fx::climbs(fx::from_double(p.x, 58), fx::from_double(p.y, 58));
     sf[j] = sqrt(0.5 * b.tau[k * W + j]);
   }
-  __syncthreads();
+  // (a column of Z with a NaN is NaN throughout, from its normalisation: the first row tells)
+  const bool any_bad = __syncthreads_or(t < ncol && !fx::finite(Zk[cb0 + t]));
   for (int idx = t; idx < W * ncol; idx += nt) {
     const int r = (int)dC.div(idx), c = idx - r * ncol;
     const int2 z = fx::limbs(fx::from_double(Zk[(size_t)r * W + cb0 + c], 58));
@@ -463,7 +464,9 @@ __global__ void __launch_bounds__(RF_NT, 2)
   for (int idx = t; idx < W * ncol; idx += nt) {
     const int r = (int)dC.div(idx), c = idx - r * ncol;
     const int4 u = su[r * LD + c];
-    Uk[(size_t)r * W + cb0 + c] = make_double2(fx::to_double(fx::value(u.x, u.y), -58), fx::to_double(fx::value(u.z, u.w), -58));
+    double2 v = make_double2(fx::to_double(fx::value(u.x, u.y), -58), fx::to_double(fx::value(u.z, u.w), -58));
+    if (any_bad && !fx::finite(Zk[cb0 + c])) v.x = v.y = __longlong_as_double(0x7FF8000000000000ll);
+    Uk[(size_t)r * W + cb0 + c] = v;
   }
 }
 
@@ -496,11 +499,13 @@ __global__ void __launch_bounds__(256) reflect_small_kernel(int W, int n, int kp
   __syncthreads();
   if (!live) return;
   int4 u[WM];
+  bool bad = false;   // an infinite or NaN entry of Z
 #pragma unroll
   for (int r = 0; r < WM; ++r) {
     u[r] = make_int4(0, 0, 0, 0);
     if (r < W) {
       const double z = Z[(size_t)k * W * W + (size_t)r * W + c];
+      bad |= !fx::finite(z);
       const double2 p = b.phase[k * W + r];
       u[r] = fx::climbs(fx::from_double(p.x * z, 58), fx::from_double(p.y * z, 58));
     }
@@ -531,9 +536,12 @@ __global__ void __launch_bounds__(256) reflect_small_kernel(int W, int n, int kp
   double2* Uk = Uout + (size_t)k * W * W;
 #pragma unroll
   for (int r = 0; r < WM; ++r)
-    if (r < W)
-      Uk[r * W + c] = make_double2(fx::to_double(fx::value(u[r].x, u[r].y), -58),
-                                   fx::to_double(fx::value(u[r].z, u[r].w), -58));
+    if (r < W) {
+      double2 v = make_double2(fx::to_double(fx::value(u[r].x, u[r].y), -58),
+                               fx::to_double(fx::value(u[r].z, u[r].w), -58));
+      if (bad) v.x = v.y = __longlong_as_double(0x7FF8000000000000ll);
+      Uk[r * W + c] = v;
+    }
 }
 
 }  // namespace
