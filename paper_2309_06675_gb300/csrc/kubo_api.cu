@@ -1244,14 +1244,21 @@ struct Job {
   size_t o_tables = 0;  // offset of neg / pairs / Rh / status in the tables region
 };
 
-// Estimated device time of a model in units of FP64 flops: the FP64 pipe runs the eigensolver
-// (and, in FP64 mode, everything else); tensor-core and FP32 work is discounted by its rate.
+// Estimated device time of a model in units of FP64-pipe flops (1.2 TFLOP/s).  FP64 mode: the Fourier sum on the
+// tensor cores at 0.03 of that pipe's time (W = 64, N_R = 1331, 4,096 k-points: 3.4 of 112 ms), the reduction at 0.6,
+// the eigenvectors at 0.5 and the rotations at 0.5 (integer pipe) or 0.1 (tensor cores); it gives 12.5 ms for that
+// call of 13.2, and 22 of 28 at W = 97, N_R = 343, 2,744 k-points.  Mixed modes: the FP64 pipe runs the reduction;
+// tensor-core and FP32 work is discounted by its rate.
 double job_cost(const Plan& p) {
   const double W = p.W, NR = p.N_R, Nk = (double)p.mesh.Nk;
-  const double fourier = 6.0 * NR * W * W * (tc_fourier(p.precision) ? 10.0 / 1500.0 : 1.0);
+  const bool f64 = p.precision == KUBO_FP64;
+  const bool tc64 = f64 && !p.no_tc64 && use_tc64(p.W, p.N_R, p.mesh.Nk);
+  const double fourier = 6.0 * NR * W * W * (tc_fourier(p.precision) ? 10.0 / 1500.0 : tc64 ? 0.03 : 1.0);
   // the double-float eigensolver runs about 2.5x faster than the FP64 one at W = 64
-  const double eig = (16.0 / 3.0 * W * W * W + 72.0 * W * W) * (df_eigh(p.precision) ? 0.4 : 1.0);
-  const double rot = 24.0 * W * W * W * (f32_rotation(p.precision) ? 1.0 / 48.0 : 1.0);
+  const double eig = (16.0 / 3.0 * W * W * W + 72.0 * W * W) * (df_eigh(p.precision) ? 0.4 : f64 ? 0.6 : 1.0) +
+                     (f64 ? 0.5 * 8.0 * W * W * W : 0.0);
+  const double rot = 24.0 * W * W * W *
+                     (f32_rotation(p.precision) ? 1.0 / 48.0 : p.W > FIX_W_MAX ? 0.1 : 0.5);
   return Nk * (fourier + eig + rot + 1e4);   // + per-k fixed cost (launch/latency share)
 }
 
