@@ -1728,7 +1728,7 @@ kubo_status kubo_ahc_batched(kubo_problem* probs, int n_probs, const kubo_option
     br.kp.symv_parts = sc.symv_parts > 0 ? sc.symv_parts : 4;
     br.kp.rotation = o.layout_unpadded ? 2 : (sc.rotation > 0 ? sc.rotation : o.rotation_tc);
     const bool tune_gm = sc.tune && sc.fourier_group_m == 0 && tc_fourier(o.precision);
-    const bool tune_sp = sc.tune && sc.symv_parts == 0;
+    const bool tune_sp = sc.tune && sc.symv_parts == 0 && o.precision != KUBO_FP64;   // (its reduction has none)
     const bool tune_rot = sc.tune && sc.rotation == 0 && !o.layout_unpadded && o.rotation_tc == 0 &&
                           f32_rotation(o.precision);
     std::vector<int64_t> sig;
