@@ -2147,7 +2147,8 @@ kubo_status kubo_berry_batched(const double* E, const double* U, const double* d
     c.s = (cudaStream_t)o.stream;
     kubo_status r = c.acquire(o);
     if (r != KUBO_OK) return r;
-    if (cudaMemsetAsync(c.at<char>(p.o_status), 0, sizeof(DevStatus), c.s) != cudaSuccess) r = KUBO_ERR_CUDA;
+    // (only the tensor-core products have a wait that can give up)
+    if (p.zk > 0 && cudaMemsetAsync(c.at<char>(p.o_status), 0, sizeof(DevStatus), c.s) != cudaSuccess) r = KUBO_ERR_CUDA;
     if (r == KUBO_OK) r = upload_etas(c, o, eta);
     const size_t WW = (size_t)W * W;
     const int64_t step = p.chunk;
@@ -2159,7 +2160,7 @@ kubo_status kubo_berry_batched(const double* E, const double* U, const double* d
         r = KUBO_ERR_CUDA;
       }
     }
-    if (r == KUBO_OK) r = read_status(c);
+    if (r == KUBO_OK && p.zk > 0) r = read_status(c);
     c.release();
     if (cudaStreamSynchronize(c.s) != cudaSuccess && r == KUBO_OK) r = KUBO_ERR_CUDA;
     return r;
