@@ -79,8 +79,17 @@ __device__ __forceinline__ int4 pin(int4 v) {
 __device__ __forceinline__ long long fold(long long h, long long m) {
   return h + ((m + (1ll << (LB - 1))) >> LB);
 }
-// round(v 2^-s), s >= 1
-__device__ __forceinline__ long long rshift(long long v, int s) { return (v + (1ll << (s - 1))) >> s; }
+// round(v 2^-s), s >= 1, halves to the even neighbour: every 2^s-th v is a half, and always up they would add
+// a constant to whatever the results are summed into
+__device__ __forceinline__ long long rshift(long long v, int s) {
+  return (v + (1ll << (s - 1)) - 1 + ((v >> s) & 1)) >> s;
+}
+// round((hh + cross 2^-28) 2^-s), s >= 1: rounded once.  (fold() and then a shift by one bit rounds every other value
+// up from a half: a quarter unit too much on average in every entry of a rank-2 update, 46 units in
+// the matrix norm at W = 128 where the roundings themselves are 9.)
+__device__ __forceinline__ long long fold_shift(long long h, long long m, int s) {
+  return (h + (m >> LB) + (1ll << (s - 1))) >> s;
+}
 
 // v 2^e (normal range) with the power of two added to the exponent field
 __device__ __forceinline__ double to_double(long long v, int e) {

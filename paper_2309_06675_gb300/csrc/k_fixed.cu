@@ -184,8 +184,8 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
         for (int j = 0; j < TN; ++j)
           if (ty + NY * i < W && tx + NX * j < W)
-            sA[row[i] * LD + col[j]] = fx::climbs(fx::rshift(fx::fold(acc[i][j].rh, acc[i][j].rm), 2),
-                                                  fx::rshift(fx::fold(acc[i][j].ih, acc[i][j].im), 2));
+            sA[row[i] * LD + col[j]] = fx::climbs(fx::fold_shift(acc[i][j].rh, acc[i][j].rm, 2),
+                                                  fx::fold_shift(acc[i][j].ih, acc[i][j].im, 2));
     __syncthreads();
     // ---- v = U^dagger T, the pairs n < m only
 #pragma unroll
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(RF_NT, 2)
     long long rh = 0, rm = 0, ih = 0, im = 0;
     fx::mad(rh, p.x, z.x); fx::mad(rm, p.x, z.y); fx::mad(rm, p.y, z.x);
     fx::mad(ih, p.z, z.x); fx::mad(im, p.z, z.y); fx::mad(im, p.w, z.x);
-    su[r * LD + c] = fx::climbs(fx::rshift(fx::fold(rh, rm), 2), fx::rshift(fx::fold(ih, im), 2));
+    su[r * LD + c] = fx::climbs(fx::fold_shift(rh, rm, 2), fx::fold_shift(ih, im, 2));
   }
   const int nblk = rf_blocks(W), nref = W - 2;
   // stage block bk: rows j0 + 1 .. W - 1 of its reflectors (zero above each one's first row)
@@ -462,12 +462,12 @@ __global__ void __launch_bounds__(RF_NT, 2)
       if (act)
 #pragma unroll 1
         for (int r = j0 + 1 + q; r < W; r += 4) {
-          // u + sum w (-h) / 2: the sums start at 2 u and the roundings' halves
+          // u + sum w (-h) / 2, rounded once: the sums start at 2 u and the half
           const int4 u = su[r * LD + c];
           fx::Acc d;
           d.rh = (long long)u.x * (1 << (fx::LB + 1)) + (2 * u.y + 1);
           d.ih = (long long)u.z * (1 << (fx::LB + 1)) + (2 * u.w + 1);
-          d.rm = d.im = 1 << (fx::LB - 1);
+          d.rm = d.im = 0;
 #pragma unroll
           for (int a = 0; a < RF_NB; ++a) {
             const int4 x = w[r * RF_NB + a];
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(256) reflect_small_kernel(int W, int n, int kp
         fx::cmadc(s, w, -w.z, -w.w, u[r]);
       }
     // h = w^dagger u (units 2^-60), u -= 2 w h
-    const int4 h = fx::climbs(fx::rshift(fx::fold(s.rh, s.rm), 2), fx::rshift(fx::fold(s.ih, s.im), 2));
+    const int4 h = fx::climbs(fx::fold_shift(s.rh, s.rm, 2), fx::fold_shift(s.ih, s.im, 2));
 #pragma unroll
     for (int r = 1; r < WM; ++r)
       if (r < W && r > j) {
@@ -549,8 +549,8 @@ __global__ void __launch_bounds__(256) reflect_small_kernel(int W, int n, int kp
         fx::Acc d;
         fx::zero(d);
         fx::cmad(d, w, -w.z, -w.w, fx::pin(h));
-        u[r] = fx::climbs(fx::value(u[r].x, u[r].y) - fx::rshift(fx::fold(d.rh, d.rm), 1),
-                          fx::value(u[r].z, u[r].w) - fx::rshift(fx::fold(d.ih, d.im), 1));
+        u[r] = fx::climbs(fx::value(u[r].x, u[r].y) - fx::fold_shift(d.rh, d.rm, 1),
+                          fx::value(u[r].z, u[r].w) - fx::fold_shift(d.ih, d.im, 1));
       }
   }
   double2* Uk = Uout + (size_t)k * W * W;

@@ -6,7 +6,10 @@
 // numbers relative to a power of two above its Frobenius norm, which the reduction's unitary
 // similarities never exceed; its symmetric product and its rank-2 update are sums of fixed-point
 // products.  A rounding is 2^-60 of that norm, at most 2^-57 of the spectral norm at W = 64, where an
-// FP64 update rounds every entry to 2^-54 of itself several times.  Only what one warp does per
+// FP64 update rounds every entry to 2^-54 of itself several times.  (Each is rounded once, to the nearest: see
+// fold_shift() for what a bias costs.  Against an 80-bit reference, geometric means over 144 k-points of random models, FP64
+// reduction -> this one: largest error of a k-point's eigenvalues 1.4e-15 -> 5.7e-16 of the norm at W = 64, 2.3e-15 -> 7.5e-16
+// at 128; of its curvatures 8.0e-14 -> 3.6e-14 and 2.4e-13 -> 1.4e-13 of the largest.)  Only what one warp does per
 // column (the column's norm, the Householder vector's scale) is FP64.
 //
 // KP k-points per CTA, TPK threads each (2 x 128 at W <= 64, 4 x 64 at 32, 8 x 32 at 16, 16 x 16 at 8,
@@ -137,8 +140,8 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
           const int4 hp = fx::pin(h0), wp = fx::pin(w0);
           fx::cmadc(acc, hp, -hp.z, -hp.w, wr);   // w_r conj(h_0) + h_r conj(w_0), units 2^-61
           fx::cmadc(acc, wp, -wp.z, -wp.w, hr);
-          vx -= fx::rshift(fx::fold(acc.rh, acc.rm), 1);
-          vy -= fx::rshift(fx::fold(acc.ih, acc.im), 1);
+          vx -= fx::fold_shift(acc.rh, acc.rm, 1);
+          vy -= fx::fold_shift(acc.ih, acc.im, 1);
           *pa = fx::climbs(vx, vy);
         }
         xr[q] = (double)vx;
@@ -258,7 +261,7 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
           fx::mad(rh, Kp.x, wq.x); fx::mad(rm, Kp.x, wq.y); fx::mad(rm, Kp.y, wq.x);
           fx::mad(ih, Kp.x, wq.z); fx::mad(im, Kp.x, wq.w); fx::mad(im, Kp.y, wq.z);
           int4* s4 = reinterpret_cast<int4*>(spk);
-          s4[r] = fx::climbs(pr[q] - fx::rshift(fx::fold(rh, rm), 2), pi[q] - fx::rshift(fx::fold(ih, im), 2));
+          s4[r] = fx::climbs(pr[q] - fx::fold_shift(rh, rm, 2), pi[q] - fx::fold_shift(ih, im, 2));
           s4[W + r] = w[q];
         }
       }
@@ -288,8 +291,8 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
         fx::cmadc(acc, wc, -wc.z, -wc.w, hr);
         int4* pa = &Ag[tri(o + r, o + c)];
         const int4 a = *pa;
-        *pa = fx::climbs(fx::value(a.x, a.y) - fx::rshift(fx::fold(acc.rh, acc.rm), 1),
-                         fx::value(a.z, a.w) - fx::rshift(fx::fold(acc.ih, acc.im), 1));
+        *pa = fx::climbs(fx::value(a.x, a.y) - fx::fold_shift(acc.rh, acc.rm, 1),
+                         fx::value(a.z, a.w) - fx::fold_shift(acc.ih, acc.im, 1));
       }
     }
     __syncthreads();
