@@ -12,6 +12,10 @@
 // at 128; of its curvatures 8.0e-14 -> 3.6e-14 and 2.4e-13 -> 1.4e-13 of the largest.)  Only what one warp does per
 // column (the column's norm, the Householder vector's scale) is FP64.
 //
+// Uncoupled blocks (consecutive orbitals without a matrix element to the others: layers, spins) whose rows' largest
+// entries differ by 2^4 or more have a scale each, so that a small block keeps its own relative accuracy beside a
+// large one: a reflector never leaves its block.
+//
 // KP k-points per CTA, TPK threads each (2 x 128 at W <= 64, 4 x 64 at 32, 8 x 32 at 16, 16 x 16 at 8,
 // 1 x 256 or 384 above 64); warp 0 runs the scalar steps of all KP k-points at once, 32 / KP lanes each.
 // Per column i with reflector I - 2 w w^dagger (w a unit vector, kept in column i of A):
@@ -40,6 +44,22 @@ __host__ __device__ constexpr size_t fix_bytes_per_k(int W, int TPK) {
   return ((size_t)W * (W + 1) / 2 + sp_len(W, TPK) + W) * 16;
 }
 
+// 2^e above the Frobenius norm: |entries|^2 add up to at most sq 2^(2 (emax - 1037))
+__device__ __forceinline__ int norm_exp(int emax, unsigned long long sq) {
+  return sq == 0ull ? 0 : emax - 1037 + ((64 - __clzll((long long)sq) + 1) >> 1);
+}
+// an entry's part of that sum: hx, hy the upper halves of its parts' magnitudes (m + 1 above the 15 leading
+// bits at exponent emax)
+__device__ __forceinline__ unsigned long long norm_part(unsigned hx, unsigned hy, int emax) {
+  const int sx = emax - (int)(hx >> 20), sy = emax - (int)(hy >> 20);
+  const unsigned m = (hx && sx < 15 ? (((hx & 0xFFFFFu) | 0x100000u) >> 6) >> sx : 0u) + 1u;
+  const unsigned l = (hy && sy < 15 ? (((hy & 0xFFFFFu) | 0x100000u) >> 6) >> sy : 0u) + 1u;
+  return 2ull * ((hx ? m * m : 0u) + (unsigned long long)(hy ? l * l : 0u));   // (diagonal: twice its share)
+}
+__device__ __forceinline__ unsigned upper_mag(double x) { return (unsigned)(mag_bits(x) >> 32); }
+
+constexpr int SPLIT_SPREAD = 4;   // binary orders between rows from which uncoupled blocks have their own scale
+
 template <int KP, int TPK, int MINB>
 __global__ void __launch_bounds__(KP* TPK, MINB)
     tridiag_fix_kernel(const double* __restrict__ Hp, int64_t ld, int W, int n, EighBufs b) {
@@ -56,10 +76,12 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
   __shared__ unsigned long long s_sq[KP];
   __shared__ unsigned s_max[KP];
   __shared__ int s_act[2][KP];   // of the odd and of the even columns
+  __shared__ int s_lo[KP];       // exponent of the smallest row; from then on: blocks have their own scale
   const int64_t k = (int64_t)blockIdx.x * KP + g;
   const bool live = k < n;
 
-  if (t < KP) { s_sq[t] = 0ull; s_max[t] = 0u; }
+  if (t < KP) { s_sq[t] = 0ull; s_max[t] = 0u; s_lo[t] = 0; }
+  int open = 0;   // an element beside the diagonal is zero
   for (int r = 1 + warp; r < W; r += KP * TPK / 32)
     for (int c = lane; c < r; c += 32) rowtab[r * (r - 1) / 2 + c] = (unsigned char)r;
   __syncthreads();
@@ -83,28 +105,94 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
     __syncthreads();
     const int emax = (int)(s_max[g] >> 20);
     unsigned long long s = 0ull;
-    if (live)
+    if (live) {
       for (int idx = th; idx < NA; idx += TPK) {
         const double2 a = Ad[idx];
-        const unsigned hx = (unsigned)(mag_bits(a.x) >> 32), hy = (unsigned)(mag_bits(a.y) >> 32);
-        const int sx = emax - (int)(hx >> 20), sy = emax - (int)(hy >> 20);
-        const unsigned m = (hx && sx < 15 ? (((hx & 0xFFFFFu) | 0x100000u) >> 6) >> sx : 0u) + 1u;
-        const unsigned l = (hy && sy < 15 ? (((hy & 0xFFFFFu) | 0x100000u) >> 6) >> sy : 0u) + 1u;
-        s += 2ull * ((hx ? m * m : 0u) + (unsigned long long)(hy ? l * l : 0u));   // (diagonal: twice its share)
+        s += norm_part(upper_mag(a.x), upper_mag(a.y), emax);
       }
+      for (int r = 1 + th; r < W; r += TPK) {
+        const double2 a = Ad[tri(r, r - 1)];
+        open |= (mag_bits(a.x) | mag_bits(a.y)) == 0ull;
+      }
+    }
     if (s) atomicAdd(&s_sq[g], s);
-    __syncthreads();
+    open = __syncthreads_or(open);
   }
   const int emax = (int)(s_max[g] >> 20);
   const bool bad = emax == 0x7FF;
-  const unsigned long long s2all = s_sq[g];
-  const int e = bad || s2all == 0ull ? 0 : emax - 1037 + ((64 - __clzll((long long)s2all) + 1) >> 1);
+  const int e = bad ? 0 : norm_exp(emax, s_sq[g]);
+  if (open) {   // (the same for the CTA)
+    // a thread per row, tables in the place of the partial sums: the first column with an entry, the first row
+    // of the row's block, that block's largest entry and sum of squares
+    unsigned long long* bsq = reinterpret_cast<unsigned long long*>(sp);
+    int* first = reinterpret_cast<int*>(bsq + W);
+    unsigned* bmax = reinterpret_cast<unsigned*>(first + W);
+    int* start = reinterpret_cast<int*>(bmax + W);
+    const double2* Ad = reinterpret_cast<const double2*>(A);
+    const bool row = live && !bad && th < W;   // (W <= TPK for every instance)
+    unsigned rowmax = 0u;
+    if (th == 0) s_lo[g] = 0x7FF;
+    __syncthreads();
+    if (row) {
+      int f = th;
+      for (int c = th; c >= 0; --c) {
+        const double2 a = Ad[tri(th, c)];
+        if ((mag_bits(a.x) | mag_bits(a.y)) != 0ull) f = c;
+        rowmax = max(rowmax, max(upper_mag(a.x), upper_mag(a.y)));
+      }
+      for (int i = th + 1; i < W; ++i) {
+        const double2 a = Ad[tri(i, th)];
+        rowmax = max(rowmax, max(upper_mag(a.x), upper_mag(a.y)));
+      }
+      first[th] = f;
+      bmax[th] = 0u;
+      bsq[th] = 0ull;
+      if (rowmax >> 20) atomicMin(&s_lo[g], (int)(rowmax >> 20));
+    }
+    __syncthreads();
+    const bool apart = live && !bad && emax - s_lo[g] >= SPLIT_SPREAD;
+    if (__syncthreads_or(apart)) {
+      const bool mine = apart && row;
+      if (mine) {   // the last row up to this one from which on no row reaches in front of it
+        int m = W, b0 = 0;
+        for (int i = W - 1; i > 0; --i) {
+          m = min(m, first[i]);
+          if (i <= th && m >= i) { b0 = i; break; }
+        }
+        start[th] = b0;
+        atomicMax(&bmax[b0], rowmax >> 20);
+      }
+      __syncthreads();
+      if (mine) {
+        const int b0 = start[th], em = (int)bmax[b0];
+        unsigned long long s = 0ull;
+        for (int c = b0; c <= th; ++c) {
+          const double2 a = Ad[tri(th, c)];
+          s += norm_part(upper_mag(a.x), upper_mag(a.y), em);
+        }
+        atomicAdd(&bsq[b0], s);
+      }
+      __syncthreads();
+      // the rows' exponents, kept in lam until the outputs are scaled back
+      if (mine) b.lam[k * W + th] = (double)norm_exp((int)bmax[start[th]], bsq[start[th]]);
+    }
+    if (th == 0) s_lo[g] = apart ? 1 : 0;
+    __syncthreads();
+  }
+  const bool split = s_lo[g] != 0;
   if (live) {
     const double2* Ad = reinterpret_cast<const double2*>(A);
     for (int idx = th; idx < NA; idx += TPK) {
       const double2 a = Ad[idx];
+      int ea = e;
+      if (split) {
+        int r = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+        while (tri(r, 0) > idx) --r;
+        while (tri(r + 1, 0) <= idx) ++r;
+        ea = (int)b.lam[k * W + r];
+      }
       A[idx] = bad ? make_int4(0, 0, 0, 0)
-                   : fx::climbs(fx::from_double(a.x, fx::BITS - e), fx::from_double(a.y, fx::BITS - e));
+                   : fx::climbs(fx::from_double(a.x, fx::BITS - ea), fx::from_double(a.y, fx::BITS - ea));
     }
   }
   __syncthreads();
@@ -304,7 +392,8 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
     double* dout = b.d + k * W;
     for (int j = th; j < W; j += TPK) {
       const int4 a = A[tri(j, j)];
-      dout[j] = bad ? nan : fx::scale_pow2((double)fx::value(a.x, a.y), e - fx::BITS);
+      const int ea = split ? (int)b.lam[k * W + j] : e;
+      dout[j] = bad ? nan : fx::scale_pow2((double)fx::value(a.x, a.y), ea - fx::BITS);
       if (j >= W - 2) b.tau[k * W + j] = 0.0;
     }
     double2* rout = b.refl + (size_t)k * W * W;
@@ -325,7 +414,8 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
     const int emk = (int)(s_max[kk] >> 20);
     const unsigned long long sqk = s_sq[kk];
     const bool badk = emk == 0x7FF;
-    const int ek = badk || sqk == 0ull ? 0 : emk - 1037 + ((64 - __clzll((long long)sqk) + 1) >> 1);
+    const int ek = badk ? 0 : norm_exp(emk, sqk);
+    const bool splitk = s_lo[kk] != 0;
     double2 u[4], pr = make_double2(1.0, 0.0);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -347,7 +437,8 @@ __global__ void __launch_bounds__(KP* TPK, MINB)
           u[q] = make_double2(bj.x * ra, bj.y * ra);
         }
         // (an infinite or NaN entry: T = NaN I, which the QL iteration leaves as it is)
-        b.e[kw * W + j] = badk ? 0.0 : fx::scale_pow2(a, ek - fx::BITS);
+        const int ea = splitk ? (int)b.lam[kw * W + j] : ek;
+        b.e[kw * W + j] = badk ? 0.0 : fx::scale_pow2(a, ea - fx::BITS);
       }
       pr = cmul(pr, u[q]);
     }
