@@ -417,11 +417,10 @@ __host__ __device__ __forceinline__ int mixed_ld(int W, int pad) {
   return pad ? W + ((4 - W) & 15) : W;
 }
 
-// X and Y: packed Hermitian rows of leading dimension ld.  FROMZ: U is assembled in FP32 from
-// the eigensolver's factors (Z, eb.phase, eb.refl, eb.tau) instead of being read.
-template <typename TIn, bool FROMZ, int TM>
+// X and Y: packed Hermitian rows of leading dimension ld.  U is assembled in FP32 from the eigensolver's
+// factors (Z, eb.phase, eb.refl, eb.tau).
+template <typename TIn, int TM>
 __global__ void __launch_bounds__(NT) berry_mixed_kernel(const double* __restrict__ E,
-                                                         const double2* __restrict__ U,
                                                          const double* __restrict__ Z,
                                                          EighBufs eb,
                                                          const TIn* __restrict__ Xp,
@@ -443,16 +442,7 @@ __global__ void __launch_bounds__(NT) berry_mixed_kernel(const double* __restric
   const int64_t k = blockIdx.x;
   const size_t WW = (size_t)W * W;
 
-  if (FROMZ) {
-    assemble_u_f32(Z + k * WW, eb.phase + k * W, eb.refl + k * WW, eb.tau + k * W, W, LD, t, sU, sA);
-  } else {
-    const FastDiv dW(W);
-    for (int idx = t; idx < W * W; idx += NT) {
-      const double2 u = U[k * WW + idx];
-      const int r = (int)dW.div(idx);
-      sU[r * LD + idx - r * W] = make_float2((float)u.x, (float)u.y);
-    }
-  }
+  assemble_u_f32(Z + k * WW, eb.phase + k * W, eb.refl + k * WW, eb.tau + k * W, W, LD, t, sU, sA);
   unpack_hermitian_f32(Xp + k * ld, sA, W, LD, t);
   for (int j = t; j < W; j += NT) sE[j] = E[k * W + j];
   if (t < n_eta) sEta[t] = etas[t];
@@ -1276,9 +1266,8 @@ size_t berry_mixed_smem(int W, int n_eta) {
   return mat + std::max(std::max(2 * mat, red), asm_stage_bytes(W));
 }
 
-template <typename TIn, bool FROMZ>
-cudaError_t launch_berry_mixed_t(const double* E, const double2* U, const double* Z,
-                                 const EighBufs& eb, const TIn* Xp, const TIn* Yp,
+template <typename TIn>
+cudaError_t launch_berry_mixed_t(const double* E, const double* Z, const EighBufs& eb, const TIn* Xp, const TIn* Yp,
                                  int64_t ld, int W, int n, const double* etas, int n_eta,
                                  double* Om, int64_t eta_stride, cudaStream_t s, int pad) {
   if (n <= 0) return cudaSuccess;
@@ -1286,20 +1275,12 @@ cudaError_t launch_berry_mixed_t(const double* E, const double2* U, const double
   auto go = [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    kern<<<n, NT, sm, s>>>(E, U, Z, eb, Xp, Yp, ld, W, etas, n_eta, Om, eta_stride, pad ? 1 : 0);
+    kern<<<n, NT, sm, s>>>(E, Z, eb, Xp, Yp, ld, W, etas, n_eta, Om, eta_stride, pad ? 1 : 0);
     return cudaGetLastError();
   };
-  if (W <= 16) return go(berry_mixed_kernel<TIn, FROMZ, 1>);
-  if (W <= 32) return go(berry_mixed_kernel<TIn, FROMZ, 2>);
-  return go(berry_mixed_kernel<TIn, FROMZ, 4>);
-}
-
-cudaError_t launch_berry_mixed_rows(const double* E, const double2* U, const double* C,
-                                    int64_t ld, int W, int n, const double* etas, int n_eta,
-                                    double* Om, int64_t eta_stride, cudaStream_t s, int pad) {
-  const int64_t WW = (int64_t)W * W;
-  return launch_berry_mixed_t<double, false>(E, U, nullptr, EighBufs{}, C + WW, C + 2 * WW, ld, W,
-                                             n, etas, n_eta, Om, eta_stride, s, pad);
+  if (W <= 16) return go(berry_mixed_kernel<TIn, 1>);
+  if (W <= 32) return go(berry_mixed_kernel<TIn, 2>);
+  return go(berry_mixed_kernel<TIn, 4>);
 }
 
 cudaError_t launch_berry_mixed_rows_z(const double* E, const double* Z, const EighBufs& eb,
@@ -1309,10 +1290,10 @@ cudaError_t launch_berry_mixed_rows_z(const double* E, const double* Z, const Ei
   const int64_t WW = (int64_t)W * W;
   if (vel32) {
     const float* X = reinterpret_cast<const float*>(C) + vel32_x0(W);
-    return launch_berry_mixed_t<float, true>(E, nullptr, Z, eb, X, X + vel32_yoff(W), 2 * ld, W,
+    return launch_berry_mixed_t<float>(E, Z, eb, X, X + vel32_yoff(W), 2 * ld, W,
                                              n, etas, n_eta, Om, eta_stride, s, pad);
   }
-  return launch_berry_mixed_t<double, true>(E, nullptr, Z, eb, C + WW, C + 2 * WW, ld, W, n, etas,
+  return launch_berry_mixed_t<double>(E, Z, eb, C + WW, C + 2 * WW, ld, W, n, etas,
                                             n_eta, Om, eta_stride, s, pad);
 }
 
@@ -1435,16 +1416,8 @@ cudaError_t launch_berry_mixed_from_f64_z(const double* E, const double* Z, cons
                                           const double* Xp, const double* Yp, int W, int n,
                                           const double* etas, int n_eta, double* Om,
                                           int64_t eta_stride, cudaStream_t s, int pad) {
-  return launch_berry_mixed_t<double, true>(E, nullptr, Z, eb, Xp, Yp, (int64_t)W * W, W, n, etas,
+  return launch_berry_mixed_t<double>(E, Z, eb, Xp, Yp, (int64_t)W * W, W, n, etas,
                                             n_eta, Om, eta_stride, s, pad);
-}
-
-cudaError_t launch_berry_mixed_from_f64(const double* E, const double2* U, const double* Xp,
-                                        const double* Yp, int W, int n, const double* etas,
-                                        int n_eta, double* Om, int64_t eta_stride,
-                                        cudaStream_t s, int pad) {
-  return launch_berry_mixed_t<double, false>(E, U, nullptr, EighBufs{}, Xp, Yp, (int64_t)W * W, W,
-                                             n, etas, n_eta, Om, eta_stride, s, pad);
 }
 
 cudaError_t launch_unpack_rows(const double* C, int64_t ld, int W, int n, double* H, double* X,

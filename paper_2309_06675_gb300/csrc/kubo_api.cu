@@ -766,34 +766,27 @@ int berry_launches(const Plan& p, int n, bool f32 = false) {
   return p.W > SMALL_W_MAX ? 5 : 1;
 }
 
-// Steps (3)-(4) from packed Hermitian dH rows X, Y of leading dimension ld; f32 = FP32
-// products.  rows = X and Y are the W*W and 2*W*W column offsets of tensor-core output rows.
+// Steps (3)-(4) from packed Hermitian dH rows X, Y of leading dimension ld and formed eigenvectors U: in FP64
+// grade, or (f32, above W = 64) as FP32 products.  The FP32 rotations up to W = 64 form U themselves.
 cudaError_t berry_any(const Call& c, const double* E, const double2* U, const double* X,
-                      const double* Y, int64_t ld, bool rows, int n, bool f32, double* Om,
-                      int64_t om_stride) {
+                      const double* Y, int64_t ld, int n, bool f32, double* Om, int64_t om_stride) {
   const Plan& p = c.p;
   const double* etas = c.at<double>(p.o_etas);
-  if (!f32) {
-    int* ue = p.user_u ? c.at<int>(p.o_ue) : nullptr;
-    if (ue) {
-      cudaError_t e = launch_unorm(U, p.W, n, ue, c.s);
-      if (e != cudaSuccess) return e;
-    }
-    if (p.zk > 0) return berry_tc64(c, E, U, ue, X, Y, ld, n, Om, om_stride);
-    return launch_berry_fix(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, ue, c.s, p.pad);
-  }
-  if (p.W > SMALL_W_MAX) {
+  if (f32) {
+    if (p.W <= SMALL_W_MAX) return cudaErrorInvalidValue;
     const size_t WW = (size_t)p.W * p.W;
     char* L = c.at<char>(p.o_L);
     const size_t cap = (size_t)std::max(1, p.chunk) * WW * sizeof(float2);
     return launch_berry_large(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, L, L + cap,
                               L + 2 * cap, c.s);
   }
-  if (rows) {
-    const double* C = X - (size_t)p.W * p.W;   // the row start (H | dxH | dyH)
-    return launch_berry_mixed_rows(E, U, C, ld, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad);
+  int* ue = p.user_u ? c.at<int>(p.o_ue) : nullptr;
+  if (ue) {
+    cudaError_t e = launch_unorm(U, p.W, n, ue, c.s);
+    if (e != cudaSuccess) return e;
   }
-  return launch_berry_mixed_from_f64(E, U, X, Y, p.W, n, etas, p.n_eta, Om, om_stride, c.s, p.pad);
+  if (p.zk > 0) return berry_tc64(c, E, U, ue, X, Y, ld, n, Om, om_stride);
+  return launch_berry_fix(E, U, X, Y, ld, p.W, n, etas, p.n_eta, Om, om_stride, ue, c.s, p.pad);
 }
 
 // Steps (1)-(4) for one batch [t0, t0+n) of a k-list; E and U go to the chunk buffers, Omega
@@ -869,7 +862,7 @@ kubo_status run_batch_mixed(Call& c, const Model& md, const KList& kl, double* E
   }
   {
     StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n, f32_rotation(p.precision)));
-    KCHECK(berry_any(c, Eout, U, C64 + WW, C64 + 2 * WW, p.Npad, true, kl.n, f32_rotation(p.precision), Om, om_stride));
+    KCHECK(berry_any(c, Eout, U, C64 + WW, C64 + 2 * WW, p.Npad, kl.n, f32_rotation(p.precision), Om, om_stride));
   }
   return KUBO_OK;
 }
@@ -922,7 +915,7 @@ kubo_status run_batch_steps(Call& c, const Model& md, const KList& kl, double* E
   }
   {
     StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n, f32_rotation(p.precision)));
-    KCHECK(berry_any(c, Eout, U, Xp, Yp, (int64_t)p.W * p.W, false, kl.n, f32_rotation(p.precision), Om, om_stride));
+    KCHECK(berry_any(c, Eout, U, Xp, Yp, (int64_t)p.W * p.W, kl.n, f32_rotation(p.precision), Om, om_stride));
   }
   return KUBO_OK;
 }
@@ -980,7 +973,7 @@ kubo_status fixup_batch(Call& c, const Model& md, const KList& kl, const double*
     KCHECK(launch_tridiag(c.at<double>(p.o_fHp), p.W, nf, eb, c.s));
     KCHECK(launch_ql(p.W, nf, eb, st, c.s));
     KCHECK(eigh_vectors(c, nf, eb, fE, U));
-    KCHECK(berry_any(c, fE, U, c.at<double>(p.o_fXp), c.at<double>(p.o_fYp), (int64_t)p.W * p.W, false, nf, false, fOm, fstride));
+    KCHECK(berry_any(c, fE, U, c.at<double>(p.o_fXp), c.at<double>(p.o_fYp), (int64_t)p.W * p.W, nf, false, fOm, fstride));
     KCHECK(launch_scale_pow2(fE, (int64_t)nf * p.W, -p.escale, c.s));
     KCHECK(launch_fixup_scatter(pos + c0, nf, p.W, p.n_eta, fE, fOm, fstride, E, Om, (int64_t)kl.n * p.W, c.s));
   }
@@ -1175,7 +1168,7 @@ kubo_status ahc_grad_device(Call& c, const kubo_options& o, const double* H_R, c
     if (out) {
       {
         StageTimer tm(c, KUBO_STAGE_BERRY, berry_launches(p, kl.n));
-        KCHECK(berry_any(c, E, U, Xp, Yp, (int64_t)WW, false, n, false, Om, (int64_t)n * p.W));
+        KCHECK(berry_any(c, E, U, Xp, Yp, (int64_t)WW, n, false, Om, (int64_t)n * p.W));
       }
       StageTimer tm(c, KUBO_STAGE_KSUM, o.kT == 0.0 ? 3 : 2);
       KCHECK(launch_ksum_partial(E, Om, p.W, n, p.n_eta, (int64_t)n * p.W, E_F, p.n_EF, o.kT, part, p.kpb, c.s));
@@ -2155,7 +2148,7 @@ kubo_status kubo_berry_batched(const double* E, const double* U, const double* d
     for (int64_t t0 = 0; t0 < n && r == KUBO_OK; t0 += step) {
       int nn = (int)std::min<int64_t>(step, n - t0);
       if (berry_any(c, E + t0 * W, (const double2*)U + t0 * WW, dHx + t0 * WW, dHy + t0 * WW, (int64_t)WW,
-                    false, nn, false, Omega + t0 * W, n * W) != cudaSuccess) {
+                    nn, false, Omega + t0 * W, n * W) != cudaSuccess) {
         cudaGetLastError();
         r = KUBO_ERR_CUDA;
       }

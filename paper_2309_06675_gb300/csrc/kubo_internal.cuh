@@ -258,12 +258,6 @@ cudaError_t launch_iit_df(int W, int n, EighBufs b, double* E, double* Z, double
 cudaError_t launch_backtransform(int W, int n, EighBufs b, double* E, double2* U,
                                  cudaStream_t s, int pad = 1);
 
-// rotations from packed dH rows of leading dimension ld (d_x H at column offset W*W, d_y H at
-// 2*W*W, as written by the tensor-core Fourier kernel), in FP32
-cudaError_t launch_berry_mixed_rows(const double* E, const double2* U, const double* C,
-                                    int64_t ld, int W, int n, const double* etas, int n_eta,
-                                    double* Om, int64_t eta_stride, cudaStream_t s, int pad = 1);
-
 // FP32 rotations with U = Q D Z assembled in FP32 inside the kernel from Z and the eigensolver
 // factors in eb (phase, refl, tau), W <= 64.  vel32 (these and the two tensor-core forms
 // below): the velocity rows of C are FP32 (vel32_x0 layout), else FP64 after the H columns.
@@ -302,12 +296,6 @@ cudaError_t launch_berry_tc_from_f64(const double* E, const double* Z, const Eig
                                      const double* Xp, const double* Yp, int W, int n,
                                      const double* etas, int n_eta, double* Om,
                                      int64_t eta_stride, DevStatus* st, cudaStream_t s);
-
-// FP32 rotation from FP64 packed arrays (error-budget mode)
-cudaError_t launch_berry_mixed_from_f64(const double* E, const double2* U, const double* Xp,
-                                        const double* Yp, int W, int n, const double* etas,
-                                        int n_eta, double* Om, int64_t eta_stride,
-                                        cudaStream_t s, int pad = 1);
 
 // tensor-core Fourier sum (k_fourier_tc.cu)
 int tc_pad_m(int n);

@@ -171,13 +171,7 @@ __device__ __forceinline__ void tmem_wait_ld16(uint32_t (&r)[16]) {
                : "memory");
 }
 
-// 32 lanes x 8 consecutive 32-bit columns, without a wait (tmem_wait_all before any use)
-__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                 "=r"(r[7])
-               : "r"(taddr));
-}
+// 32 lanes x 4 consecutive 32-bit columns, without a wait (tmem_wait_ld4 before any use)
 __device__ __forceinline__ void tmem_ld4_async(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -185,13 +179,6 @@ __device__ __forceinline__ void tmem_ld4_async(uint32_t taddr, uint32_t* r) {
 }
 // completes the thread's outstanding TMEM loads; the loaded registers pass through so that no
 // use of them is scheduled before it
-__device__ __forceinline__ void tmem_wait_ld8(uint32_t* r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
-                 "+r"(r[7])
-               :
-               : "memory");
-}
 __device__ __forceinline__ void tmem_wait_ld4(uint32_t* r) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
 }
