@@ -59,10 +59,16 @@ typedef enum {
 } kubo_status;
 
 typedef enum {
-  KUBO_FP64 = 0,            /* every step in FP64 or in arithmetic of at least its accuracy: the
-                               products of steps (1)-(3) as fixed-point digit products (55 to 59
-                               fractional bits, exact sums) on the tensor cores and the integer
-                               pipe, everything else in FP64 */
+  KUBO_FP64 = 0,            /* every step in FP64 or in arithmetic of at least its accuracy relative
+                               to the norms of its operands: the products of steps (1)-(3) as
+                               fixed-point digit products (55 to 59 fractional bits, exact sums) on
+                               the tensor cores and the integer pipe, everything else in FP64.
+                               The scales are a matrix element's largest term over R in step (1),
+                               the Frobenius norm in the reduction (of each block, where consecutive
+                               orbitals are uncoupled from the others) and the largest entry or the
+                               norm of the velocity matrix in step (3): in a block uncoupled from
+                               another one s times larger, velocities carry 2^-56 s of their size
+                               (2^-60 s up to W = 24) where FP64 products carry 2^-53. */
   KUBO_MIXED = 1,           /* the mixed-precision form: step (1) on the tensor cores (fixed-point
                                BF16 slices with exact FP32 block accumulation: H(k) to ~2^-31
                                relative, the velocity columns, which feed only step (3), to
@@ -130,7 +136,10 @@ typedef struct kubo_options {
                                (cudaMemPoolAttrReleaseThreshold) to the largest workspace it
                                has used, and never lowers it; other cudaMallocAsync users of the
                                same pool in the process see that threshold too.  A caller that
-                               must keep its own threshold passes a workspace here. */
+                               must keep its own threshold passes a workspace here.  Where the
+                               allocation fails and KUBO_FP64's sliced Fourier operands are
+                               64 MiB of it or more, it is tried once more without them (step
+                               (1) then runs on the FP64 pipe). */
   size_t workspace_bytes;
   int chunk_k;              /* k-points per internal batch; 0 = automatic (a fixed 24 GiB of
                                batch buffers, at most 65,536 k-points) */

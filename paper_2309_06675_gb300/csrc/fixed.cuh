@@ -1,8 +1,8 @@
 // Fixed-point arithmetic of FP64 grade on the integer pipe.
 //
 // GB300 issues an FP64 multiply-add for 2 lanes per SM clock and a 32 x 32 + 64-bit integer
-// multiply-add (IMAD.WIDE) for 60 (both measured), so a product of two 59-bit fixed-point numbers by
-// three integer multiply-adds runs ten times faster than an FP64 one.  A number |x| < 1 is
+// multiply-add (IMAD.WIDE) for 32 (both measured), so a product of two 59-bit fixed-point numbers by
+// three integer multiply-adds runs five times as fast as an FP64 one.  A number |x| < 1 is
 // X = round(x 2^59), held as two signed limbs, X = h 2^28 + l with |h| < 2^31 and |l| <= 2^27;
 //   X Y = hh 2^56 + (h l' + l h') 2^28 + l l',
 // and the last term (2^-62 r.m.s. of 1 for sums of 128 products) is dropped.  The sums of the

@@ -3,7 +3,7 @@
 //   iit_kernel            eigenvalue sort + eigenvectors of the tridiagonal T by inverse
 //                         iteration, one thread per cluster, persistent CTAs; LU factors in
 //                         per-CTA global scratch laid out [i][thread] (coalesced), iterates in
-//                         their column of Z (also used for W <= 64 when U is formed in FP32)
+//                         their column of Z (every order, but for MIXED_DF and a lean workspace)
 //   reflect_wy_kernel     U = Q D Z in FP32 by blocked compact-WY products (FP64: k_fixed.cu)
 //   cgemm_herm_u_kernel   T = dH U   (dH from packed Hermitian rows)          } FP32 (FP64:
 //   cgemm_uh_t_kernel     V = U^H T                                            } k_zgemm_tc64.cu)

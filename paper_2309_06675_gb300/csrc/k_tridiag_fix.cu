@@ -25,7 +25,8 @@
 //               w = v / |v|, v = x + e^{i arg x_0} |x| e_0
 //     (others)  the rest of the lower triangle of that update
 // The next column's reflector is a chain of some 2,000 clocks; beside the update it is hidden (on
-// its own between two barriers: W = 64, 4,096 k-points 2.87 ms, now 2.77; W = 97, 2,744: 11.4, now 11.0).
+// its own between two barriers: W = 64, 4,096 k-points 2.87 ms, beside it 2.77; W = 97, 2,744, with one CTA per SM: 11.4
+// and 11.0, and 6.5 with the two CTAs of launch_tridiag_fix).
 // What bounds it: the integer multiply-adds (12 per complex product) and, for short columns, the
 // latency of step 2, which the other CTAs of the SM fill.
 #include <algorithm>
