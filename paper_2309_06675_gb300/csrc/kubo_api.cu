@@ -235,6 +235,10 @@ int auto_chunk(int W, int n_eta, int64_t n_total, size_t extra_per_k = 0) {
 // 0.071; W = 32, N_R = 729 1.30 -> 0.157; W = 64, N_R = 1331 2.56 -> 0.465; the sum alone at W = 64, N_R = 1331, 4,096
 // k-points 112 -> 3.4).  So: from 24 vectors, fewer (from 16) where there are 1e8 operations.
 // The sliced basis (42 bytes per complex entry of H(R)) stays within 16 GiB, and 256 MiB below 1e8 operations.
+// There, and up to one row of tiles (128 k-points), the two are compared: the FMA kernel takes 1.74 us a vector for each wave
+// of its CTAs (128 columns by 16 k-points), the tensor-core form 5.7 us per 64 vectors for each wave of 32-column tiles,
+// the slicing at 3 TB/s and 12 us of small launches.  Preparation and sum, one k-point, N_R = 27, us: W = 64 47
+// and 35, W = 91 47 and 59, W = 128 47 and 81 (32 k-points: 86 and 83).
 constexpr double kTc64MinFlops = 1e8;
 constexpr size_t kTc64MaxBasis = (size_t)16 << 30;
 constexpr int kTc64MinVectors = 24;
@@ -245,7 +249,12 @@ bool use_tc64(int W, int N_R, int64_t n) {
   const size_t basis = (size_t)2 * tc64_slices() * tc64_pad_n(W) * tc_pad_k(N_R);
   if (W < 4 || N_R < 16) return false;
   if (6.0 * N_R * W * W * (double)n >= kTc64MinFlops) return basis <= kTc64MaxBasis;
-  return N_R >= kTc64MinVectors && basis <= kTc64SmallBasis;
+  if (N_R < kTc64MinVectors || basis > kTc64SmallBasis) return false;
+  if (n > 128) return true;
+  const int64_t sms = 152;
+  const int64_t fma_waves = ((W * W + 127) / 128 * ((n + 15) / 16) + sms - 1) / sms;
+  const int64_t tc_waves = (tc64_pad_n(W) / 32 + sms - 1) / sms;
+  return 12.0 + 5.7 * (tc_pad_k(N_R) / 64) * (double)tc_waves + (double)basis / 3e6 < 1.74 * N_R * (double)fma_waves;
 }
 
 void plan_layout(Plan& p, bool host_io, int64_t n_list_outputs_unused) {
