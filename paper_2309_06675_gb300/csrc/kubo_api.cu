@@ -31,6 +31,10 @@ constexpr int ZG_BATCH = 152 * 8;
 // this order: W = 16, 13,824 k-points 0.49 -> 0.16 ms, W = 48, 777: 3.55 -> 0.13, W = 64, 4,096: 6.2 -> 0.63; at
 // W = 6, 147,456 k-points, the QL lanes fill the chip and take 0.15 ms
 constexpr int BISECT_W_MIN = 9;
+// kubo_eigh_batched below that order, up to so many matrices: their eigenvectors in one launch with a CTA per matrix, while
+// those fill less than four CTAs per SM.  The whole call on the GPU, two launches (matrices packed into CTAs) and one,
+// us: W = 6, 64 matrices 138 and 127, 608 147 and 135, 1,216 147 and 162; W = 4 77 and 71, 79 and 75, 78 and 94
+constexpr int64_t LEAN_N = 608;
 constexpr int KSUM_KPB = 32;         // k-points per deterministic k-sum block (at least)
 constexpr size_t KSUM_PART_BYTES = (size_t)256 << 20;   // cap on the per-block partials
 // mixed precision: share of each batch (largest ||Omega(k)||_inf) redone in FP64
@@ -171,7 +175,7 @@ struct Plan {
   bool grad = false;    // reverse-mode buffers (kubo_ahc_grad)
   bool iit = false;     // inverse-iteration scratch (separate eigenvector kernel)
   int zk = 0;           // k-points per sub-batch of the tensor-core FP64 rotations (W > FIX_W_MAX)
-  bool lean = false;    // a caller's workspace too small for Z, the iteration scratch and zg (W <= 64)
+  bool lean = false;    // W <= 64: without Z, the iteration scratch and zg (a small workspace, LEAN_N)
   bool bisect = false;  // FP64 with eigenvectors: shifts by bisection, eigenvalues as Rayleigh quotients
   bool user_u = false;  // eigenvectors from the caller (kubo_berry_batched): column norms on the device
   int iit_slots = 0;
@@ -2101,6 +2105,7 @@ kubo_status kubo_eigh_batched(const double* A, int W, int64_t n, double* E, doub
     p.ql_cap = o.ql_max_sweeps;
     p.eigh = true;
     p.lbuf = W > SMALL_W_MAX;
+    p.lean = W < BISECT_W_MIN && n <= LEAN_N;
     plan_layout(p, false, 0);
     fit_workspace(p, o);
     c.s = (cudaStream_t)o.stream;
